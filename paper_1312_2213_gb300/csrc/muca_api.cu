@@ -58,7 +58,7 @@ constexpr size_t kMaxSmem = 227u * 1024u;  // dynamic shared memory a block can 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t lat, bin, T, lnW, lnW_sampled, G, lnR, H, Hpart, rlist, reach, state, out, Eq, lnWq, obs, metrics, tun, total;
+    size_t lat, bin, T, lnW, lnW_sampled, G, lnR, H, Hpart, rlist, reach, state, out, Eq, lnWq, obs, metrics, tun, scratch, total;
 };
 
 }  // namespace
@@ -83,6 +83,7 @@ struct muca_ctx {
     unsigned long long *obs = nullptr;  // [0, 3B): sums being filled, [3B, 6B): of the last update
     unsigned long long *metrics = nullptr;  // kMetricWords counters, see UpdateArgs::metrics
     uint8_t *tun = nullptr;                 // [p] tunnelling state per walker
+    void *scratch = nullptr;                // the recursion launch's words (update_scratch_bytes)
     int pipeline = 2;  // spins: code form (2), producer/consumer (1) or one warp per walker group (0)
     int pstride = 0, wpw = 0, nblk_max = 0;
     cudaStream_t stream = nullptr;
@@ -220,6 +221,7 @@ Layout plan(const muca_ctx *c)
         l.out = take(sizeof(double) * (4 + Bc));
         l.metrics = take(sizeof(unsigned long long) * kMetricWords);
         l.tun = take((size_t)c->p);
+        l.scratch = take(update_scratch_bytes(kPolyMaxBins));
         l.total = off;
         return l;
     }
@@ -239,6 +241,7 @@ Layout plan(const muca_ctx *c)
     l.obs = take(sizeof(unsigned long long) * 6 * (size_t)c->B);
     l.metrics = take(sizeof(unsigned long long) * kMetricWords);
     l.tun = take((size_t)c->p);
+    l.scratch = take(update_scratch_bytes(c->B));
     l.total = off;
     return l;
 }
@@ -261,6 +264,7 @@ UpdateArgs update_args(const muca_ctx *c)
     a.bin_w = 1.0 / (double)c->bin_k;
     a.recursion = c->recursion;
     a.metrics = c->metrics;
+    a.scratch = c->scratch;
     if (c->system == kPolymer) a.nblocks = 1;  // the open histogram is one global slot
     a.reach = c->reach;
     a.rlist = c->rlist;
@@ -432,6 +436,7 @@ int setup(muca_ctx *c)
     c->out = (double *)(base + l.out);
     c->metrics = (unsigned long long *)(base + l.metrics);
     c->tun = (uint8_t *)(base + l.tun);
+    c->scratch = base + l.scratch;
     if (c->system == kPolymer) {
         c->Eq = (long long *)(base + l.Eq);
         c->lnWq = (long long *)(base + l.lnWq);

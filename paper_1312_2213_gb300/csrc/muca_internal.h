@@ -97,7 +97,7 @@ cudaError_t launch_sweep_batch(const SpinSweepArgs *d_sys, const int2 *d_tiles, 
 // Polymer (bead-spring chain, Eq. 7 reading).  Master coordinates are int64 on a
 // 2^-44 grid, walker-major and axis-major: X[(w*3 + a)*N + j]; energies are int64
 // in units of 2^-32; the window is [elo_q, elo_q + B/10) in the same units.
-constexpr int kPolyMaxBins = 12288;  // the recursion stages 2 doubles a bin in shared memory
+constexpr int kPolyMaxBins = 12288;  // the recursion stages a double a bin in shared memory
 constexpr int kPolyMaxN = 128;
 constexpr long long kPolyStepQ = 1229;  // displacement grid units per unit of (u - 2^31)
 
@@ -161,7 +161,11 @@ struct UpdateArgs {
     // total accepted, total events, sweeps of the last iteration, sweep counter at the last
     // update}; the recursion launch closes them (null: none)
     unsigned long long *metrics;
+    // the recursion launch's own words (update_scratch_bytes): zero before the first update
+    void *scratch;
 };
+// Scratch bytes of an update over at most `bins` bins.
+size_t update_scratch_bytes(int bins);
 cudaError_t launch_merge(const UpdateArgs &a, cudaStream_t s);
 // Batched update kernels over n systems (argument arrays in device memory).
 cudaError_t launch_merge_batch(const UpdateArgs *d_args, int n, int max_bins, cudaStream_t s);

@@ -23,110 +23,264 @@ namespace muca {
 
 #define kNegInf (__longlong_as_double((long long)0xfff0000000000000ULL))
 
-__device__ __forceinline__ void merge_body(const UpdateArgs &a, int b)
+// Merge: 32 bins x 8 slot rows a block.  A thread that walked all ceil(p / block) slots of its bin
+// alone waited for one L2 round trip after the other (52 us for 128 slots of 8193 bins, 34 us for
+// the nine systems of the mix); eight rows with four loads in flight each take 6.3 and 4.6 us.
+constexpr int kMergeBins = 32, kMergeRows = 8;
+
+__device__ __forceinline__ void merge_body(const UpdateArgs &a)
 {
-    if (b >= a.B) return;
+    __shared__ unsigned long long part[kMergeRows][kMergeBins];
+    const int tx = threadIdx.x % kMergeBins, ty = threadIdx.x / kMergeBins;
+    const int b = blockIdx.x * kMergeBins + tx;
+    if (blockIdx.x * kMergeBins >= a.B) return;  // whole blocks only
     unsigned long long s = 0ull;
-    for (int k = 0; k < a.nblocks; ++k) {
-        unsigned long long *p = a.Hpart + (size_t)k * a.B + b;
-        s += *p;
-        *p = 0ull;
+    if (b < a.B) {
+#pragma unroll 4
+        for (int k = ty; k < a.nblocks; k += kMergeRows) {
+            unsigned long long *p = a.Hpart + (size_t)k * a.B + b;
+            const unsigned long long v = *p;
+            s += v;
+            if (v) *p = 0ull;
+        }
     }
-    a.H[b] = s;
+    part[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && b < a.B) {
+#pragma unroll
+        for (int r = 1; r < kMergeRows; ++r) s += part[r][tx];
+        a.H[b] = s;
+    }
 }
 
-__global__ void k_merge(const UpdateArgs a) { merge_body(a, blockIdx.x * blockDim.x + threadIdx.x); }
+__global__ void __launch_bounds__(kMergeBins *kMergeRows) k_merge(const UpdateArgs a) { merge_body(a); }
 
-__global__ void k_merge_batch(const UpdateArgs *__restrict__ arr)
+__global__ void __launch_bounds__(kMergeBins *kMergeRows) k_merge_batch(const UpdateArgs *__restrict__ arr)
 {
-    merge_body(arr[blockIdx.y], blockIdx.x * blockDim.x + threadIdx.x);
+    merge_body(arr[blockIdx.y]);
+}
+
+// The sequential sum acc <- RN(acc + r_k) of the recursion, with its roundings, a window of
+// kPrefixWindow terms at a time.  A dependent binary64 addition takes 64 cycles on GB300, 252 us for
+// the 8192 terms of L = 64 Potts; the windows take about 15 where the sum is smooth.
+// While acc stays in one binade [2^e, 2^(e+1)) it is an integer multiple A of u = 2^(e-52) and
+// RN(A u + r) = u (A + round(r / u)), where a tie rounds to an even sum: a term with a fractional
+// part of exactly one half adds f + ((A + f) & 1), f = floor(r / u).  So every term is a map of A
+// that depends on A through its parity alone, such maps compose associatively, and a window is an
+// integer scan of (increment for even A, increment for odd A).  The scan is right up to the first
+// term at which the sum leaves 2^52 < A < 2^53 or whose |r| is not below 2^e; that term is added in
+// binary64 and the next window starts behind it.  acc = 0 (bins not visited yet) passes over zero
+// terms.  For negative acc everything is mirrored, as rounding to nearest even is.
+// A window costs about as much as twenty additions, so behind the term that ended one early some
+// more are added singly: eight, or, where the window got less than kPrefixWorth terms far (a sum
+// that wanders about small values crosses binades at every few terms), four times as many as the
+// last time; at worst all are.  (These numbers had the least cost over the ln W of the mix's
+// systems and of L = 32, of init 1..64, worth 16..64, factors 2 and 4.)
+constexpr int kRecThreads = 256;
+constexpr int kPrefixPerThread = 2;
+constexpr int kPrefixWindow = kRecThreads * kPrefixPerThread;
+constexpr int kPrefixWorth = 16, kPrefixSerialMax = 2048;
+
+struct PrefixShared {
+    long long tot[kRecThreads / 32][2];  // each warp's composed map
+    int first;                           // first term of the window that the scan cannot take
+    double acc;                          // sum before that term
+};
+
+__device__ __forceinline__ void prefix_term(double r, bool neg, bool zero, int e, long long &f, bool &tie, bool &bad)
+{
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(r);
+    unsigned long long m = bits & 0x000fffffffffffffull;
+    int er = (int)((bits >> 52) & 0x7ffull);
+    f = 0;
+    tie = false;
+    if (zero) {
+        bad = (bits << 1) != 0ull;  // (+-0 leaves +0 as it is)
+        return;
+    }
+    if (er) m |= 0x0010000000000000ull;
+    else er = 1;
+    const int sh = e - er;  // r / u = m 2^-sh
+    bad = sh <= 0 && m != 0ull;  // |r| >= 2^e, infinite or NaN
+    if (bad || sh > 54 || m == 0ull) return;  // (sh > 54: |r / u| < 1/4)
+    const unsigned long long fl = m >> sh, rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
+    tie = rem == half;
+    const bool minus = ((bits >> 63) != 0ull) != neg;
+    const long long up = (long long)(fl + (rem > half ? 1ull : 0ull));
+    f = tie ? (minus ? -(long long)fl - 1 : (long long)fl) : (minus ? -up : up);
+}
+
+__device__ __forceinline__ long long prefix_step(long long d, long long f, bool tie, long long A)
+{
+    return d + f + (tie ? ((A + d + f) & 1ll) : 0ll);
+}
+
+// r[k] <- r_0 + ... + r_k for k < n, every sum rounded as in sequence; r in shared memory; the
+// whole block (kRecThreads) calls it.
+__device__ void exact_prefix(double *r, int n, PrefixShared &ps)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double acc = 0.0;
+    // a short sum is made as it stands, and so is the start of a longer one, where acc is no larger
+    // than the terms yet
+    int s = 0, serial = n <= 128 ? n : 16, streak = 1;
+    while (s < n) {
+        if (serial > 0) {
+            const int end = min(s + serial, n);
+            if (tid == 0) {
+                // eight terms read ahead while the eight before them are added
+                const int full = s + (end - s) / 8 * 8;
+                double nx[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) nx[i] = r[min(s + i, end - 1)];
+#pragma unroll 1
+                for (int k = s; k < full; k += 8) {
+                    double x[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) x[i] = nx[i];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) nx[i] = r[min(k + 8 + i, end - 1)];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        acc = __dadd_rn(acc, x[i]);
+                        x[i] = acc;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) r[k + i] = x[i];
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (full + i < end) {
+                        acc = __dadd_rn(acc, nx[i]);
+                        r[full + i] = acc;
+                    }
+                ps.acc = acc;
+            }
+            __syncthreads();
+            acc = ps.acc;
+            s = end;
+            serial = 0;
+            __syncthreads();  // ps is rewritten by the next window
+            continue;
+        }
+        const unsigned long long ab = (unsigned long long)__double_as_longlong(acc);
+        const int e = (int)((ab >> 52) & 0x7ffull);
+        const bool zero = ab == 0ull, neg = (ab >> 63) != 0ull;
+        if (!zero && (e == 0 || e == 0x7ff)) {  // subnormal or not finite
+            serial = 64;
+            continue;
+        }
+        const int end = min(s + kPrefixWindow, n);
+        const long long A0 = zero ? 0ll : (long long)((ab & 0x000fffffffffffffull) | 0x0010000000000000ull);
+        const int k0 = s + tid * kPrefixPerThread;
+        long long f[kPrefixPerThread];
+        bool tie[kPrefixPerThread], bad[kPrefixPerThread];
+        long long d0 = 0, d1 = 0;  // this thread's terms: increment for even A, for odd A
+#pragma unroll
+        for (int i = 0; i < kPrefixPerThread; ++i) {
+            prefix_term(k0 + i < end ? r[k0 + i] : 0.0, neg, zero, e, f[i], tie[i], bad[i]);
+            d0 = prefix_step(d0, f[i], tie[i], 0ll);
+            d1 = prefix_step(d1, f[i], tie[i], 1ll);
+        }
+        // inclusive scan of the maps over the warp, then over the warps before this one; without a
+        // tie in the warp (most have none) both parities move alike
+        long long i0 = d0, i1 = d1;
+        if (__any_sync(0xffffffffu, d0 != d1)) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long p0 = __shfl_up_sync(0xffffffffu, i0, o), p1 = __shfl_up_sync(0xffffffffu, i1, o);
+                if (lane >= o) {
+                    const long long n0 = p0 + ((p0 & 1ll) ? i1 : i0), n1 = p1 + (((p1 + 1ll) & 1ll) ? i1 : i0);
+                    i0 = n0;
+                    i1 = n1;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long p0 = __shfl_up_sync(0xffffffffu, i0, o);
+                if (lane >= o) i0 += p0;
+            }
+            i1 = i0;
+        }
+        if (lane == 31) {
+            ps.tot[warp][0] = i0;
+            ps.tot[warp][1] = i1;
+        }
+        if (tid == 0) {
+            ps.first = end;
+            ps.acc = acc;
+        }
+        __syncthreads();
+        long long A = A0;
+        long long t0[kRecThreads / 32 - 1], t1[kRecThreads / 32 - 1];  // (read together, not in a chain)
+#pragma unroll
+        for (int w = 0; w < kRecThreads / 32 - 1; ++w) {
+            t0[w] = ps.tot[w][0];
+            t1[w] = ps.tot[w][1];
+        }
+#pragma unroll
+        for (int w = 0; w < kRecThreads / 32 - 1; ++w)
+            if (w < warp) A += (A & 1ll) ? t1[w] : t0[w];
+        long long x0 = __shfl_up_sync(0xffffffffu, i0, 1), x1 = __shfl_up_sync(0xffffffffu, i1, 1);
+        if (lane == 0) x0 = x1 = 0ll;
+        A += (A & 1ll) ? x1 : x0;
+        // the sums behind this thread's terms, while they stay inside the binade
+        long long a[kPrefixPerThread];
+        int bad_at = end;
+#pragma unroll
+        for (int i = 0; i < kPrefixPerThread; ++i) {
+            A += prefix_step(0ll, f[i], tie[i], A);
+            a[i] = A;
+            const bool in = zero || (A > 0x0010000000000000ll && A < 0x0020000000000000ll);
+            if (k0 + i < bad_at && (bad[i] || !in)) bad_at = k0 + i;
+        }
+        const int wmin = __reduce_min_sync(0xffffffffu, bad_at);
+        if (lane == 0 && wmin < end) atomicMin(&ps.first, wmin);
+        __syncthreads();
+        const int v = ps.first;
+#pragma unroll
+        for (int i = 0; i < kPrefixPerThread; ++i) {
+            if (k0 + i < v) {
+                const double val = zero ? 0.0
+                                        : __longlong_as_double((long long)((ab & 0xfff0000000000000ull) |
+                                                                           ((unsigned long long)a[i] & 0x000fffffffffffffull)));
+                r[k0 + i] = val;
+                if (k0 + i == v - 1) ps.acc = val;
+            }
+        }
+        __syncthreads();
+        acc = ps.acc;
+        if (v < end) {
+            streak = v - s < kPrefixWorth ? min(4 * streak, kPrefixSerialMax) : 8;
+            serial = streak;
+        }
+        s = v;
+        __syncthreads();  // ps is rewritten by the next window
+    }
 }
 
 // Recursion over the ordered reachable bins r_0 < ... < r_{K-1}.  For each
 // neighbouring pair with h0 = H(r_k) > 0 and h1 = H(r_{k+1}) > 0:
 //   g = h0 h1 / (h0 + h1);  G_k += g;  kappa = g / G_k;
 //   lnR_k += kappa (ln h0 - ln h1),
-// then ln W(r_0) = 0 and ln W(r_{k+1}) = ln W(r_k) + lnR_k, summed in order by
-// one thread.  Pairs are independent, so the first part runs on all threads.
-__device__ __forceinline__ void recursion_body(const UpdateArgs &a, double *sm)
-{
-    double *slog = sm;
-    double *slnR = sm + a.nreach;
-    __shared__ unsigned long long s_min, s_max, s_sum;
-    const int tid = threadIdx.x, bs = blockDim.x;
-    if (tid == 0) {
-        s_min = ~0ull;
-        s_max = 0ull;
-        s_sum = 0ull;
-    }
-    for (int b = tid; b < a.B; b += bs) a.lnW_sampled[b] = a.lnW[b];
-    __syncthreads();  // lnW_sampled is the source of the plain update below
-    unsigned long long mn = ~0ull, mx = 0ull, sum = 0ull;
-    for (int k = tid; k < a.nreach; k += bs) {
-        const unsigned long long h = a.H[a.rlist[k]];
-        slog[k] = h ? dm_log(__ull2double_rn(h)) : 0.0;
-        mn = h < mn ? h : mn;
-        mx = h > mx ? h : mx;
-        sum += h;
-    }
-    __syncthreads();
-    atomicMin(&s_min, mn);
-    atomicMax(&s_max, mx);
-    atomicAdd(&s_sum, sum);
-    if (a.recursion == 1) {
-        // the plain rule W(n+1) = W(n)/H(n) in log form: x_k = ln W(r_k) - ln max(H(r_k), 1),
-        // ln W(r_k) = x_k - x_0 (an unvisited bin keeps its weight)
-        const double x0 = __dsub_rn(a.lnW_sampled[a.rlist[0]], slog[0]);
-        for (int k = tid; k < a.nreach; k += bs)
-            a.lnW[a.rlist[k]] = __dsub_rn(__dsub_rn(a.lnW_sampled[a.rlist[k]], slog[k]), x0);
-        __syncthreads();
-        if (tid == 0) {
-            const double mean = __ddiv_rn(__ull2double_rn(s_sum), (double)a.nreach);
-            a.state->flat_min = __ull2double_rn(s_min);
-            a.state->flat_mean = mean;
-            a.state->flat_max = __ull2double_rn(s_max);
-            a.state->flat = (s_min > 0ull) && (__ddiv_rn(__ull2double_rn(s_min), mean) >= a.flat_ratio);
-            a.state->iteration += 1ull;
-        }
-        return;
-    }
-    for (int k = tid; k + 1 < a.nreach; k += bs) {
-        const unsigned long long h0 = a.H[a.rlist[k]], h1 = a.H[a.rlist[k + 1]];
-        double r = a.lnR[k];
-        if (h0 != 0ull && h1 != 0ull) {
-            const double x0 = __ull2double_rn(h0), x1 = __ull2double_rn(h1);
-            const double g = __ddiv_rn(__dmul_rn(x0, x1), __dadd_rn(x0, x1));
-            const double G = __dadd_rn(a.G[k], g);
-            a.G[k] = G;
-            const double kappa = __ddiv_rn(g, G);
-            r = __dadd_rn(r, __dmul_rn(kappa, __dsub_rn(slog[k], slog[k + 1])));
-            a.lnR[k] = r;
-        }
-        slnR[k] = r;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        double acc = 0.0;
-        a.lnW[a.rlist[0]] = acc;
-        for (int k = 0; k + 1 < a.nreach; ++k) {
-            acc = __dadd_rn(acc, slnR[k]);
-            a.lnW[a.rlist[k + 1]] = acc;
-        }
-        const double mean = __ddiv_rn(__ull2double_rn(s_sum), (double)a.nreach);
-        a.state->flat_min = __ull2double_rn(s_min);
-        a.state->flat_mean = mean;
-        a.state->flat_max = __ull2double_rn(s_max);
-        a.state->flat = (s_min > 0ull) && (__ddiv_rn(__ull2double_rn(s_min), mean) >= a.flat_ratio);
-        a.state->iteration += 1ull;
-    }
-}
+// then ln W(r_0) = 0 and ln W(r_{k+1}) = ln W(r_k) + lnR_k, summed in order
+// (exact_prefix).  The pairs are independent: a block takes kRecPairs of them, one logarithm and
+// one pair a thread, so that they spread over the SMs (GB300 has two FP64 lanes a clock and SM, and
+// 8193 bins on one SM took over 200 us); the last block to finish sums them up.  The whole
+// recursion took 489 us for 8193 bins on one SM with one thread adding, and takes 50; 86 and 29
+// for the 1025 bins of L = 32 Ising, 301 and 49 for the mix.  What is left is latency: the chains of
+// FP64 operations (log, three divisions: about 10 us in all) and the windows of the sum.
+constexpr int kRecPairs = 63;
+
+__device__ __forceinline__ int recursion_blocks(int nreach) { return max(1, (nreach - 1 + kRecPairs - 1) / kRecPairs); }
 
 // The iteration's metrics become the "last" ones (and are added to the totals);
 // the open counters restart.  Runs once per update, after the sweeps' atomics.
 __device__ __forceinline__ void close_metrics(const UpdateArgs &a)
 {
     unsigned long long *m = a.metrics;
-    if (!m || threadIdx.x != 0) return;
+    if (!m) return;
     m[2] = m[0];
     m[3] = m[1];
     m[4] += m[0];
@@ -138,19 +292,126 @@ __device__ __forceinline__ void close_metrics(const UpdateArgs &a)
     m[1] = 0ull;
 }
 
-__global__ void __launch_bounds__(1024) k_recursion(const UpdateArgs a)
+// Scratch of an update (UpdateArgs::scratch): the count of finished blocks, each block's
+// {min, max, sum} of its bins' counts and, for the plain rule, ln W(r_k) - ln max(H(r_k), 1).
+__device__ __forceinline__ void recursion_body(const UpdateArgs &a, double *sm)
+{
+    __shared__ double slog[kRecPairs + 1];
+    __shared__ unsigned long long red[3][kRecThreads / 32];
+    __shared__ PrefixShared ps;
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nblk = recursion_blocks(a.nreach);
+    if ((int)blockIdx.x >= nblk) return;  // whole blocks only (batches size the grid for the largest system)
+    unsigned *done = (unsigned *)a.scratch;
+    unsigned long long *part = (unsigned long long *)a.scratch + 1;
+    double *plain = (double *)(part + 3 * nblk);
+    // the weights the merged histogram was sampled with; the last block overwrites lnW afterwards
+    for (int b = blockIdx.x * kRecThreads + tid; b < a.B; b += nblk * kRecThreads) a.lnW_sampled[b] = a.lnW[b];
+    const int base = blockIdx.x * kRecPairs;
+    unsigned long long h = 0ull, mn = ~0ull, mx = 0ull, sum = 0ull;
+    const int k = base + tid;
+    if (tid <= kRecPairs && k < a.nreach) {
+        h = a.H[a.rlist[k]];
+        slog[tid] = h ? dm_log(__ull2double_rn(h)) : 0.0;
+        if (tid < kRecPairs || k == a.nreach - 1) mn = mx = sum = h;  // (the bin two blocks share counts once)
+        if (a.recursion == 1) plain[k] = __dsub_rn(a.lnW[a.rlist[k]], slog[tid]);
+    }
+    __syncthreads();
+    if (a.recursion != 1 && tid < kRecPairs && k + 1 < a.nreach) {
+        const unsigned long long h1 = a.H[a.rlist[k + 1]];
+        if (h != 0ull && h1 != 0ull) {
+            const double x0 = __ull2double_rn(h), x1 = __ull2double_rn(h1);
+            const double g = __ddiv_rn(__dmul_rn(x0, x1), __dadd_rn(x0, x1));
+            const double G = __dadd_rn(a.G[k], g);
+            a.G[k] = G;
+            const double kappa = __ddiv_rn(g, G);
+            a.lnR[k] = __dadd_rn(a.lnR[k], __dmul_rn(kappa, __dsub_rn(slog[tid], slog[tid + 1])));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long n = __shfl_xor_sync(0xffffffffu, mn, o), x = __shfl_xor_sync(0xffffffffu, mx, o);
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        mn = n < mn ? n : mn;
+        mx = x > mx ? x : mx;
+    }
+    if (lane == 0) {
+        red[0][warp] = mn;
+        red[1][warp] = mx;
+        red[2][warp] = sum;
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kRecThreads / 32; ++w) {
+            mn = red[0][w] < mn ? red[0][w] : mn;
+            mx = red[1][w] > mx ? red[1][w] : mx;
+            sum += red[2][w];
+        }
+        part[3 * blockIdx.x] = mn;
+        part[3 * blockIdx.x + 1] = mx;
+        part[3 * blockIdx.x + 2] = sum;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == (unsigned)nblk - 1u;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (a.recursion == 1) {
+        // the plain rule W(n+1) = W(n)/H(n) in log form: x_k = ln W(r_k) - ln max(H(r_k), 1),
+        // ln W(r_k) = x_k - x_0 (an unvisited bin keeps its weight)
+        const double x0 = __ldcg(plain);
+        for (int i = tid; i < a.nreach; i += kRecThreads) a.lnW[a.rlist[i]] = __dsub_rn(__ldcg(plain + i), x0);
+    } else {
+        for (int i = tid; i + 1 < a.nreach; i += kRecThreads) sm[i] = __ldcg(a.lnR + i);
+    }
+    __syncthreads();
+    if (warp == kRecThreads / 32 - 1) {  // while the first warp starts on the sum
+        mn = ~0ull;
+        mx = sum = 0ull;
+        for (int i = lane; i < nblk; i += 32) {
+            const unsigned long long n = __ldcg(part + 3 * i), x = __ldcg(part + 3 * i + 1);
+            sum += __ldcg(part + 3 * i + 2);
+            mn = n < mn ? n : mn;
+            mx = x > mx ? x : mx;
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long n = __shfl_xor_sync(0xffffffffu, mn, o), x = __shfl_xor_sync(0xffffffffu, mx, o);
+            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            mn = n < mn ? n : mn;
+            mx = x > mx ? x : mx;
+        }
+        if (lane == 0) {
+            const double mean = __ddiv_rn(__ull2double_rn(sum), (double)a.nreach);
+            a.state->flat_min = __ull2double_rn(mn);
+            a.state->flat_mean = mean;
+            a.state->flat_max = __ull2double_rn(mx);
+            a.state->flat = (mn > 0ull) && (__ddiv_rn(__ull2double_rn(mn), mean) >= a.flat_ratio);
+            a.state->iteration += 1ull;
+            *done = 0u;  // ready for the next update
+            close_metrics(a);
+        }
+    }
+    if (a.recursion != 1) {
+        exact_prefix(sm, a.nreach - 1, ps);
+        if (tid == 0) a.lnW[a.rlist[0]] = 0.0;
+        for (int i = tid; i + 1 < a.nreach; i += kRecThreads) a.lnW[a.rlist[i + 1]] = sm[i];
+    }
+}
+
+__global__ void __launch_bounds__(kRecThreads) k_recursion(const UpdateArgs a)
 {
     extern __shared__ double sm[];
     recursion_body(a, sm);
-    close_metrics(a);
 }
 
-__global__ void __launch_bounds__(1024) k_recursion_batch(const UpdateArgs *__restrict__ arr)
+__global__ void __launch_bounds__(kRecThreads) k_recursion_batch(const UpdateArgs *__restrict__ arr)
 {
     extern __shared__ double sm[];
     const UpdateArgs a = arr[blockIdx.y];
     recursion_body(a, sm);
-    close_metrics(a);
 }
 
 __device__ __forceinline__ void thresholds_body(const UpdateArgs &a, int i)
@@ -414,18 +675,29 @@ cudaError_t launch_det_math(int fn, const double *in, double *out, long long n, 
     return cudaGetLastError();
 }
 
+// Launch shape of the recursion: its blocks, and shared memory for the last block's terms.
+static int recursion_grid(int nreach) { return nreach > kRecPairs ? (nreach - 1 + kRecPairs - 1) / kRecPairs : 1; }
+static size_t recursion_smem(int nreach) { return (size_t)nreach * sizeof(double); }
+
+size_t update_scratch_bytes(int bins)
+{
+    return sizeof(unsigned long long) * (1 + 3 * (size_t)recursion_grid(bins) + (size_t)bins);
+}
+
 cudaError_t launch_merge(const UpdateArgs &a, cudaStream_t s)
 {
-    k_merge<<<(a.B + 255) / 256, 256, 0, s>>>(a);
+    k_merge<<<(a.B + kMergeBins - 1) / kMergeBins, kMergeBins * kMergeRows, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_recursion(const UpdateArgs &a, cudaStream_t s)
 {
-    const size_t smem = (size_t)2 * a.nreach * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_recursion, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_recursion<<<1, 1024, smem, s>>>(a);
+    const size_t smem = recursion_smem(a.nreach);
+    if (smem > 40u * 1024u) {  // above what a launch may ask for without the attribute
+        const cudaError_t e = cudaFuncSetAttribute(k_recursion, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_recursion<<<recursion_grid(a.nreach), kRecThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -438,21 +710,20 @@ cudaError_t launch_thresholds(const UpdateArgs &a, cudaStream_t s)
 
 cudaError_t launch_merge_batch(const UpdateArgs *d_args, int n, int max_bins, cudaStream_t s)
 {
-    k_merge_batch<<<dim3((max_bins + 255) / 256, n), 256, 0, s>>>(d_args);
+    k_merge_batch<<<dim3((max_bins + kMergeBins - 1) / kMergeBins, n), kMergeBins * kMergeRows, 0, s>>>(d_args);
     return cudaGetLastError();
 }
 
 cudaError_t launch_recursion_batch(const UpdateArgs *d_args, int n, int max_nreach, cudaStream_t s)
 {
-    const size_t smem = (size_t)2 * max_nreach * sizeof(double);
-    k_recursion_batch<<<dim3(1, n), 1024, smem, s>>>(d_args);
+    k_recursion_batch<<<dim3(recursion_grid(max_nreach), n), kRecThreads, recursion_smem(max_nreach), s>>>(d_args);
     return cudaGetLastError();
 }
 
 cudaError_t prepare_recursion_batch(int max_nreach)
 {
     return cudaFuncSetAttribute(k_recursion_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)((size_t)2 * max_nreach * sizeof(double)));
+                                (int)recursion_smem(max_nreach));
 }
 
 cudaError_t launch_thresholds_batch(const UpdateArgs *d_args, int n, int max_cells, cudaStream_t s)
