@@ -68,6 +68,7 @@ struct muca_ctx {
     uint64_t seed = 0;
     double beta = 0.0, flat_ratio = 0.5;
     int record = 0, block = 64, walker_offset = 0;
+    bool block_set = false;      // "block" was set by the caller (polymer: else the launch chooses)
     bool block_small_p = false;  // q-Potts: 32 walkers a block because every block has an SM to itself
     int lanes = 0;     // polymer: lanes per walker in the sweep (8, 16, 32; 0 = chosen by N)
     int model = 0;     // polymer: 0 benchmark parameters, 1 the paper's (Eq. 7)
@@ -739,6 +740,7 @@ int muca_set_param(muca_ctx *c, const char *key, double v)
         if ((double)b != v || b < 32 || b > kMaxSweepBlock || (b % 32) != 0)
             return fail(MUCA_ERR_ARG, "block must be a multiple of 32 in [32, %d]", kMaxSweepBlock);
         c->block = b;
+        c->block_set = true;
         c->block_small_p = false;
         return MUCA_OK;
     }
@@ -847,7 +849,7 @@ int muca_iterate(muca_ctx *c, int64_t sweeps)
                 return fail(MUCA_ERR_ARG, "trace buffer holds %lld records; this iterate makes %lld",
                             (long long)c->trace_n, (long long)need);
         }
-        MUCA_CUDA(launch_poly_sweep(pa, c->block, c->stream));
+        MUCA_CUDA(launch_poly_sweep(pa, c->block_set ? c->block : 0, c->stream));
         MUCA_CUDA(launch_advance(c->state, sweeps, c->stream));
         // refresh the running energies from scratch; the largest change is recorded
         MUCA_CUDA(launch_poly_energy(pa, 1, c->stream));
@@ -1365,7 +1367,7 @@ int batch_enqueue_iteration(muca_batch *b, int64_t sweeps)
             muca_ctx *c = b->sys[i];
             if (c->system == kPolymer) {  // as muca_iterate: the sweeps, then the energies from scratch
                 const PolyArgs pa = poly_args(c, b->h_sys[i].sweeps);
-                MUCA_CUDA(launch_poly_sweep(pa, c->block, b->sub[i]));
+                MUCA_CUDA(launch_poly_sweep(pa, c->block_set ? c->block : 0, b->sub[i]));
                 MUCA_CUDA(launch_poly_energy(pa, 1, b->sub[i]));
             } else {
                 MUCA_CUDA(launch_system_sweep(c, b->h_own[i], b->sub[i], b->blk[i]));

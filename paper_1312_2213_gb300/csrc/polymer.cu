@@ -218,12 +218,10 @@ __device__ __forceinline__ bool group_any(bool p, int gi)
 // Marsaglia's method on (m.z, m.w) and then on tag-4 blocks (64 i + t), two pairs
 // a block, at most 64 pairs.  Every step is a correctly rounded binary64
 // operation on exact grid values, so the new grid position is bit-identical to
-// any implementation that follows the same steps.  Returns false when no point
-// was found (the move is then rejected).
-__device__ bool poly_rotation(const long long *Xg, int N, int i, uint32_t g, uint32_t wid, const uint4 m,
-                              const uint32_t (&rk)[20], long long out[3])
+// any implementation that follows the same steps.  poly_unit draws n and returns
+// false when no point was found (the move is then rejected).
+__device__ bool poly_unit(int i, uint32_t g, uint32_t wid, const uint4 m, const uint32_t (&rk)[20], double n[3])
 {
-    const int pv = (i == 0) ? 1 : (i == N - 1) ? N - 2 : ((m.y & 1u) ? i + 1 : i - 1);
     double v1 = 0.0, v2 = 0.0, s = 0.0;
     bool found = false;
     uint4 blk = make_uint4(0u, 0u, m.z, m.w);
@@ -238,55 +236,169 @@ __device__ bool poly_rotation(const long long *Xg, int N, int i, uint32_t g, uin
     }
     if (!found) return false;
     const double f = __dmul_rn(2.0, __dsqrt_rn(__dsub_rn(1.0, s)));
-    const double n[3] = {__dmul_rn(v1, f), __dmul_rn(v2, f), __dsub_rn(1.0, __dmul_rn(2.0, s))};
-    double dd[3];
-    long long P[3];
-    for (int c = 0; c < 3; ++c) {
-        P[c] = Xg[c * N + pv];
-        dd[c] = __dmul_rn((double)(Xg[c * N + i] - P[c]), 0x1p-44);
-    }
-    const double d = __dsqrt_rn(
-        __dadd_rn(__dadd_rn(__dmul_rn(dd[0], dd[0]), __dmul_rn(dd[1], dd[1])), __dmul_rn(dd[2], dd[2])));
-    for (int c = 0; c < 3; ++c) out[c] = P[c] + (long long)rint(__dmul_rn(__dmul_rn(n[c], d), 0x1p44));
+    n[0] = __dmul_rn(v1, f);
+    n[1] = __dmul_rn(v2, f);
+    n[2] = __dsub_rn(1.0, __dmul_rn(2.0, s));
     return true;
 }
 
-// Shared-memory floats of one walker's slot: the float-pair shadows (6 N) and the
-// energies of its N - 1 bonds, rounded up to a multiple of 4 so that the uint4
-// Philox blocks behind all slots start 16-byte aligned for any walker count and
-// odd N.  (Padding the slots so that the walkers of a warp read disjoint banks was
-// measured on GB300 with the 6 N layout: within 1 % at N = 64 and 128, 2-5 %
-// slower at N = 32 and 13, so it is not done.)
-template <int G>
-__host__ __device__ inline int poly_slot_floats(int N)
+// One axis' share (dd, squared by the caller) of d and the new grid coordinate of one axis.
+__device__ __forceinline__ double poly_axis_diff(long long x, long long pivot)
 {
-    return (7 * N + 3) & ~3;  // hi[3N], lo[3N], bond energies[N]; a multiple of 4 floats
+    return __dmul_rn((double)(x - pivot), 0x1p-44);
+}
+__device__ __forceinline__ double poly_distance(double dx, double dy, double dz)
+{
+    return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
+}
+__device__ __forceinline__ long long poly_rotated(long long pivot, double n, double d)
+{
+    return pivot + (long long)rint(__dmul_rn(__dmul_rn(n, d), 0x1p44));
 }
 
-// Sweeps: G lanes per walker, 32/G walkers a warp, all on the same bead i.  A
-// walker's float-pair shadows and this sweep's Philox blocks live in shared
-// memory (40 N bytes, 56 N with rotations); its int64 master coordinates stay in
-// global memory (read at the sweep start and for the moved bead, written on
-// acceptance).  The two
-// bonds of bead i (FENE) are taken by lanes 0 and 1 of the group, the other
-// partners (LJ, |i - j| >= 2) by lanes j mod G, so no lane runs both branches.
-template <int G, int RECORD>
+// Packed pairs of floats (PTX f32x2): one instruction for the same operation on both halves, each
+// rounded as the scalar one.
+using float_pair = unsigned long long;
+__device__ __forceinline__ float_pair pair_of(float lo, float hi)
+{
+    float_pair r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void halves_of(float_pair v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ float_pair add_pair(float_pair a, float_pair b)
+{
+    float_pair r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float_pair mul_pair(float_pair a, float_pair b)
+{
+    float_pair r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float_pair fma_pair(float_pair a, float_pair b, float_pair c)
+{
+    float_pair r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Minus the moved bead's position, old in the low halves and new in the high ones.
+struct MovedBead {
+    float_pair x, y, z, lx, ly, lz;
+};
+
+// LJ energy of the moved bead with one partner, new position minus old: lj_energy on both at once.
+// (The squares do not see the sign of a separation.)
+__device__ __forceinline__ float lj_change(const float4 &pj, const float2 &qj, const MovedBead &m, const PolyArgs &a)
+{
+    const float_pair dx = add_pair(add_pair(pair_of(pj.x, pj.x), m.x), add_pair(pair_of(pj.w, pj.w), m.lx));
+    const float_pair dy = add_pair(add_pair(pair_of(pj.y, pj.y), m.y), add_pair(pair_of(qj.x, qj.x), m.ly));
+    const float_pair dz = add_pair(add_pair(pair_of(pj.z, pj.z), m.z), add_pair(pair_of(qj.y, qj.y), m.lz));
+#ifndef POLY_R2
+#define POLY_R2 0
+#endif
+#if POLY_R2 == 0
+    const float_pair r2 = fma_pair(dz, dz, fma_pair(dx, dx, mul_pair(dy, dy)));
+#else
+    const float_pair r2 = fma_pair(dz, dz, fma_pair(dy, dy, mul_pair(dx, dx)));
+#endif
+    float r2o, r2n;
+    halves_of(r2, r2o, r2n);
+    const float_pair ir2 = mul_pair(pair_of(rcp_approx(r2o), rcp_approx(r2n)), pair_of(a.lj_sigma2, a.lj_sigma2));
+    const float_pair ir6 = mul_pair(mul_pair(ir2, ir2), ir2);
+    float ho, hn;
+    halves_of(ir6, ho, hn);
+    const float_pair v = fma_pair(pair_of(fmaf(ho, ho, -ho), fmaf(hn, hn, -hn)), pair_of(4.0f, 4.0f),
+                                  pair_of(-a.lj_shift, -a.lj_shift));
+    float vo, vn;
+    halves_of(v, vo, vn);
+    return (r2n < a.lj_rc2 ? vn : 0.0f) - (r2o < a.lj_rc2 ? vo : 0.0f);
+}
+
+// Energy of a new bond over the separation (bx, by, bz), NaN if it breaks.
+__device__ __forceinline__ float bond_or_nan(float bx, float by, float bz, const PolyArgs &a)
+{
+    const float r2n = bx * bx + by * by + bz * bz;
+    return fene_intact(r2n, a) ? fene_energy(r2n, a) : __int_as_float(0x7fffffff);
+}
+
+// Shared memory of one walker's slot.  Beads: the float-pair shadows, (x, y, z, lo x) in pa and
+// (lo y, lo z) in pb, and the energies eb of the N - 1 bonds.  The chunk of beads being visited
+// (poly_chunk of them at a time): the proposed shadows and what else an attempt needs of its own
+// bead.  Every attempt's loads are then two wide ones a partner and three for the moved bead.
+template <int G>
+__host__ __device__ constexpr int poly_chunk() { return G > 16 ? G : 16; }
+
+template <int G, int MOVES>
+struct PolySlot {
+    static constexpr int CH = poly_chunk<G>();
+    float4 *pa;      // [N]
+    float4 *na;      // [CH] proposed x, y, z, lo x
+    float4 *nb;      // [CH] proposed lo y, lo z; ln of the acceptance word; energy of bond (j, j+1), j moved
+    float4 *nc;      // [CH] energy of bond (j-1, j), j moved: j-1 where it was, j-1 moved; random words x, y
+    float2 *pb;      // [N]
+    long long *nx;   // [CH][3] (MOVES) proposed grid position, or the rotation's unit vector
+    float *eb;       // [N]
+    uint32_t *wz;    // [CH] random word z
+    uint32_t *how;   // [CH] (MOVES) kReady, kLate, kNoPoint
+    static __host__ __device__ size_t bytes(int N)
+    {
+        const size_t b = (size_t)N * 28 + CH * (size_t)(48 + 4 + (MOVES ? 28 : 0));
+        return (b + 15) / 16 * 16;
+    }
+    __device__ PolySlot(unsigned char *p, int N)
+    {
+        pa = (float4 *)p;
+        na = pa + N;
+        nb = na + CH;
+        nc = nb + CH;
+        pb = (float2 *)(nc + CH);
+        nx = (long long *)(pb + N);
+        eb = (float *)(MOVES ? nx + 3 * CH : nx);
+        wz = (uint32_t *)(eb + N);
+        how = wz + CH;
+    }
+};
+enum : uint32_t { kReady = 0u, kLate = 1u, kNoPoint = 2u };
+
+// Sweeps: G lanes per walker, 32/G walkers a warp, all on the same bead i.  The two bonds of bead i
+// (FENE) are taken by lanes 0 and 1 of the group, the other partners (LJ, |i - j| >= 2) by lanes
+// j mod G, in ascending order, so the FP32 sums do not depend on anything else.
+//
+// Bound by issue (3.4 warps a scheduler at 4096 walkers; of 370 warp instructions an attempt at
+// N = 13 one seventh was pair work), so what is not pair work is taken out of the serial loop: a
+// bead is visited once a sweep and stands still until then, so its random words, its proposed
+// position and the energies of its new bonds (the left one for both outcomes of the bead before it)
+// are known before the loop reaches it.  Every lane prepares its own beads of the next poly_chunk
+// beads, and the attempt only reads them.  Accepted moves reach the int64 master coordinates behind
+// the chunk, in parallel again.  Old and new pair energies go through packed instructions
+// (lj_change).  With rotations (MOVES) a proposal about bead i - 1 needs that bead's outcome: its
+// unit vector is prepared, the position (binary64, one axis a lane) made when the bead is reached.
+template <int G, int MOVES>
 __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs a)
 {
     constexpr int W = 32 / G;
+    constexpr int CH = poly_chunk<G>();
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5, N = a.N;
     const int gi = lane / G, li = lane % G;
-    const int spb = wpb * W, slot = wib * W + gi, sst = poly_slot_floats<G>(N);
-    float *xs = (float *)smem + (size_t)slot * sst;
-    float *xl = xs + 3 * N;
-    float *eb = xs + 6 * N;  // eb[j]: FP32 energy of bond (j, j+1) at the current shadows
-    uint4 *su = (uint4 *)(smem + (size_t)spb * sst * sizeof(float)) + (size_t)slot * N;
-    uint4 *sm = su + (size_t)spb * N;  // moves
-    // the block's histogram counters and its count of finished warps, after all slots and
-    // Philox blocks
-    unsigned *hs = (unsigned *)(smem + (size_t)spb * sst * sizeof(float) +
-                                (size_t)spb * N * (a.moves ? 2 : 1) * sizeof(uint4));
+    const int spb = wpb * W, slot = wib * W + gi;
+    const size_t sst = PolySlot<G, MOVES>::bytes(N);
+    const PolySlot<G, MOVES> S(smem + slot * sst, N);
+    // the block's histogram counters and its count of finished warps, behind all slots
+    unsigned *hs = (unsigned *)(smem + spb * sst);
     unsigned *done = hs + a.B;
     for (int i = threadIdx.x; i <= a.B; i += blockDim.x) hs[i] = 0u;
     __syncthreads();
@@ -299,6 +411,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
     long long *Xg = a.X + (size_t)wr * 3 * N;
     long long E = a.E[wr];
     int b = poly_bin(E, a);
+    long long lw = (b >= 0 && b < a.B) ? __ldg(a.lnWq + b) : 0;  // ln W of the current bin
     const uint32_t g0 = (uint32_t)(a.state->sweep_counter + a.sweep_base);
     const int npl = (N + G - 1) / G;
     // metrics: accepted moves and tunnelling between bins 0 and B-1 (group-uniform values)
@@ -310,162 +423,285 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
         const uint32_t g = g0 + (uint32_t)sw;
         const long long A0 = Xg[0], A1 = Xg[N], A2 = Xg[2 * N];
         for (int j = li; j < N; j += G) {
-            grid_to_ff(Xg[j] - A0, xs[j], xl[j]);
-            grid_to_ff(Xg[N + j] - A1, xs[N + j], xl[N + j]);
-            grid_to_ff(Xg[2 * N + j] - A2, xs[2 * N + j], xl[2 * N + j]);
-            uint4 r = philox4x32_10_rk(make_uint4((uint32_t)j, g, wid, kTagSweep), a.rk);
-            // the acceptance test u 2^-32 < exp(d) is taken as ln(u 2^-32) < d: the logarithm
-            // (FP32, -inf for u = 0) is taken here, once a bead and sweep, off the serial path
-            r.w = __float_as_uint(logf((float)r.w * 0x1p-32f));
-            su[j] = r;
-            if (a.moves) sm[j] = philox4x32_10_rk(make_uint4((uint32_t)j, g, wid, kTagPolyMove), a.rk);
+            float4 p;
+            float2 q;
+            grid_to_ff(Xg[j] - A0, p.x, p.w);
+            grid_to_ff(Xg[N + j] - A1, p.y, q.x);
+            grid_to_ff(Xg[2 * N + j] - A2, p.z, q.y);
+            S.pa[j] = p;
+            S.pb[j] = q;
         }
         __syncwarp();
         for (int j = li; j + 1 < N; j += G) {
-            const float dx = (xs[j] - xs[j + 1]) + (xl[j] - xl[j + 1]);
-            const float dy = (xs[N + j] - xs[N + j + 1]) + (xl[N + j] - xl[N + j + 1]);
-            const float dz = (xs[2 * N + j] - xs[2 * N + j + 1]) + (xl[2 * N + j] - xl[2 * N + j + 1]);
-            eb[j] = fene_energy(dx * dx + dy * dy + dz * dz, a);
+            const float4 p = S.pa[j], r = S.pa[j + 1];
+            const float2 q = S.pb[j], t = S.pb[j + 1];
+            const float dx = (p.x - r.x) + (p.w - r.w);
+            const float dy = (p.y - r.y) + (q.x - t.x);
+            const float dz = (p.z - r.z) + (q.y - t.y);
+            S.eb[j] = fene_energy(dx * dx + dy * dy + dz * dz, a);
         }
-        __syncwarp();
 #pragma unroll 1
-        for (int i = 0; i < N; ++i) {
-            const uint4 u = su[i];
-            // move (u - 2^31) * 1229 grid units per axis: exact on the int64 master
-            // coordinates; the float-pair shadow moves by the same amount in FP32
-            // (the shadows are rebuilt exactly from the masters every sweep)
-            const int sx = (int)(u.x ^ 0x80000000u), sy = (int)(u.y ^ 0x80000000u), sz = (int)(u.z ^ 0x80000000u);
-            const long long X0 = Xg[i], X1 = Xg[N + i], X2 = Xg[2 * N + i];
-            const float xo = xs[i], yo = xs[N + i], zo = xs[2 * N + i];
-            const float lxo = xl[i], lyo = xl[N + i], lzo = xl[2 * N + i];
-            const float dx = (float)sx * kStep, dy = (float)sy * kStep, dz = (float)sz * kStep;
-            float xn = xo + dx, yn = yo + dy, zn = zo + dz;
-            float lxn = lxo + ((xo - xn) + dx), lyn = lyo + ((yo - yn) + dy), lzn = lzo + ((zo - zn) + dz);
-            // (32 x 32-bit products: the grid step fits an int)
-            long long n0 = X0 + (long long)sx * (long long)a.step_q, n1 = X1 + (long long)sy * (long long)a.step_q,
-                      n2 = X2 + (long long)sz * (long long)a.step_q;
-            float s = 0.0f, c = 0.0f;
-            bool broken = false;
-            if (a.moves) {
-                const uint4 mv = sm[i];
-                if (mv.x >= 0x80000000u) {  // spherical rotation about a bonded neighbour
-                    long long nr[3];
-                    if (poly_rotation(Xg, N, i, g, wid, mv, a.rk, nr)) {
-                        n0 = nr[0];
-                        n1 = nr[1];
-                        n2 = nr[2];
-                        grid_to_ff(n0 - A0, xn, lxn);
-                        grid_to_ff(n1 - A1, yn, lyn);
-                        grid_to_ff(n2 - A2, zn, lzn);
-                    } else {
-                        broken = true;  // no point in 64 pairs: rejected
+        for (int c0 = 0; c0 < N; c0 += CH) {
+            // ---- prepare the chunk, a bead a lane
+#pragma unroll 1
+            for (int t = li; t < CH; t += G) {
+                const int j = c0 + t;
+                if (j >= N) break;
+                const uint4 r = philox4x32_10_rk(make_uint4((uint32_t)j, g, wid, kTagSweep), a.rk);
+                // move (u - 2^31) * 1229 grid units per axis: exact on the int64 master
+                // coordinates; the float-pair shadow moves by the same amount in FP32
+                // (the shadows are rebuilt exactly from the masters every sweep)
+                const int sx = (int)(r.x ^ 0x80000000u), sy = (int)(r.y ^ 0x80000000u), sz = (int)(r.z ^ 0x80000000u);
+                const float4 p = S.pa[j];
+                const float2 q = S.pb[j];
+                const float dx = (float)sx * kStep, dy = (float)sy * kStep, dz = (float)sz * kStep;
+                const float xo = p.x, yo = p.y, zo = p.z;
+                float xn = xo + dx, yn = yo + dy, zn = zo + dz;
+                float lxn = p.w + ((xo - xn) + dx), lyn = q.x + ((yo - yn) + dy), lzn = q.y + ((zo - zn) + dz);
+                if (MOVES) {
+                    const long long X0 = Xg[j], X1 = Xg[N + j], X2 = Xg[2 * N + j];
+                    long long n0 = X0 + (long long)sx * (long long)a.step_q, n1 = X1 + (long long)sy * (long long)a.step_q,
+                              n2 = X2 + (long long)sz * (long long)a.step_q;
+                    const uint4 mv = philox4x32_10_rk(make_uint4((uint32_t)j, g, wid, kTagPolyMove), a.rk);
+                    uint32_t how = kReady;
+                    if (mv.x >= 0x80000000u) {  // spherical rotation about a bonded neighbour
+                        double n[3];
+                        if (!poly_unit(j, g, wid, mv, a.rk, n)) {
+                            how = kNoPoint;
+                        } else if (j == 0 || (j != N - 1 && (mv.y & 1u))) {  // about bead j + 1, not visited yet
+                            const long long P0 = Xg[j + 1], P1 = Xg[N + j + 1], P2 = Xg[2 * N + j + 1];
+                            const double d = poly_distance(poly_axis_diff(X0, P0), poly_axis_diff(X1, P1),
+                                                           poly_axis_diff(X2, P2));
+                            n0 = poly_rotated(P0, n[0], d);
+                            n1 = poly_rotated(P1, n[1], d);
+                            n2 = poly_rotated(P2, n[2], d);
+                            grid_to_ff(n0 - A0, xn, lxn);
+                            grid_to_ff(n1 - A1, yn, lyn);
+                            grid_to_ff(n2 - A2, zn, lzn);
+                        } else {  // about bead j - 1: when it has been visited
+                            how = kLate;
+                            n0 = __double_as_longlong(n[0]);
+                            n1 = __double_as_longlong(n[1]);
+                            n2 = __double_as_longlong(n[2]);
+                        }
                     }
+                    S.nx[3 * t] = n0;
+                    S.nx[3 * t + 1] = n1;
+                    S.nx[3 * t + 2] = n2;
+                    S.how[t] = how;
+                }
+                S.na[t] = make_float4(xn, yn, zn, lxn);
+                // the acceptance test u 2^-32 < exp(d) is taken as ln(u 2^-32) < d: the logarithm
+                // (FP32, -inf for u = 0) is taken here, off the serial path
+                S.nb[t] = make_float4(lyn, lzn, logf((float)r.w * 0x1p-32f), 0.0f);
+                if (!MOVES) {
+                    S.nc[t].z = __uint_as_float(r.x);
+                    S.nc[t].w = __uint_as_float(r.y);
+                    S.wz[t] = r.z;
                 }
             }
-            // the bonds (i-1, i) and (i, i+1): lanes 0 and 1 of the group, or the walker's only lane
-            // for both when G = 1; the old energies come from the bond cache, the new ones are
-            // kept to update it if the move is accepted
-            float vnb[2] = {0.0f, 0.0f};
+            __syncwarp();
+            if (!MOVES) {
+#pragma unroll 1
+                for (int t = li; t < CH; t += G) {
+                    const int j = c0 + t;
+                    if (j >= N) break;
+                    const float4 p = S.na[t], q = S.nb[t];
+                    if (j + 1 < N) {
+                        const float4 r = S.pa[j + 1];
+                        const float2 u = S.pb[j + 1];
+                        S.nb[t].w = bond_or_nan((p.x - r.x) + (p.w - r.w), (p.y - r.y) + (q.x - u.x),
+                                                (p.z - r.z) + (q.y - u.y), a);
+                    }
+                    if (j > 0) {
+                        const float4 r = S.pa[j - 1];
+                        const float2 u = S.pb[j - 1];
+                        S.nc[t].x = bond_or_nan((p.x - r.x) + (p.w - r.w), (p.y - r.y) + (q.x - u.x),
+                                                (p.z - r.z) + (q.y - u.y), a);
+                    }
+                    if (t > 0) {  // (the bead before the chunk stands where pa has it)
+                        const float4 r = S.na[t - 1], u = S.nb[t - 1];
+                        S.nc[t].y = bond_or_nan((p.x - r.x) + (p.w - r.w), (p.y - r.y) + (q.x - u.x),
+                                                (p.z - r.z) + (q.y - u.y), a);
+                    }
+                }
+                __syncwarp();
+            }
+            // ---- the attempts, one after the other
+            const int nt = min(CH, N - c0);
+            uint32_t accs = 0u;   // accepted beads of the chunk (group-uniform)
+            bool acc = false;     // the bead before was moved
+#pragma unroll 1
+            for (int t = 0; t < nt; ++t) {
+                const int i = c0 + t;
+                const float4 po = S.pa[i];
+                const float2 qo = S.pb[i];
+                bool broken = false;
+                if (MOVES) {
+                    const uint32_t how = S.how[t];
+                    broken = how == kNoPoint;
+                    if (__any_sync(0xffffffffu, how == kLate)) {
+                        // about bead i - 1, where it is now; lanes 0, 1, 2 of the group an axis each
+                        // (fewer lanes take the axes in turn)
+                        const int pv = i > 0 ? i - 1 : 0;
+                        double dd[3];
+                        if (G >= 4) {
+                            const int c = min(li, 2);
+                            const double own = poly_axis_diff(Xg[c * N + i], Xg[c * N + pv]);
 #pragma unroll
-            for (int t = 0; t < (G == 1 ? 2 : 1); ++t) {
-                const int jb = (G == 1 ? t == 0 : li == 0) ? i - 1 : i + 1;
-                if ((G == 1 || li < 2) && jb >= 0 && jb < N) {
-                    const float xj = xs[jb], yj = xs[N + jb], zj = xs[2 * N + jb];
-                    const float ljx = xl[jb], ljy = xl[N + jb], ljz = xl[2 * N + jb];
-                    const float bx = (xn - xj) + (lxn - ljx), by = (yn - yj) + (lyn - ljy), bz = (zn - zj) + (lzn - ljz);
-                    const float r2n = bx * bx + by * by + bz * bz;
-                    const bool brk = !fene_intact(r2n, a);
-                    broken = broken || brk;
-                    const float vo = eb[jb < i ? jb : i];
-                    const float vn = brk ? vo : fene_energy(r2n, a);
-                    vnb[t] = vn;
-                    const float y = (vn - vo) - c;  // compensated, as the pair terms below
+                            for (int k = 0; k < 3; ++k) dd[k] = __shfl_sync(0xffffffffu, own, gi * G + min(k, G - 1));
+                        } else {
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) dd[k] = poly_axis_diff(Xg[k * N + i], Xg[k * N + pv]);
+                        }
+                        const double d = poly_distance(dd[0], dd[1], dd[2]);
+                        if (how == kLate) {
+                            for (int c = li; c < 3; c += G) {
+                                const long long nn =
+                                    poly_rotated(Xg[c * N + pv], __longlong_as_double(S.nx[3 * t + c]), d);
+                                float hi, lo;
+                                grid_to_ff(nn - (c == 0 ? A0 : (c == 1 ? A1 : A2)), hi, lo);
+                                S.nx[3 * t + c] = nn;
+                                ((float *)&S.na[t])[c] = hi;
+                                if (c == 0) S.na[t].w = lo;
+                                else ((float *)&S.nb[t])[c - 1] = lo;
+                            }
+                        }
+                        __syncwarp();
+                    }
+                }
+                const float4 pn = S.na[t], qn = S.nb[t];
+                MovedBead m;
+                m.x = pair_of(-po.x, -pn.x);
+                m.y = pair_of(-po.y, -pn.y);
+                m.z = pair_of(-po.z, -pn.z);
+                m.lx = pair_of(-po.w, -pn.w);
+                m.ly = pair_of(-qo.x, -qn.x);
+                m.lz = pair_of(-qo.y, -qn.y);
+                // the bonds (i-1, i) and (i, i+1): lanes 0 and 1 of the group, or the walker's only lane
+                // for both when G = 1; a broken bond counts as unchanged (the move is rejected)
+                const bool has_l = i > 0, has_r = i + 1 < N;
+                const float ol = has_l ? S.eb[i - 1] : 0.0f, orr = has_r ? S.eb[i] : 0.0f;
+                float nl = ol, nr = orr;
+                if (!MOVES) {
+                    const float4 c = S.nc[t];
+                    if (has_l) nl = acc ? c.y : c.x;
+                    if (has_r) nr = qn.w;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < (G == 1 ? 2 : 1); ++k) {
+                        const bool left = (G == 1) ? k == 0 : li == 0;
+                        if ((G == 1 || li < 2) && (left ? has_l : has_r)) {
+                            const int jb = left ? i - 1 : i + 1;
+                            const float4 r = S.pa[jb];
+                            const float2 u = S.pb[jb];
+                            const float v = bond_or_nan((pn.x - r.x) + (pn.w - r.w), (pn.y - r.y) + (qn.x - u.x),
+                                                        (pn.z - r.z) + (qn.y - u.y), a);
+                            if (left) nl = v;
+                            else nr = v;
+                        }
+                    }
+                    if (G > 1) {  // every lane of the group sees both
+                        nl = __shfl_sync(0xffffffffu, nl, gi * G);
+                        nr = __shfl_sync(0xffffffffu, nr, gi * G + (G > 1 ? 1 : 0));
+                    }
+                }
+                broken = broken || nl != nl || nr != nr;
+                float s = 0.0f, c = 0.0f;
+                if (G == 1) {
+                    s += (nl != nl) ? 0.0f : nl - ol;
+                    const float y = ((nr != nr) ? 0.0f : nr - orr) - c;
                     const float tt = s + y;
                     c = (tt - s) - y;
                     s = tt;
-                }
-            }
-#pragma unroll 2
-            for (int k = 0; k < npl; ++k) {
-                const int j = li + G * k, dj = j - i;
-                if (j < N && (dj > 1 || dj < -1)) {
-                    const float xj = xs[j], yj = xs[N + j], zj = xs[2 * N + j];
-                    const float ljx = xl[j], ljy = xl[N + j], ljz = xl[2 * N + j];
-                    const float ax = (xo - xj) + (lxo - ljx), ay = (yo - yj) + (lyo - ljy), az = (zo - zj) + (lzo - ljz);
-                    const float bx = (xn - xj) + (lxn - ljx), by = (yn - yj) + (lyn - ljy), bz = (zn - zj) + (lzn - ljz);
-                    const float r2o = ax * ax + ay * ay + az * az;
-                    const float r2n = bx * bx + by * by + bz * bz;
-                    const float y = (lj_energy(r2n, a) - lj_energy(r2o, a)) - c;
-                    const float t = s + y;
-                    c = (t - s) - y;
-                    s = t;
-                }
-            }
-            broken = group_any<G>(broken, gi);
-            // |lane sum| >= 2^22 only for overlapping beads: such a move is rejected
-            const bool huge = group_any<G>(!(fabsf(s) < 4194304.0f), gi);
-            // the lanes' compensated sums added in FP32 by a butterfly: every lane adds the same
-            // two operands at every step (a + b = b + a exactly), so all lanes of the group end
-            // with the same sum, converted once to 2^-32 fixed point
-            float lane_sum = s - c;
-#pragma unroll
-            for (int off = G / 2; off; off >>= 1) lane_sum += __shfl_xor_sync(0xffffffffu, lane_sum, off);
-            const long long q = huge ? 0 : f2ll_exact(lane_sum * 0x1p32f);
-            const long long En = E + q;
-            const int bn = poly_bin(En, a);
-            bool acc = false;
-            if (!broken && !huge) {
-                if (b >= 0 && b < a.B) {
-                    if (bn >= 0 && bn < a.B) {
-                        const long long dq = __ldg(a.lnWq + bn) - __ldg(a.lnWq + b);
-                        // accept iff d >= 0 or ln(u 2^-32) < d (the logarithm is in u.w)
-                        acc = dq >= 0 || __uint_as_float(u.w) < q32_to_float(dq);
-                    }
                 } else {
-                    const long long dold = (b < 0) ? a.elo_q - E : E - a.ehi_q;
-                    const long long dnew = (bn < 0) ? a.elo_q - En : (bn >= a.B ? En - a.ehi_q : 0);
-                    acc = dnew <= dold;
+                    const float vn = li == 0 ? nl : nr, vo = li == 0 ? ol : orr;
+                    if (li < 2 && vn == vn) s += vn - vo;  // (+0 where there is no bond)
                 }
-            }
-            if (a.trace && li == 0 && active) {  // parity inspection only
-                PolyTraceRec r;
-                r.dq = q;
-                r.E = acc ? En : E;
-                r.bn = bn;
-                r.b = acc ? bn : b;
-                r.flags = (acc ? 1 : 0) | (broken ? 2 : 0) | (huge ? 4 : 0);
-                r.pad = 0;
-                a.trace[((size_t)w * (size_t)a.trace_sweeps + (size_t)(a.sweep_base + sw)) * (size_t)N + i] = r;
-            }
-            if (acc) {
-                if (G == 1) {
-                    if (i > 0) eb[i - 1] = vnb[0];
-                    if (i + 1 < N) eb[i] = vnb[1];
-                } else if (li < 2) {
-                    const int jb = li == 0 ? i - 1 : i + 1;
-                    if (jb >= 0 && jb < N) eb[jb < i ? jb : i] = vnb[0];
-                }
-                if (li == 0) {
-                    if (active) {
-                        Xg[i] = n0;
-                        Xg[N + i] = n1;
-                        Xg[2 * N + i] = n2;
+                // the other partners, compensated (Kahan)
+#pragma unroll 2
+                for (int k = 0; k < npl; ++k) {
+                    const int j = li + G * k, dj = j - i;
+                    if (j < N && (dj > 1 || dj < -1)) {
+                        const float y = lj_change(S.pa[j], S.pb[j], m, a) - c;
+                        const float tt = s + y;
+                        c = (tt - s) - y;
+                        s = tt;
                     }
-                    xs[i] = xn;
-                    xs[N + i] = yn;
-                    xs[2 * N + i] = zn;
-                    xl[i] = lxn;
-                    xl[N + i] = lyn;
-                    xl[2 * N + i] = lzn;
                 }
-                E = En;
-                b = bn;
-                ++nacc;
+                // |lane sum| >= 2^22 only for overlapping beads: such a move is rejected
+                const bool huge = group_any<G>(!(fabsf(s) < 4194304.0f), gi);
+                // the lanes' compensated sums added in FP32 by a butterfly: every lane adds the same
+                // two operands at every step (a + b = b + a exactly), so all lanes of the group end
+                // with the same sum, converted once to 2^-32 fixed point
+                float lane_sum = s - c;
+#pragma unroll
+                for (int off = G / 2; off; off >>= 1) lane_sum += __shfl_xor_sync(0xffffffffu, lane_sum, off);
+                const long long q = huge ? 0 : f2ll_exact(lane_sum * 0x1p32f);
+                const long long En = E + q;
+                const int bn = poly_bin(En, a);
+                const long long lwn = (bn >= 0 && bn < a.B) ? __ldg(a.lnWq + bn) : 0;
+                acc = false;
+                if (!broken && !huge) {
+                    if (b >= 0 && b < a.B) {
+                        if (bn >= 0 && bn < a.B) {
+                            const long long dq = lwn - lw;
+                            // accept iff d >= 0 or ln(u 2^-32) < d
+                            acc = dq >= 0 || qn.z < q32_to_float(dq);
+                        }
+                    } else {
+                        const long long dold = (b < 0) ? a.elo_q - E : E - a.ehi_q;
+                        const long long dnew = (bn < 0) ? a.elo_q - En : (bn >= a.B ? En - a.ehi_q : 0);
+                        acc = dnew <= dold;
+                    }
+                }
+                if (a.trace && li == 0 && active) {  // parity inspection only
+                    PolyTraceRec r;
+                    r.dq = q;
+                    r.E = acc ? En : E;
+                    r.bn = bn;
+                    r.b = acc ? bn : b;
+                    r.flags = (acc ? 1 : 0) | (broken ? 2 : 0) | (huge ? 4 : 0);
+                    r.pad = 0;
+                    a.trace[((size_t)w * (size_t)a.trace_sweeps + (size_t)(a.sweep_base + sw)) * (size_t)N + i] = r;
+                }
+                if (acc) {
+                    if (li == 0) {
+                        S.pa[i] = pn;
+                        S.pb[i] = make_float2(qn.x, qn.y);
+                        if (has_l) S.eb[i - 1] = nl;
+                        if (has_r) S.eb[i] = nr;
+                        if (MOVES && active) {
+                            Xg[i] = S.nx[3 * t];
+                            Xg[N + i] = S.nx[3 * t + 1];
+                            Xg[2 * N + i] = S.nx[3 * t + 2];
+                        }
+                    }
+                    E = En;
+                    b = bn;
+                    lw = lwn;
+                    ++nacc;
+                    accs |= 1u << t;
+                }
+                __syncwarp();
+                if (a.record == 0 && li == 0 && active && b >= 0 && b < a.B) count_visits(&hs[b], 1u);
             }
-            __syncwarp();
-            if (RECORD == 0 && li == 0 && active && b >= 0 && b < a.B) count_visits(&hs[b], 1u);
+            // ---- the accepted moves on the master coordinates (32 x 32-bit products: the grid step fits an int)
+            if (!MOVES && active) {
+#pragma unroll 1
+                for (int t = li; t < nt; t += G) {
+                    if ((accs >> t) & 1u) {
+                        const float4 c = S.nc[t];
+                        const int j = c0 + t;
+                        Xg[j] += (long long)(int)(__float_as_uint(c.z) ^ 0x80000000u) * (long long)a.step_q;
+                        Xg[N + j] += (long long)(int)(__float_as_uint(c.w) ^ 0x80000000u) * (long long)a.step_q;
+                        Xg[2 * N + j] += (long long)(int)(S.wz[t] ^ 0x80000000u) * (long long)a.step_q;
+                    }
+                }
+            }
+            __syncwarp();  // the chunk's records are rewritten
         }
-        if (RECORD == 1 && li == 0 && active && b >= 0 && b < a.B) count_visits(&hs[b], 1u);
+        if (a.record == 1 && li == 0 && active && b >= 0 && b < a.B) count_visits(&hs[b], 1u);
         tunnel_step(b, 0, a.B - 1, tst, ev);
         __syncwarp();
     }
@@ -532,12 +768,11 @@ cudaError_t launch_poly_energy(const PolyArgs &a, int track_drift, cudaStream_t 
     return cudaGetLastError();
 }
 
-// Shared memory of one warp of the sweep: 32/G walkers' float-pair shadows and Philox blocks.
+// Shared memory of one warp of the sweep: 32/G walkers' slots.
 template <int G>
 static size_t poly_warp_smem(const PolyArgs &a)
 {
-    return (size_t)(32 / G) * ((size_t)poly_slot_floats<G>(a.N) * sizeof(float) +
-                               (size_t)a.N * (a.moves ? 2 : 1) * sizeof(uint4));
+    return (size_t)(32 / G) * (a.moves ? PolySlot<G, 1>::bytes(a.N) : PolySlot<G, 0>::bytes(a.N));
 }
 
 constexpr size_t kPolySmemMax = 227u * 1024u;
@@ -548,11 +783,25 @@ static size_t poly_hist_smem(const PolyArgs &a)
     return ((size_t)(a.B + 1) * sizeof(unsigned) + 15) / 16 * 16;
 }
 
-template <int G>
+// Warps a block when the caller has set none: the walkers' warps spread evenly over the SMs (the
+// fullest SM sets the time: 256-thread blocks put 16 warps on most SMs and 8 on the rest at 4096
+// walkers, where 14 everywhere do), in blocks of at most eight warps.
+static int poly_auto_warps(int p, int walkers_a_warp)
+{
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+        return 8;
+    const int warps = (p + walkers_a_warp - 1) / walkers_a_warp, each = (warps + nsm - 1) / nsm;
+    const int blocks = (each + 7) / 8;
+    return (each + blocks - 1) / blocks;
+}
+
+template <int G, int MOVES>
 static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
 {
     // as many warps of the requested block as fit the shared memory of one block
-    int wpb = block / 32;
+    int wpb = block > 0 ? block / 32 : poly_auto_warps(a.p, 32 / G);
     const size_t per_warp = poly_warp_smem<G>(a), hist = poly_hist_smem(a);
     if (hist + (size_t)wpb * per_warp > kPolySmemMax)
         wpb = hist < kPolySmemMax ? (int)((kPolySmemMax - hist) / per_warp) : 0;
@@ -561,9 +810,7 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
     const int spb = wpb * (32 / G);
     const size_t smem = (size_t)wpb * per_warp + hist;
     const int nblk = (a.p + spb - 1) / spb;
-    cudaError_t e = (a.record == 0)
-                        ? cudaFuncSetAttribute(k_sweep_polymer<G, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                        : cudaFuncSetAttribute(k_sweep_polymer<G, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_sweep_polymer<G, MOVES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // one launch per chunk of sweeps whose visits fit the block's 32-bit counters (spb N a sweep
     // at most), or fewer ("flush_every")
@@ -574,10 +821,7 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
         c.sweep_base = s0;
         c.sweeps = (a.sweeps - s0 < fe) ? a.sweeps - s0 : fe;
         c.trace_sweeps = a.sweeps;
-        if (a.record == 0)
-            k_sweep_polymer<G, 0><<<nblk, block, smem, s>>>(c);
-        else
-            k_sweep_polymer<G, 1><<<nblk, block, smem, s>>>(c);
+        k_sweep_polymer<G, MOVES><<<nblk, block, smem, s>>>(c);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -591,18 +835,21 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
 // 128: fewer lanes share the fixed cost among more walkers but leave 4096 G / 32
 // warps to hide latency (G = 4: 2.1e9 against 3.0e9 attempts/s at N = 13; G = 1:
 // 1.1e9), so 16 stays the default.
-template <int G>
-static bool poly_fits(const PolyArgs &a)
+// (What fits is still counted in the bytes of a slot that holds a whole sweep's random words: the
+// lanes decide the rounding of the FP32 sums, so a request keeps the grouping it always had.  The
+// slots above are smaller where this line matters.)
+static bool poly_fits(const PolyArgs &a, int g)
 {
-    return poly_warp_smem<G>(a) + poly_hist_smem(a) <= kPolySmemMax;
+    const size_t slot = (size_t)((7 * a.N + 3) & ~3) * sizeof(float) + (size_t)a.N * (a.moves ? 2 : 1) * sizeof(uint4);
+    return (size_t)(32 / g) * slot + poly_hist_smem(a) <= kPolySmemMax;
 }
 
 int poly_lanes(const PolyArgs &a, int requested)
 {
     int g = (requested == 1 || requested == 2 || requested == 4 || requested == 8 || requested == 16 ||
              requested == 32) ? requested : 16;
-    if (g == 1 && !poly_fits<1>(a)) g = 2;
-    if (g == 2 && !poly_fits<2>(a)) g = 4;
+    if (g == 1 && !poly_fits(a, 1)) g = 2;
+    if (g == 2 && !poly_fits(a, 2)) g = 4;
     return g;
 }
 
@@ -610,12 +857,12 @@ cudaError_t launch_poly_sweep(const PolyArgs &a, int block, cudaStream_t s)
 {
     if (!polymer_supported(a.N)) return cudaErrorInvalidValue;
     switch (poly_lanes(a, a.lanes)) {
-    case 1: return launch_g<1>(a, block, s);
-    case 2: return launch_g<2>(a, block, s);
-    case 4: return launch_g<4>(a, block, s);
-    case 8: return launch_g<8>(a, block, s);
-    case 16: return launch_g<16>(a, block, s);
-    default: return launch_g<32>(a, block, s);
+    case 1: return a.moves ? launch_g<1, 1>(a, block, s) : launch_g<1, 0>(a, block, s);
+    case 2: return a.moves ? launch_g<2, 1>(a, block, s) : launch_g<2, 0>(a, block, s);
+    case 4: return a.moves ? launch_g<4, 1>(a, block, s) : launch_g<4, 0>(a, block, s);
+    case 8: return a.moves ? launch_g<8, 1>(a, block, s) : launch_g<8, 0>(a, block, s);
+    case 16: return a.moves ? launch_g<16, 1>(a, block, s) : launch_g<16, 0>(a, block, s);
+    default: return a.moves ? launch_g<32, 1>(a, block, s) : launch_g<32, 0>(a, block, s);
     }
 }
 
