@@ -85,18 +85,6 @@ __device__ __forceinline__ long long warp_sum_ll(long long q)
     return q;
 }
 
-// llrint(t) for |t| < 2^62 without a 64-bit conversion instruction (those run on
-// the FP64 pipe, a small fraction of FP32 on GB300): below 2^31 a 32-bit rounding
-// conversion; above, t is an integer m * 2^e with e >= 8, rebuilt from its bits.
-__device__ __forceinline__ long long f2ll_exact(float t)
-{
-    const uint32_t b = __float_as_uint(t);
-    const int e = (int)((b >> 23) & 0xffu) - 150;
-    const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
-    const long long big = (e >= 0 ? (m << (e & 63)) : 0);
-    return fabsf(t) < 2147483648.0f ? (long long)__float2int_rn(t) : ((b >> 31) ? -big : big);
-}
-
 // A 2^-32 fixed-point value as a float, from its two 32-bit halves (32-bit
 // conversions only).
 __device__ __forceinline__ float q32_to_float(long long v)
@@ -108,6 +96,26 @@ __device__ __forceinline__ int poly_bin(long long E, const PolyArgs &a)
 {
     const long long b = ((E - a.elo_q) * a.bin_k) >> 32;
     return b < -1 ? -1 : (b > (long long)a.B ? a.B : (int)b);
+}
+
+// poly_bin of a relative energy r = E - elo_q, from its 32-bit halves: floor(r k 2^-32) is
+// (whole part) k + umulhi(fraction, k) for r >= 0, far above the window past 2^20.
+__device__ __forceinline__ int poly_bin_rel(long long r, const PolyArgs &a)
+{
+    const int hi = (int)(r >> 32);
+    const uint32_t up = min((uint32_t)hi, 1u << 20) * (uint32_t)a.bin_k + __umulhi((uint32_t)r, (uint32_t)a.bin_k);
+    return hi < 0 ? -1 : (int)min(up, (uint32_t)a.B);
+}
+
+// llrint(v 2^32) for |v| < 2^31, through 32-bit conversions: the whole part and the fraction of |v|
+// are exact floats; only a fraction below 2^-8 has bits past 2^-32, rounded to nearest even as v is.
+__device__ __forceinline__ long long float_to_q32(float v)
+{
+    const float m = fabsf(v);
+    const uint32_t whole = (uint32_t)(int)m;
+    const uint32_t frac = __float2uint_rn((m - (float)(int)whole) * 0x1p32f);
+    const long long q = (long long)(((unsigned long long)whole << 32) | frac);
+    return v < 0.0f ? -q : q;
 }
 
 // n visits of a bin: a shared-memory reduction without a returned value, so nothing
@@ -294,37 +302,27 @@ __device__ __forceinline__ float rcp_approx(float x)
     return r;
 }
 
-// Minus the moved bead's position, old in the low halves and new in the high ones.
-struct MovedBead {
-    float_pair x, y, z, lx, ly, lz;
-};
-
-// LJ energy of the moved bead with one partner, new position minus old: lj_energy on both at once.
-// (The squares do not see the sign of a separation.)
-__device__ __forceinline__ float lj_change(const float4 &pj, const float2 &qj, const MovedBead &m, const PolyArgs &a)
+// LJ energies (lj_energy) of a bead at minus (px, py, pz) with two partners, each coordinate a
+// float pair hi + lo; the partners' coordinates are packed, the bead's are in both halves.
+// (The squares do not see the sign of a separation; n6 = -(sigma/r)^6.)
+__device__ __forceinline__ void lj_two(const float4 &j0, const float4 &j1, const float4 &j2, const float4 &b0,
+                                       const float4 &b1, const float4 &b2, const PolyArgs &a, float &v0, float &v1)
 {
-    const float_pair dx = add_pair(add_pair(pair_of(pj.x, pj.x), m.x), add_pair(pair_of(pj.w, pj.w), m.lx));
-    const float_pair dy = add_pair(add_pair(pair_of(pj.y, pj.y), m.y), add_pair(pair_of(qj.x, qj.x), m.ly));
-    const float_pair dz = add_pair(add_pair(pair_of(pj.z, pj.z), m.z), add_pair(pair_of(qj.y, qj.y), m.lz));
-#ifndef POLY_R2
-#define POLY_R2 0
-#endif
-#if POLY_R2 == 0
+    const float_pair dx = add_pair(add_pair(pair_of(j0.x, j0.y), pair_of(b0.x, b0.y)),
+                                   add_pair(pair_of(j1.z, j1.w), pair_of(b1.z, b1.w)));
+    const float_pair dy = add_pair(add_pair(pair_of(j0.z, j0.w), pair_of(b0.z, b0.w)),
+                                   add_pair(pair_of(j2.x, j2.y), pair_of(b2.x, b2.y)));
+    const float_pair dz = add_pair(add_pair(pair_of(j1.x, j1.y), pair_of(b1.x, b1.y)),
+                                   add_pair(pair_of(j2.z, j2.w), pair_of(b2.z, b2.w)));
     const float_pair r2 = fma_pair(dz, dz, fma_pair(dx, dx, mul_pair(dy, dy)));
-#else
-    const float_pair r2 = fma_pair(dz, dz, fma_pair(dy, dy, mul_pair(dx, dx)));
-#endif
-    float r2o, r2n;
-    halves_of(r2, r2o, r2n);
-    const float_pair ir2 = mul_pair(pair_of(rcp_approx(r2o), rcp_approx(r2n)), pair_of(a.lj_sigma2, a.lj_sigma2));
-    const float_pair ir6 = mul_pair(mul_pair(ir2, ir2), ir2);
-    float ho, hn;
-    halves_of(ir6, ho, hn);
-    const float_pair v = fma_pair(pair_of(fmaf(ho, ho, -ho), fmaf(hn, hn, -hn)), pair_of(4.0f, 4.0f),
-                                  pair_of(-a.lj_shift, -a.lj_shift));
-    float vo, vn;
-    halves_of(v, vo, vn);
-    return (r2n < a.lj_rc2 ? vn : 0.0f) - (r2o < a.lj_rc2 ? vo : 0.0f);
+    float r0, r1;
+    halves_of(r2, r0, r1);
+    const float_pair n2 = mul_pair(pair_of(rcp_approx(r0), rcp_approx(r1)), pair_of(-a.lj_sigma2, -a.lj_sigma2));
+    const float_pair n6 = mul_pair(mul_pair(n2, n2), n2);
+    const float_pair v = fma_pair(fma_pair(n6, n6, n6), pair_of(4.0f, 4.0f), pair_of(-a.lj_shift, -a.lj_shift));
+    halves_of(v, v0, v1);
+    v0 = r0 < a.lj_rc2 ? v0 : 0.0f;
+    v1 = r1 < a.lj_rc2 ? v1 : 0.0f;
 }
 
 // Energy of a new bond over the separation (bx, by, bz), NaN if it breaks.
@@ -334,69 +332,170 @@ __device__ __forceinline__ float bond_or_nan(float bx, float by, float bz, const
     return fene_intact(r2n, a) ? fene_energy(r2n, a) : __int_as_float(0x7fffffff);
 }
 
-// Shared memory of one walker's slot.  Beads: the float-pair shadows, (x, y, z, lo x) in pa and
-// (lo y, lo z) in pb, and the energies eb of the N - 1 bonds.  The chunk of beads being visited
-// (poly_chunk of them at a time): the proposed shadows and what else an attempt needs of its own
-// bead.  Every attempt's loads are then two wide ones a partner and three for the moved bead.
+// A bead's float-pair shadow.
+struct Shadow {
+    float c[6];  // x, y, z, lo x, lo y, lo z
+};
+__device__ __forceinline__ float bond_between(const Shadow &p, const Shadow &r, const PolyArgs &a)
+{
+    return bond_or_nan((p.c[0] - r.c[0]) + (p.c[3] - r.c[3]), (p.c[1] - r.c[1]) + (p.c[4] - r.c[4]),
+                       (p.c[2] - r.c[2]) + (p.c[5] - r.c[5]), a);
+}
+
+// Shared memory of one walker's slot.  The shadows of all beads are in pos, two partners of a lane
+// (beads j and j + G) side by side so that one packed instruction takes both: 4-vectors
+// (x x' y y'), (z z' lo x, lo x'), (lo y, lo y', lo z, lo z'), nP of each.  With at most one partner
+// a lane (ONE, N <= G) both halves hold bead j, and the packed instruction takes the moved bead's
+// old and proposed place at once.  eb[j] is the energy of
+// the bond (j - 1, j), 0 at both ends.  The chunk of beads being visited (poly_chunk of them at a
+// time): minus the bead's old and proposed shadow, each number twice (twelve 2-vectors in six
+// 4-vectors, in the order of pos; ONE: old and proposed side by side, three), and rec = (energy of the left bond with the bead moved: left bead
+// where it was / left bead moved; energy of the right bond; ln of the acceptance word).
 template <int G>
 __host__ __device__ constexpr int poly_chunk() { return G > 16 ? G : 16; }
 
-template <int G, int MOVES>
+template <int G, int MOVES, bool ONE>
 struct PolySlot {
     static constexpr int CH = poly_chunk<G>();
-    float4 *pa;      // [N]
-    float4 *na;      // [CH] proposed x, y, z, lo x
-    float4 *nb;      // [CH] proposed lo y, lo z; ln of the acceptance word; energy of bond (j, j+1), j moved
-    float4 *nc;      // [CH] energy of bond (j-1, j), j moved: j-1 where it was, j-1 moved; random words x, y
-    float2 *pb;      // [N]
+    static constexpr int BV = ONE ? 3 : 6;  // 4-vectors of a chunk bead
+    float4 *pos;     // [3][nP]
+    float4 *bead;    // [CH][BV]
+    float4 *rec;     // [CH]
     long long *nx;   // [CH][3] (MOVES) proposed grid position, or the rotation's unit vector
-    float *eb;       // [N]
-    uint32_t *wz;    // [CH] random word z
-    uint32_t *how;   // [CH] (MOVES) kReady, kLate, kNoPoint
+    uint32_t *how;   // [CH] (MOVES) kReady, kLate, kNoPoint; else [CH][3] the random words of the step
+    float *eb;       // [N + 1]
+    int nP;
+    static __host__ __device__ int pairs(int N) { return ONE ? G : (N + 2 * G - 1) / (2 * G) * G; }
     static __host__ __device__ size_t bytes(int N)
     {
-        const size_t b = (size_t)N * 28 + CH * (size_t)(48 + 4 + (MOVES ? 28 : 0));
+        const size_t b = (size_t)48 * pairs(N) + (size_t)CH * (16 * BV + 16 + (MOVES ? 28 : 12)) + 4 * (size_t)(N + 1);
         return (b + 15) / 16 * 16;
     }
     __device__ PolySlot(unsigned char *p, int N)
     {
-        pa = (float4 *)p;
-        na = pa + N;
-        nb = na + CH;
-        nc = nb + CH;
-        pb = (float2 *)(nc + CH);
-        nx = (long long *)(pb + N);
-        eb = (float *)(MOVES ? nx + 3 * CH : nx);
-        wz = (uint32_t *)(eb + N);
-        how = wz + CH;
+        nP = pairs(N);
+        pos = (float4 *)p;
+        bead = pos + 3 * nP;
+        rec = bead + BV * CH;
+        nx = (long long *)(rec + CH);
+        how = (uint32_t *)(MOVES ? nx + 3 * CH : nx);
+        eb = (float *)(how + (MOVES ? CH : 3 * CH));
+    }
+    // component c (in the order x y | z lx | ly lz of pos) of bead j
+    __device__ float *at(int j, int c) const
+    {
+        if (ONE) return (float *)(pos + (c >> 1) * nP + j) + 2 * (c & 1);
+        const int idx = j / (2 * G) * G + j % G, half = (j / G) & 1;
+        return (float *)(pos + (c >> 1) * nP + idx) + 2 * (c & 1) + half;
+    }
+    __device__ void set(int j, int c, float v) const
+    {
+        if (ONE) *(float2 *)at(j, c) = make_float2(v, v);
+        else *at(j, c) = v;
+    }
+    __device__ Shadow get(int j) const
+    {
+        return Shadow{{*at(j, 0), *at(j, 1), *at(j, 2), *at(j, 3), *at(j, 4), *at(j, 5)}};
+    }
+    __device__ void put(int j, const Shadow &s) const
+    {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) set(j, c, s.c[c]);
+    }
+    // minus component c of the proposed shadow of chunk bead t
+    __device__ float proposed(int t, int c) const
+    {
+        return ONE ? ((float *)(bead + 3 * t))[2 * c + 1] : ((float *)(bead + 6 * t + 3))[2 * c];
+    }
+    __device__ void set_proposed(int t, int c, float v) const
+    {
+        if (ONE) ((float *)(bead + 3 * t))[2 * c + 1] = -v;
+        else *(float2 *)((float *)(bead + 6 * t + 3) + 2 * c) = make_float2(-v, -v);
+    }
+    __device__ Shadow get_proposed(int t) const
+    {
+        return Shadow{{-proposed(t, 0), -proposed(t, 1), -proposed(t, 2), -proposed(t, 3), -proposed(t, 4),
+                       -proposed(t, 5)}};
+    }
+    __device__ void put_bead(int t, const Shadow &o, const Shadow &n) const
+    {
+        float4 *b = bead + BV * t;
+        if (ONE) {
+            b[0] = make_float4(-o.c[0], -n.c[0], -o.c[1], -n.c[1]);
+            b[1] = make_float4(-o.c[2], -n.c[2], -o.c[3], -n.c[3]);
+            b[2] = make_float4(-o.c[4], -n.c[4], -o.c[5], -n.c[5]);
+        } else {
+            b[0] = make_float4(-o.c[0], -o.c[0], -o.c[1], -o.c[1]);
+            b[1] = make_float4(-o.c[2], -o.c[2], -o.c[3], -o.c[3]);
+            b[2] = make_float4(-o.c[4], -o.c[4], -o.c[5], -o.c[5]);
+            b[BV - 3] = make_float4(-n.c[0], -n.c[0], -n.c[1], -n.c[1]);
+            b[BV - 2] = make_float4(-n.c[2], -n.c[2], -n.c[3], -n.c[3]);
+            b[BV - 1] = make_float4(-n.c[4], -n.c[4], -n.c[5], -n.c[5]);
+        }
     }
 };
+
+// LJ energy changes of chunk bead t with this lane's partners of 4-vector k: of both (new minus old),
+// or of the one (ONE, d1 unused).
+template <class SLOT, bool ONE>
+__device__ __forceinline__ void lj_changes(const SLOT &S, int t, int k, const PolyArgs &a, float &d0, float &d1)
+{
+    const float4 j0 = S.pos[k], j1 = S.pos[S.nP + k], j2 = S.pos[2 * S.nP + k];
+    const float4 *own = S.bead + SLOT::BV * t;
+    float vo0, vo1, vn0, vn1;
+    lj_two(j0, j1, j2, own[0], own[1], own[2], a, vo0, vo1);
+    if (ONE) {  // (old, new) of one partner
+        d0 = vo1 - vo0;
+        d1 = 0.0f;
+        return;
+    }
+    lj_two(j0, j1, j2, own[SLOT::BV - 3], own[SLOT::BV - 2], own[SLOT::BV - 1], a, vn0, vn1);
+    d0 = vn0 - vo0;
+    d1 = vn1 - vo1;
+}
+
+__device__ __forceinline__ void kahan_add(float &s, float &c, float v)
+{
+    const float y = v - c;
+    const float t = s + y;
+    c = (t - s) - y;
+    s = t;
+}
 enum : uint32_t { kReady = 0u, kLate = 1u, kNoPoint = 2u };
 
 // Sweeps: G lanes per walker, 32/G walkers a warp, all on the same bead i.  The two bonds of bead i
 // (FENE) are taken by lanes 0 and 1 of the group, the other partners (LJ, |i - j| >= 2) by lanes
 // j mod G, in ascending order, so the FP32 sums do not depend on anything else.
 //
-// Bound by issue (3.4 warps a scheduler at 4096 walkers; of 370 warp instructions an attempt at
-// N = 13 one seventh was pair work), so what is not pair work is taken out of the serial loop: a
-// bead is visited once a sweep and stands still until then, so its random words, its proposed
-// position and the energies of its new bonds (the left one for both outcomes of the bead before it)
-// are known before the loop reaches it.  Every lane prepares its own beads of the next poly_chunk
-// beads, and the attempt only reads them.  Accepted moves reach the int64 master coordinates behind
-// the chunk, in parallel again.  Old and new pair energies go through packed instructions
-// (lj_change).  With rotations (MOVES) a proposal about bead i - 1 needs that bead's outcome: its
-// unit vector is prepared, the position (binary64, one axis a lane) made when the bead is reached.
-template <int G, int MOVES>
+// Bound by issue and by fixed latencies (3.4 warps a scheduler at 4096 walkers), so what is not pair
+// work is taken out of the serial loop: a bead is visited once a sweep and stands still until then,
+// so its random words, its proposed position and the energies of its new bonds (the left one for
+// both outcomes of the bead before it) are known before the loop reaches it.  Every lane prepares
+// its own beads of the next poly_chunk beads, and the attempt only reads them.  Accepted moves reach
+// the int64 master coordinates behind the chunk, in parallel again.  Pair energies are evaluated for
+// two partners at once in packed instructions (lj_two).  With rotations (MOVES) a proposal about
+// bead i - 1 needs that bead's outcome: its unit vector is prepared, the position (binary64, one
+// axis a lane) made when the bead is reached.
+//
+// NP > 0 (shifts, NP 4-vectors of partners a lane; kOnePartner: N <= G): the pair terms of bead
+// i + 1 do not depend on the outcome of bead i, which is bonded to it, so they are evaluated beside
+// the sum, the conversion, the table load and the decision of bead i, whose latencies they fill.
+// NP = 0 evaluates them in the attempt (any N).
+constexpr int kOnePartner = 5;
+template <int G, int MOVES, int NP>
 __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs a)
 {
     constexpr int W = 32 / G;
     constexpr int CH = poly_chunk<G>();
+    constexpr bool ONE = NP == kOnePartner;
+    constexpr int NV = ONE ? 1 : (NP > 0 ? NP : 1);  // 4-vectors evaluated ahead
+    using Slot = PolySlot<G, MOVES, ONE>;
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5, N = a.N;
     const int gi = lane / G, li = lane % G;
     const int spb = wpb * W, slot = wib * W + gi;
-    const size_t sst = PolySlot<G, MOVES>::bytes(N);
-    const PolySlot<G, MOVES> S(smem + slot * sst, N);
+    const size_t sst = Slot::bytes(N);
+    const Slot S(smem + slot * sst, N);
     // the block's histogram counters and its count of finished warps, behind all slots
     unsigned *hs = (unsigned *)(smem + spb * sst);
     unsigned *done = hs + a.B;
@@ -406,14 +505,15 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
     if (w0 >= a.p) return;  // whole warps only; no block-wide barrier follows
     const int w = w0 + gi;
     const bool active = w < a.p;
+    const bool counts = active && li == 0;  // the lane that counts its walker's visits
     const int wr = active ? w : w0;  // a group past the last walker shadows the warp's first one, read-only
     const uint32_t wid = (uint32_t)(wr + a.walker_offset);
     long long *Xg = a.X + (size_t)wr * 3 * N;
-    long long E = a.E[wr];
-    int b = poly_bin(E, a);
-    long long lw = (b >= 0 && b < a.B) ? __ldg(a.lnWq + b) : 0;  // ln W of the current bin
+    long long E = a.E[wr] - a.elo_q;  // energies relative to the window
+    int b = poly_bin_rel(E, a);
+    bool inside = (unsigned)b < (unsigned)a.B;
+    long long lw = __ldg(a.lnWq + (inside ? b : 0));  // ln W of the current bin
     const uint32_t g0 = (uint32_t)(a.state->sweep_counter + a.sweep_base);
-    const int npl = (N + G - 1) / G;
     // metrics: accepted moves and tunnelling between bins 0 and B-1 (group-uniform values)
     unsigned long long nacc = 0;
     unsigned ev = 0;
@@ -423,22 +523,23 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
         const uint32_t g = g0 + (uint32_t)sw;
         const long long A0 = Xg[0], A1 = Xg[N], A2 = Xg[2 * N];
         for (int j = li; j < N; j += G) {
-            float4 p;
-            float2 q;
-            grid_to_ff(Xg[j] - A0, p.x, p.w);
-            grid_to_ff(Xg[N + j] - A1, p.y, q.x);
-            grid_to_ff(Xg[2 * N + j] - A2, p.z, q.y);
-            S.pa[j] = p;
-            S.pb[j] = q;
+            Shadow p;
+            grid_to_ff(Xg[j] - A0, p.c[0], p.c[3]);
+            grid_to_ff(Xg[N + j] - A1, p.c[1], p.c[4]);
+            grid_to_ff(Xg[2 * N + j] - A2, p.c[2], p.c[5]);
+            S.put(j, p);
         }
         __syncwarp();
-        for (int j = li; j + 1 < N; j += G) {
-            const float4 p = S.pa[j], r = S.pa[j + 1];
-            const float2 q = S.pb[j], t = S.pb[j + 1];
-            const float dx = (p.x - r.x) + (p.w - r.w);
-            const float dy = (p.y - r.y) + (q.x - t.x);
-            const float dz = (p.z - r.z) + (q.y - t.y);
-            S.eb[j] = fene_energy(dx * dx + dy * dy + dz * dz, a);
+        for (int j = li; j <= N; j += G) {
+            float v = 0.0f;
+            if (j > 0 && j < N) {
+                const Shadow p = S.get(j - 1), r = S.get(j);
+                const float dx = (p.c[0] - r.c[0]) + (p.c[3] - r.c[3]);
+                const float dy = (p.c[1] - r.c[1]) + (p.c[4] - r.c[4]);
+                const float dz = (p.c[2] - r.c[2]) + (p.c[5] - r.c[5]);
+                v = fene_energy(dx * dx + dy * dy + dz * dz, a);
+            }
+            S.eb[j] = v;
         }
 #pragma unroll 1
         for (int c0 = 0; c0 < N; c0 += CH) {
@@ -452,12 +553,11 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 // coordinates; the float-pair shadow moves by the same amount in FP32
                 // (the shadows are rebuilt exactly from the masters every sweep)
                 const int sx = (int)(r.x ^ 0x80000000u), sy = (int)(r.y ^ 0x80000000u), sz = (int)(r.z ^ 0x80000000u);
-                const float4 p = S.pa[j];
-                const float2 q = S.pb[j];
+                const Shadow p = S.get(j);
                 const float dx = (float)sx * kStep, dy = (float)sy * kStep, dz = (float)sz * kStep;
-                const float xo = p.x, yo = p.y, zo = p.z;
+                const float xo = p.c[0], yo = p.c[1], zo = p.c[2];
                 float xn = xo + dx, yn = yo + dy, zn = zo + dz;
-                float lxn = p.w + ((xo - xn) + dx), lyn = q.x + ((yo - yn) + dy), lzn = q.y + ((zo - zn) + dz);
+                float lxn = p.c[3] + ((xo - xn) + dx), lyn = p.c[4] + ((yo - yn) + dy), lzn = p.c[5] + ((zo - zn) + dz);
                 if (MOVES) {
                     const long long X0 = Xg[j], X1 = Xg[N + j], X2 = Xg[2 * N + j];
                     long long n0 = X0 + (long long)sx * (long long)a.step_q, n1 = X1 + (long long)sy * (long long)a.step_q,
@@ -489,16 +589,15 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                     S.nx[3 * t + 1] = n1;
                     S.nx[3 * t + 2] = n2;
                     S.how[t] = how;
+                } else {
+                    S.how[3 * t] = r.x;
+                    S.how[3 * t + 1] = r.y;
+                    S.how[3 * t + 2] = r.z;
                 }
-                S.na[t] = make_float4(xn, yn, zn, lxn);
+                S.put_bead(t, p, Shadow{{xn, yn, zn, lxn, lyn, lzn}});
                 // the acceptance test u 2^-32 < exp(d) is taken as ln(u 2^-32) < d: the logarithm
                 // (FP32, -inf for u = 0) is taken here, off the serial path
-                S.nb[t] = make_float4(lyn, lzn, logf((float)r.w * 0x1p-32f), 0.0f);
-                if (!MOVES) {
-                    S.nc[t].z = __uint_as_float(r.x);
-                    S.nc[t].w = __uint_as_float(r.y);
-                    S.wz[t] = r.z;
-                }
+                S.rec[t] = make_float4(0.0f, 0.0f, 0.0f, logf((float)r.w * 0x1p-32f));
             }
             __syncwarp();
             if (!MOVES) {
@@ -506,24 +605,11 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 for (int t = li; t < CH; t += G) {
                     const int j = c0 + t;
                     if (j >= N) break;
-                    const float4 p = S.na[t], q = S.nb[t];
-                    if (j + 1 < N) {
-                        const float4 r = S.pa[j + 1];
-                        const float2 u = S.pb[j + 1];
-                        S.nb[t].w = bond_or_nan((p.x - r.x) + (p.w - r.w), (p.y - r.y) + (q.x - u.x),
-                                                (p.z - r.z) + (q.y - u.y), a);
-                    }
-                    if (j > 0) {
-                        const float4 r = S.pa[j - 1];
-                        const float2 u = S.pb[j - 1];
-                        S.nc[t].x = bond_or_nan((p.x - r.x) + (p.w - r.w), (p.y - r.y) + (q.x - u.x),
-                                                (p.z - r.z) + (q.y - u.y), a);
-                    }
-                    if (t > 0) {  // (the bead before the chunk stands where pa has it)
-                        const float4 r = S.na[t - 1], u = S.nb[t - 1];
-                        S.nc[t].y = bond_or_nan((p.x - r.x) + (p.w - r.w), (p.y - r.y) + (q.x - u.x),
-                                                (p.z - r.z) + (q.y - u.y), a);
-                    }
+                    const Shadow p = S.get_proposed(t);
+                    if (j > 0) S.rec[t].x = bond_between(p, S.get(j - 1), a);
+                    // (the bead before the chunk stands where pos has it)
+                    if (t > 0) S.rec[t].y = bond_between(p, S.get_proposed(t - 1), a);
+                    if (j + 1 < N) S.rec[t].z = bond_between(p, S.get(j + 1), a);
                 }
                 __syncwarp();
             }
@@ -531,15 +617,18 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
             const int nt = min(CH, N - c0);
             uint32_t accs = 0u;   // accepted beads of the chunk (group-uniform)
             bool acc = false;     // the bead before was moved
+            float dn[2 * NV];     // pair terms of the next attempt
+            if (NP > 0) {
+#pragma unroll
+                for (int m = 0; m < NV; ++m) lj_changes<Slot, ONE>(S, 0, G * m + li, a, dn[2 * m], dn[2 * m + 1]);
+            }
 #pragma unroll 1
             for (int t = 0; t < nt; ++t) {
                 const int i = c0 + t;
-                const float4 po = S.pa[i];
-                const float2 qo = S.pb[i];
-                bool broken = false;
+                bool no_point = false;
                 if (MOVES) {
                     const uint32_t how = S.how[t];
-                    broken = how == kNoPoint;
+                    no_point = how == kNoPoint;
                     if (__any_sync(0xffffffffu, how == kLate)) {
                         // about bead i - 1, where it is now; lanes 0, 1, 2 of the group an axis each
                         // (fewer lanes take the axes in turn)
@@ -562,146 +651,133 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                                 float hi, lo;
                                 grid_to_ff(nn - (c == 0 ? A0 : (c == 1 ? A1 : A2)), hi, lo);
                                 S.nx[3 * t + c] = nn;
-                                ((float *)&S.na[t])[c] = hi;
-                                if (c == 0) S.na[t].w = lo;
-                                else ((float *)&S.nb[t])[c - 1] = lo;
+                                S.set_proposed(t, c, hi);
+                                S.set_proposed(t, 3 + c, lo);
                             }
                         }
                         __syncwarp();
                     }
                 }
-                const float4 pn = S.na[t], qn = S.nb[t];
-                MovedBead m;
-                m.x = pair_of(-po.x, -pn.x);
-                m.y = pair_of(-po.y, -pn.y);
-                m.z = pair_of(-po.z, -pn.z);
-                m.lx = pair_of(-po.w, -pn.w);
-                m.ly = pair_of(-qo.x, -qn.x);
-                m.lz = pair_of(-qo.y, -qn.y);
+                const float4 rec = S.rec[t];
                 // the bonds (i-1, i) and (i, i+1): lanes 0 and 1 of the group, or the walker's only lane
                 // for both when G = 1; a broken bond counts as unchanged (the move is rejected)
-                const bool has_l = i > 0, has_r = i + 1 < N;
-                const float ol = has_l ? S.eb[i - 1] : 0.0f, orr = has_r ? S.eb[i] : 0.0f;
-                float nl = ol, nr = orr;
-                if (!MOVES) {
-                    const float4 c = S.nc[t];
-                    if (has_l) nl = acc ? c.y : c.x;
-                    if (has_r) nr = qn.w;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < (G == 1 ? 2 : 1); ++k) {
-                        const bool left = (G == 1) ? k == 0 : li == 0;
-                        if ((G == 1 || li < 2) && (left ? has_l : has_r)) {
-                            const int jb = left ? i - 1 : i + 1;
-                            const float4 r = S.pa[jb];
-                            const float2 u = S.pb[jb];
-                            const float v = bond_or_nan((pn.x - r.x) + (pn.w - r.w), (pn.y - r.y) + (qn.x - u.x),
-                                                        (pn.z - r.z) + (qn.y - u.y), a);
-                            if (left) nl = v;
-                            else nr = v;
-                        }
-                    }
-                    if (G > 1) {  // every lane of the group sees both
-                        nl = __shfl_sync(0xffffffffu, nl, gi * G);
-                        nr = __shfl_sync(0xffffffffu, nr, gi * G + (G > 1 ? 1 : 0));
-                    }
-                }
-                broken = broken || nl != nl || nr != nr;
                 float s = 0.0f, c = 0.0f;
-                if (G == 1) {
-                    s += (nl != nl) ? 0.0f : nl - ol;
-                    const float y = ((nr != nr) ? 0.0f : nr - orr) - c;
-                    const float tt = s + y;
-                    c = (tt - s) - y;
-                    s = tt;
-                } else {
-                    const float vn = li == 0 ? nl : nr, vo = li == 0 ? ol : orr;
-                    if (li < 2 && vn == vn) s += vn - vo;  // (+0 where there is no bond)
+                bool broken = false;
+                float vb[2] = {0.0f, 0.0f};
+#pragma unroll
+                for (int k = 0; k < (G == 1 ? 2 : 1); ++k) {
+                    const bool left = (G == 1) ? k == 0 : li == 0;
+                    float vn = left ? (acc ? rec.y : rec.x) : rec.z;
+                    const float vo = S.eb[left ? i : i + 1];
+                    if (MOVES) {
+                        vn = 0.0f;
+                        if ((G == 1 || li < 2) && (left ? i > 0 : i + 1 < N))
+                            vn = bond_between(S.get_proposed(t), S.get(left ? i - 1 : i + 1), a);
+                    }
+                    if (G == 1 || li < 2) {
+                        broken = broken || vn != vn;
+                        vb[k] = vn;
+                        kahan_add(s, c, vn == vn ? vn - vo : 0.0f);
+                    }
                 }
-                // the other partners, compensated (Kahan)
-#pragma unroll 2
-                for (int k = 0; k < npl; ++k) {
-                    const int j = li + G * k, dj = j - i;
-                    if (j < N && (dj > 1 || dj < -1)) {
-                        const float y = lj_change(S.pa[j], S.pb[j], m, a) - c;
-                        const float tt = s + y;
-                        c = (tt - s) - y;
-                        s = tt;
+                // the other partners, in order, compensated (Kahan); li + 2 G m - i + 1 is 0, 1, 2 for
+                // the bonded beads and i itself
+                const unsigned u = (unsigned)(li - i + 1);
+                if (NP > 0) {
+#pragma unroll
+                    for (int m = 0; m < NV; ++m) {
+                        const int j = li + 2 * G * m;
+                        if (u + 2 * G * m > 2u && j < N) kahan_add(s, c, dn[2 * m]);
+                        if (!ONE && u + 2 * G * m + G > 2u && j + G < N) kahan_add(s, c, dn[2 * m + 1]);
+                    }
+                    const int tn = min(t + 1, CH - 1);  // (behind the chunk's end: not used)
+#pragma unroll
+                    for (int m = 0; m < NV; ++m) lj_changes<Slot, ONE>(S, tn, G * m + li, a, dn[2 * m], dn[2 * m + 1]);
+                } else {
+#pragma unroll 1
+                    for (int m = 0; li + 2 * G * m < N; ++m) {
+                        float d0, d1;
+                        lj_changes<Slot, ONE>(S, t, G * m + li, a, d0, d1);
+                        if (u + 2 * G * m > 2u) kahan_add(s, c, d0);
+                        if (u + 2 * G * m + G > 2u && li + 2 * G * m + G < N) kahan_add(s, c, d1);
                     }
                 }
                 // |lane sum| >= 2^22 only for overlapping beads: such a move is rejected
-                const bool huge = group_any<G>(!(fabsf(s) < 4194304.0f), gi);
+                const bool huge = !(fabsf(s) < 4194304.0f);
+                const bool refused = group_any<G>(huge || broken, gi) || no_point;
                 // the lanes' compensated sums added in FP32 by a butterfly: every lane adds the same
                 // two operands at every step (a + b = b + a exactly), so all lanes of the group end
                 // with the same sum, converted once to 2^-32 fixed point
                 float lane_sum = s - c;
 #pragma unroll
                 for (int off = G / 2; off; off >>= 1) lane_sum += __shfl_xor_sync(0xffffffffu, lane_sum, off);
-                const long long q = huge ? 0 : f2ll_exact(lane_sum * 0x1p32f);
+                const long long q = float_to_q32(lane_sum);  // (a refused move's is not used)
                 const long long En = E + q;
-                const int bn = poly_bin(En, a);
-                const long long lwn = (bn >= 0 && bn < a.B) ? __ldg(a.lnWq + bn) : 0;
-                acc = false;
-                if (!broken && !huge) {
-                    if (b >= 0 && b < a.B) {
-                        if (bn >= 0 && bn < a.B) {
-                            const long long dq = lwn - lw;
-                            // accept iff d >= 0 or ln(u 2^-32) < d
-                            acc = dq >= 0 || qn.z < q32_to_float(dq);
-                        }
-                    } else {
-                        const long long dold = (b < 0) ? a.elo_q - E : E - a.ehi_q;
-                        const long long dnew = (bn < 0) ? a.elo_q - En : (bn >= a.B ? En - a.ehi_q : 0);
-                        acc = dnew <= dold;
-                    }
+                const int bn = poly_bin_rel(En, a);
+                const bool lands = (unsigned)bn < (unsigned)a.B;
+                const long long lwn = __ldg(a.lnWq + (lands ? bn : 0));
+                const long long dq = lwn - lw;
+                // accept iff d >= 0 or ln(u 2^-32) < d
+                acc = lands && (dq >= 0 || rec.w < q32_to_float(dq));
+                if (!inside) {  // walking in: not further from the window than before
+                    const long long span = a.ehi_q - a.elo_q;
+                    const long long dold = (b < 0) ? -E : E - span;
+                    const long long dnew = (bn < 0) ? -En : (bn >= a.B ? En - span : 0);
+                    acc = dnew <= dold;
                 }
-                if (a.trace && li == 0 && active) {  // parity inspection only
+                acc = acc && !refused;
+                if (a.trace) {  // parity inspection only
+                    const bool any_huge = group_any<G>(huge, gi), any_broken = group_any<G>(broken, gi) || no_point;
                     PolyTraceRec r;
-                    r.dq = q;
-                    r.E = acc ? En : E;
-                    r.bn = bn;
+                    r.dq = any_huge ? 0 : q;
+                    r.E = (acc ? En : E) + a.elo_q;
+                    r.bn = any_huge ? poly_bin_rel(E, a) : bn;
                     r.b = acc ? bn : b;
-                    r.flags = (acc ? 1 : 0) | (broken ? 2 : 0) | (huge ? 4 : 0);
+                    r.flags = (acc ? 1 : 0) | (any_broken ? 2 : 0) | (any_huge ? 4 : 0);
                     r.pad = 0;
-                    a.trace[((size_t)w * (size_t)a.trace_sweeps + (size_t)(a.sweep_base + sw)) * (size_t)N + i] = r;
+                    if (counts)
+                        a.trace[((size_t)w * (size_t)a.trace_sweeps + (size_t)(a.sweep_base + sw)) * (size_t)N + i] = r;
                 }
                 if (acc) {
-                    if (li == 0) {
-                        S.pa[i] = pn;
-                        S.pb[i] = make_float2(qn.x, qn.y);
-                        if (has_l) S.eb[i - 1] = nl;
-                        if (has_r) S.eb[i] = nr;
-                        if (MOVES && active) {
-                            Xg[i] = S.nx[3 * t];
-                            Xg[N + i] = S.nx[3 * t + 1];
-                            Xg[2 * N + i] = S.nx[3 * t + 2];
-                        }
+                    for (int k = li; k < 6; k += G) {
+                        // shadow component k (x y z and their lo parts), as bead holds it, to pos
+                        S.set(i, k, -S.proposed(t, k));
+                    }
+                    if (G == 1) {
+                        if (i > 0) S.eb[i] = vb[0];
+                        if (i + 1 < N) S.eb[i + 1] = vb[1];
+                    } else if (li < 2) {
+                        S.eb[li == 0 ? i : i + 1] = vb[0];
+                    }
+                    if (MOVES && counts) {
+                        Xg[i] = S.nx[3 * t];
+                        Xg[N + i] = S.nx[3 * t + 1];
+                        Xg[2 * N + i] = S.nx[3 * t + 2];
                     }
                     E = En;
                     b = bn;
                     lw = lwn;
-                    ++nacc;
+                    inside = lands;
                     accs |= 1u << t;
                 }
                 __syncwarp();
-                if (a.record == 0 && li == 0 && active && b >= 0 && b < a.B) count_visits(&hs[b], 1u);
+                if (a.record == 0 && counts && inside) count_visits(&hs[b], 1u);
             }
+            nacc += (unsigned)__popc(accs);
             // ---- the accepted moves on the master coordinates (32 x 32-bit products: the grid step fits an int)
             if (!MOVES && active) {
 #pragma unroll 1
                 for (int t = li; t < nt; t += G) {
                     if ((accs >> t) & 1u) {
-                        const float4 c = S.nc[t];
-                        const int j = c0 + t;
-                        Xg[j] += (long long)(int)(__float_as_uint(c.z) ^ 0x80000000u) * (long long)a.step_q;
-                        Xg[N + j] += (long long)(int)(__float_as_uint(c.w) ^ 0x80000000u) * (long long)a.step_q;
-                        Xg[2 * N + j] += (long long)(int)(S.wz[t] ^ 0x80000000u) * (long long)a.step_q;
+#pragma unroll
+                        for (int c = 0; c < 3; ++c)
+                            Xg[c * N + c0 + t] += (long long)(int)(S.how[3 * t + c] ^ 0x80000000u) * (long long)a.step_q;
                     }
                 }
             }
             __syncwarp();  // the chunk's records are rewritten
         }
-        if (a.record == 1 && li == 0 && active && b >= 0 && b < a.B) count_visits(&hs[b], 1u);
+        if (a.record == 1 && counts && inside) count_visits(&hs[b], 1u);
         tunnel_step(b, 0, a.B - 1, tst, ev);
         __syncwarp();
     }
@@ -732,7 +808,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
         Xg[2 * N + t] -= A2;
     }
     if (li == 0) {
-        a.E[w] = E;
+        a.E[w] = E + a.elo_q;
         a.bin[w] = b;
     }
 }
@@ -769,10 +845,10 @@ cudaError_t launch_poly_energy(const PolyArgs &a, int track_drift, cudaStream_t 
 }
 
 // Shared memory of one warp of the sweep: 32/G walkers' slots.
-template <int G>
+template <int G, int MOVES, int NP>
 static size_t poly_warp_smem(const PolyArgs &a)
 {
-    return (size_t)(32 / G) * (a.moves ? PolySlot<G, 1>::bytes(a.N) : PolySlot<G, 0>::bytes(a.N));
+    return (size_t)(32 / G) * (NP == kOnePartner ? PolySlot<G, MOVES, true>::bytes(a.N) : PolySlot<G, MOVES, false>::bytes(a.N));
 }
 
 constexpr size_t kPolySmemMax = 227u * 1024u;
@@ -797,12 +873,12 @@ static int poly_auto_warps(int p, int walkers_a_warp)
     return (each + blocks - 1) / blocks;
 }
 
-template <int G, int MOVES>
+template <int G, int MOVES, int NP>
 static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
 {
     // as many warps of the requested block as fit the shared memory of one block
     int wpb = block > 0 ? block / 32 : poly_auto_warps(a.p, 32 / G);
-    const size_t per_warp = poly_warp_smem<G>(a), hist = poly_hist_smem(a);
+    const size_t per_warp = poly_warp_smem<G, MOVES, NP>(a), hist = poly_hist_smem(a);
     if (hist + (size_t)wpb * per_warp > kPolySmemMax)
         wpb = hist < kPolySmemMax ? (int)((kPolySmemMax - hist) / per_warp) : 0;
     if (wpb < 1) return cudaErrorInvalidValue;
@@ -810,7 +886,7 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
     const int spb = wpb * (32 / G);
     const size_t smem = (size_t)wpb * per_warp + hist;
     const int nblk = (a.p + spb - 1) / spb;
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_polymer<G, MOVES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_sweep_polymer<G, MOVES, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // one launch per chunk of sweeps whose visits fit the block's 32-bit counters (spb N a sweep
     // at most), or fewer ("flush_every")
@@ -821,7 +897,7 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
         c.sweep_base = s0;
         c.sweeps = (a.sweeps - s0 < fe) ? a.sweeps - s0 : fe;
         c.trace_sweeps = a.sweeps;
-        k_sweep_polymer<G, MOVES><<<nblk, block, smem, s>>>(c);
+        k_sweep_polymer<G, MOVES, NP><<<nblk, block, smem, s>>>(c);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -857,12 +933,20 @@ cudaError_t launch_poly_sweep(const PolyArgs &a, int block, cudaStream_t s)
 {
     if (!polymer_supported(a.N)) return cudaErrorInvalidValue;
     switch (poly_lanes(a, a.lanes)) {
-    case 1: return a.moves ? launch_g<1, 1>(a, block, s) : launch_g<1, 0>(a, block, s);
-    case 2: return a.moves ? launch_g<2, 1>(a, block, s) : launch_g<2, 0>(a, block, s);
-    case 4: return a.moves ? launch_g<4, 1>(a, block, s) : launch_g<4, 0>(a, block, s);
-    case 8: return a.moves ? launch_g<8, 1>(a, block, s) : launch_g<8, 0>(a, block, s);
-    case 16: return a.moves ? launch_g<16, 1>(a, block, s) : launch_g<16, 0>(a, block, s);
-    default: return a.moves ? launch_g<32, 1>(a, block, s) : launch_g<32, 0>(a, block, s);
+    case 1: return a.moves ? launch_g<1, 1, 0>(a, block, s) : launch_g<1, 0, 0>(a, block, s);
+    case 2: return a.moves ? launch_g<2, 1, 0>(a, block, s) : launch_g<2, 0, 0>(a, block, s);
+    case 4: return a.moves ? launch_g<4, 1, 0>(a, block, s) : launch_g<4, 0, 0>(a, block, s);
+    case 8: return a.moves ? launch_g<8, 1, 0>(a, block, s) : launch_g<8, 0, 0>(a, block, s);
+    case 16:  // the default: unrolled by the partners of a lane
+        if (a.N <= 16) return a.moves ? launch_g<16, 1, 0>(a, block, s) : launch_g<16, 0, kOnePartner>(a, block, s);
+        if (a.moves) return launch_g<16, 1, 0>(a, block, s);
+        switch ((a.N + 31) / 32) {
+        case 1: return launch_g<16, 0, 1>(a, block, s);
+        case 2: return launch_g<16, 0, 2>(a, block, s);
+        case 3: return launch_g<16, 0, 3>(a, block, s);
+        default: return launch_g<16, 0, 4>(a, block, s);
+        }
+    default: return a.moves ? launch_g<32, 1, 0>(a, block, s) : launch_g<32, 0, 0>(a, block, s);
     }
 }
 
