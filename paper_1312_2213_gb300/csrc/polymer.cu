@@ -32,6 +32,8 @@
 // warp to finish adds to the 64-bit histogram (an iterate longer than they can
 // hold runs as several launches), so that walkers crowding one bin (right after
 // they walk in, say) do not queue on one global counter.
+#include <type_traits>
+
 #include "muca_device.cuh"
 #include "muca_internal.h"
 
@@ -92,30 +94,47 @@ __device__ __forceinline__ float q32_to_float(long long v)
     return (float)(int)(v >> 32) + (float)(uint32_t)v * 0x1p-32f;
 }
 
+// lnu < q32_to_float(v) for v < 0 and lnu in (-23, 0] or -inf, without conversion instructions (their
+// latency is on the attempt's chain): 16-bit integers become floats under an exponent of 2^23, and
+// 65536 h + l rounds once, as the conversion does.  Whole parts below -2^21 are all the same.
+__device__ __forceinline__ bool less_than_q32(float lnu, long long v)
+{
+    const uint32_t lo = (uint32_t)v;
+    const float h = __uint_as_float(0x4B000000u | (lo >> 16)) - 8388608.0f;
+    const float l = __uint_as_float(0x4B000000u | (lo & 0xFFFFu)) - 8388608.0f;
+    const float whole = __int_as_float(0x4B400000 + max((int)(v >> 32), -(1 << 21))) - 12582912.0f;
+    return lnu < fmaf(fmaf(h, 65536.0f, l), 0x1p-32f, whole);
+}
+
 __device__ __forceinline__ int poly_bin(long long E, const PolyArgs &a)
 {
     const long long b = ((E - a.elo_q) * a.bin_k) >> 32;
     return b < -1 ? -1 : (b > (long long)a.B ? a.B : (int)b);
 }
 
-// poly_bin of a relative energy r = E - elo_q, from its 32-bit halves: floor(r k 2^-32) is
-// (whole part) k + umulhi(fraction, k) for r >= 0, far above the window past 2^20.
+// poly_bin of a relative energy r = E - elo_q: the upper half of the 64-bit product r k, modulo 2^64
+// as poly_bin forms it (an overlapping initial chain can have an energy beyond that product), from
+// the 32-bit halves of r.
 __device__ __forceinline__ int poly_bin_rel(long long r, const PolyArgs &a)
 {
-    const int hi = (int)(r >> 32);
-    const uint32_t up = min((uint32_t)hi, 1u << 20) * (uint32_t)a.bin_k + __umulhi((uint32_t)r, (uint32_t)a.bin_k);
-    return hi < 0 ? -1 : (int)min(up, (uint32_t)a.B);
+    const int v = (int)((uint32_t)(r >> 32) * (uint32_t)a.bin_k + __umulhi((uint32_t)r, (uint32_t)a.bin_k));
+    return min(max(v, -1), a.B);
 }
 
-// llrint(v 2^32) for |v| < 2^31, through 32-bit conversions: the whole part and the fraction of |v|
-// are exact floats; only a fraction below 2^-8 has bits past 2^-32, rounded to nearest even as v is.
+// llrint(v 2^32) for |v| < 2^26.  Conversion instructions have twice the latency of additions, and
+// this is on the attempt's chain, so v is cut into integers by adding 1.5 2^23 (the integer then
+// sits in the low mantissa bits): v = 16 h + r, 2^12 r = m + x, q = 2^36 h + 2^20 m + rint(2^20 x),
+// every difference exact (a multiple of v's last place that is no longer than v).  Only the last
+// step rounds, to nearest even beside even terms, as the conversion of v would.
 __device__ __forceinline__ long long float_to_q32(float v)
 {
-    const float m = fabsf(v);
-    const uint32_t whole = (uint32_t)(int)m;
-    const uint32_t frac = __float2uint_rn((m - (float)(int)whole) * 0x1p32f);
-    const long long q = (long long)(((unsigned long long)whole << 32) | frac);
-    return v < 0.0f ? -q : q;
+    const float M = 12582912.0f;
+    const int MB = 0x4B400000;
+    const float th = fmaf(v, 0.0625f, M), r = fmaf(th - M, -16.0f, v);
+    const float tm = fmaf(r, 4096.0f, M), x = fmaf(r, 4096.0f, -(tm - M));
+    const float tl = fmaf(x, 1048576.0f, M);
+    const int h = __float_as_int(th) - MB, m = __float_as_int(tm) - MB, l = __float_as_int(tl) - MB;
+    return (long long)m * (1 << 20) + l + ((long long)(h * 16) << 32);
 }
 
 // n visits of a bin: a shared-memory reduction without a returned value, so nothing
@@ -349,8 +368,9 @@ __device__ __forceinline__ float bond_between(const Shadow &p, const Shadow &r, 
 // old and proposed place at once.  eb[j] is the energy of
 // the bond (j - 1, j), 0 at both ends.  The chunk of beads being visited (poly_chunk of them at a
 // time): minus the bead's old and proposed shadow, each number twice (twelve 2-vectors in six
-// 4-vectors, in the order of pos; ONE: old and proposed side by side, three), and rec = (energy of the left bond with the bead moved: left bead
-// where it was / left bead moved; energy of the right bond; ln of the acceptance word).
+// 4-vectors, in the order of pos; ONE: old and proposed side by side, three), and rec = (energy
+// change of the left bond, left bead where it was / left bead moved; of the right bond, right bead
+// where it is; ln of the acceptance word); a change is NaN where the bond breaks.
 template <int G>
 __host__ __device__ constexpr int poly_chunk() { return G > 16 ? G : 16; }
 
@@ -363,12 +383,13 @@ struct PolySlot {
     float4 *rec;     // [CH]
     long long *nx;   // [CH][3] (MOVES) proposed grid position, or the rotation's unit vector
     uint32_t *how;   // [CH] (MOVES) kReady, kLate, kNoPoint; else [CH][3] the random words of the step
+    float *nr;       // [CH] energy of the right bond with the bead moved
     float *eb;       // [N + 1]
     int nP;
     static __host__ __device__ int pairs(int N) { return ONE ? G : (N + 2 * G - 1) / (2 * G) * G; }
     static __host__ __device__ size_t bytes(int N)
     {
-        const size_t b = (size_t)48 * pairs(N) + (size_t)CH * (16 * BV + 16 + (MOVES ? 28 : 12)) + 4 * (size_t)(N + 1);
+        const size_t b = (size_t)48 * pairs(N) + (size_t)CH * (16 * BV + 16 + (MOVES ? 28 : 12) + 4) + 4 * (size_t)(N + 1);
         return (b + 15) / 16 * 16;
     }
     __device__ PolySlot(unsigned char *p, int N)
@@ -379,7 +400,8 @@ struct PolySlot {
         rec = bead + BV * CH;
         nx = (long long *)(rec + CH);
         how = (uint32_t *)(MOVES ? nx + 3 * CH : nx);
-        eb = (float *)(how + (MOVES ? CH : 3 * CH));
+        nr = (float *)(how + (MOVES ? CH : 3 * CH));
+        eb = nr + CH;
     }
     // component c (in the order x y | z lx | ly lz of pos) of bead j
     __device__ float *at(int j, int c) const
@@ -506,6 +528,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
     const int w = w0 + gi;
     const bool active = w < a.p;
     const bool counts = active && li == 0;  // the lane that counts its walker's visits
+    const bool visits = counts && a.record == 0;
     const int wr = active ? w : w0;  // a group past the last walker shadows the warp's first one, read-only
     const uint32_t wid = (uint32_t)(wr + a.walker_offset);
     long long *Xg = a.X + (size_t)wr * 3 * N;
@@ -605,23 +628,88 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 for (int t = li; t < CH; t += G) {
                     const int j = c0 + t;
                     if (j >= N) break;
-                    const Shadow p = S.get_proposed(t);
-                    if (j > 0) S.rec[t].x = bond_between(p, S.get(j - 1), a);
                     // (the bead before the chunk stands where pos has it)
-                    if (t > 0) S.rec[t].y = bond_between(p, S.get_proposed(t - 1), a);
-                    if (j + 1 < N) S.rec[t].z = bond_between(p, S.get(j + 1), a);
+                    const Shadow p = S.get_proposed(t);
+                    const float l0 = bond_between(p, S.get(max(j - 1, 0)), a);
+                    const float l1 = bond_between(p, S.get_proposed(max(t - 1, 0)), a);
+                    const float r = bond_between(p, S.get(min(j + 1, N - 1)), a);
+                    S.nr[t] = r;
+                    S.rec[t].x = j > 0 ? l0 - S.eb[j] : 0.0f;
+                    S.rec[t].y = l1;
+                    S.rec[t].z = j + 1 < N ? r - S.eb[j + 1] : 0.0f;
                 }
+                __syncwarp();
+#pragma unroll 1
+                for (int t = li; t < CH; t += G)
+                    if (t > 0 && c0 + t < N) S.rec[t].y -= S.nr[t - 1];  // (only used if bead t - 1 moved: not NaN)
                 __syncwarp();
             }
             // ---- the attempts, one after the other
             const int nt = min(CH, N - c0);
             uint32_t accs = 0u;   // accepted beads of the chunk (group-uniform)
             bool acc = false;     // the bead before was moved
-            float dn[2 * NV];     // pair terms of the next attempt
-            if (NP > 0) {
+            const int kc = min(li, 5);  // G >= 8: the shadow component this lane writes
+            // The unrolled loop, in two versions: for a warp with a walker that is not inside the window yet
+            // (some chains that start with beads on top of each other take long), and for one without
+            // (inside, none leaves the window again).
+            auto unrolled = [&](auto walk) {
+                constexpr bool WALK = decltype(walk)::value;
+                const long long span = a.ehi_q - a.elo_q;
+                long long dist = b < 0 ? -E : E - span;  // outside: distance to the window
+                float4 rec_n = S.rec[0];
+                float own_n = S.proposed(0, kc);
+                float dn[2 * NV];  // pair terms of the next attempt
 #pragma unroll
                 for (int m = 0; m < NV; ++m) lj_changes<Slot, ONE>(S, 0, G * m + li, a, dn[2 * m], dn[2 * m + 1]);
-            }
+#pragma unroll 1
+                for (int t = 0; t < nt; ++t) {
+                    const int i = c0 + t, tn = min(t + 1, CH - 1);  // (behind the chunk's end: not used)
+                    const float4 rec = rec_n;
+                    const float own = own_n;
+                    rec_n = S.rec[tn];
+                    own_n = S.proposed(tn, kc);
+                    // the sums as in the other loop below; a broken bond (NaN) or a lane sum that is too
+                    // large makes the walker's sum NaN, and the move is rejected
+                    float s = 0.0f + (li == 0 ? (acc ? rec.y : rec.x) : (li == 1 ? rec.z : 0.0f)), c = 0.0f;
+                    const unsigned u = (unsigned)(li - i + 1);
+#pragma unroll
+                    for (int m = 0; m < NV; ++m) {
+                        const int j = li + 2 * G * m;
+                        if (u + 2 * G * m > 2u && j < N) kahan_add(s, c, dn[2 * m]);
+                        if (!ONE && u + 2 * G * m + G > 2u && j + G < N) kahan_add(s, c, dn[2 * m + 1]);
+                    }
+#pragma unroll
+                    for (int m = 0; m < NV; ++m) lj_changes<Slot, ONE>(S, tn, G * m + li, a, dn[2 * m], dn[2 * m + 1]);
+                    float lane_sum = fabsf(s) < 4194304.0f ? s - c : __int_as_float(0x7fffffff);
+#pragma unroll
+                    for (int off = G / 2; off; off >>= 1) lane_sum += __shfl_xor_sync(0xffffffffu, lane_sum, off);
+                    const long long En = E + float_to_q32(lane_sum);
+                    const int bn = poly_bin_rel(En, a);
+                    const bool lands = (unsigned)bn < (unsigned)a.B && lane_sum == lane_sum;
+                    const long long lwn = __ldg(a.lnWq + (lands ? bn : 0));
+                    const long long dq = lwn - lw;
+                    acc = lands && (dq >= 0 || less_than_q32(rec.w, dq));
+                    const long long dnew = bn < 0 ? -En : (bn >= a.B ? En - span : 0);
+                    if (WALK) acc = inside ? acc : dnew <= dist && lane_sum == lane_sum;
+                    // (selects: a branch costs more latency than what it skips)
+                    if (acc && li < 6) S.set(i, kc, -own);
+                    E = acc ? En : E;
+                    b = acc ? bn : b;
+                    lw = acc ? lwn : lw;
+                    if (WALK) {
+                        inside = acc ? lands : inside;
+                        dist = acc ? dnew : dist;
+                    }
+                    accs |= acc ? 1u << t : 0u;
+                    __syncwarp();
+                    if (visits && (!WALK || inside)) count_visits(&hs[b], 1u);
+                }
+            };
+            if (NP > 0 && !a.trace) {
+                if (__any_sync(0xffffffffu, !inside)) unrolled(std::true_type{});
+                else unrolled(std::false_type{});
+            } else {
+            // (The loop for anything: rotations, any G, traces.)
 #pragma unroll 1
             for (int t = 0; t < nt; ++t) {
                 const int i = c0 + t;
@@ -667,41 +755,29 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
 #pragma unroll
                 for (int k = 0; k < (G == 1 ? 2 : 1); ++k) {
                     const bool left = (G == 1) ? k == 0 : li == 0;
-                    float vn = left ? (acc ? rec.y : rec.x) : rec.z;
-                    const float vo = S.eb[left ? i : i + 1];
+                    float d = left ? (acc ? rec.y : rec.x) : rec.z;
                     if (MOVES) {
-                        vn = 0.0f;
-                        if ((G == 1 || li < 2) && (left ? i > 0 : i + 1 < N))
-                            vn = bond_between(S.get_proposed(t), S.get(left ? i - 1 : i + 1), a);
+                        d = 0.0f;
+                        if ((G == 1 || li < 2) && (left ? i > 0 : i + 1 < N)) {
+                            vb[k] = bond_between(S.get_proposed(t), S.get(left ? i - 1 : i + 1), a);
+                            d = vb[k] - S.eb[left ? i : i + 1];
+                        }
                     }
                     if (G == 1 || li < 2) {
-                        broken = broken || vn != vn;
-                        vb[k] = vn;
-                        kahan_add(s, c, vn == vn ? vn - vo : 0.0f);
+                        broken = broken || d != d;
+                        kahan_add(s, c, d == d ? d : 0.0f);
                     }
                 }
                 // the other partners, in order, compensated (Kahan); li + 2 G m - i + 1 is 0, 1, 2 for
                 // the bonded beads and i itself
                 const unsigned u = (unsigned)(li - i + 1);
-                if (NP > 0) {
-#pragma unroll
-                    for (int m = 0; m < NV; ++m) {
-                        const int j = li + 2 * G * m;
-                        if (u + 2 * G * m > 2u && j < N) kahan_add(s, c, dn[2 * m]);
-                        if (!ONE && u + 2 * G * m + G > 2u && j + G < N) kahan_add(s, c, dn[2 * m + 1]);
-                    }
-                    const int tn = min(t + 1, CH - 1);  // (behind the chunk's end: not used)
-#pragma unroll
-                    for (int m = 0; m < NV; ++m) lj_changes<Slot, ONE>(S, tn, G * m + li, a, dn[2 * m], dn[2 * m + 1]);
-                } else {
 #pragma unroll 1
-                    for (int m = 0; li + 2 * G * m < N; ++m) {
+                for (int m = 0; li + 2 * G * m < N; ++m) {
                         float d0, d1;
                         lj_changes<Slot, ONE>(S, t, G * m + li, a, d0, d1);
                         if (u + 2 * G * m > 2u) kahan_add(s, c, d0);
-                        if (u + 2 * G * m + G > 2u && li + 2 * G * m + G < N) kahan_add(s, c, d1);
+                        if (!ONE && u + 2 * G * m + G > 2u && li + 2 * G * m + G < N) kahan_add(s, c, d1);
                     }
-                }
                 // |lane sum| >= 2^22 only for overlapping beads: such a move is rejected
                 const bool huge = !(fabsf(s) < 4194304.0f);
                 const bool refused = group_any<G>(huge || broken, gi) || no_point;
@@ -739,15 +815,14 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                         a.trace[((size_t)w * (size_t)a.trace_sweeps + (size_t)(a.sweep_base + sw)) * (size_t)N + i] = r;
                 }
                 if (acc) {
-                    for (int k = li; k < 6; k += G) {
-                        // shadow component k (x y z and their lo parts), as bead holds it, to pos
-                        S.set(i, k, -S.proposed(t, k));
-                    }
-                    if (G == 1) {
-                        if (i > 0) S.eb[i] = vb[0];
-                        if (i + 1 < N) S.eb[i + 1] = vb[1];
-                    } else if (li < 2) {
-                        S.eb[li == 0 ? i : i + 1] = vb[0];
+                    for (int k = li; k < 6; k += G) S.set(i, k, -S.proposed(t, k));
+                    if (MOVES) {
+                        if (G == 1) {
+                            if (i > 0) S.eb[i] = vb[0];
+                            if (i + 1 < N) S.eb[i + 1] = vb[1];
+                        } else if (li < 2) {
+                            S.eb[li == 0 ? i : i + 1] = vb[0];
+                        }
                     }
                     if (MOVES && counts) {
                         Xg[i] = S.nx[3 * t];
@@ -761,9 +836,12 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                     accs |= 1u << t;
                 }
                 __syncwarp();
-                if (a.record == 0 && counts && inside) count_visits(&hs[b], 1u);
+                if (visits && inside) count_visits(&hs[b], 1u);
+            }
             }
             nacc += (unsigned)__popc(accs);
+            // the bond into the next chunk (the others are rebuilt with the next sweep)
+            if (!MOVES && li == 0 && ((accs >> (nt - 1)) & 1u) && c0 + nt < N) S.eb[c0 + nt] = S.nr[nt - 1];
             // ---- the accepted moves on the master coordinates (32 x 32-bit products: the grid step fits an int)
             if (!MOVES && active) {
 #pragma unroll 1
