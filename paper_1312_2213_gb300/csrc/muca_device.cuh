@@ -65,6 +65,54 @@ __device__ __forceinline__ uint4 philox4x32_10_rk(uint4 c, const uint32_t (&rk)[
     return c;
 }
 
+// The lattice sweeps' blocks: counter (word group, sweep, walker, kTagSweep), the group the same for
+// every lane of a warp.  The first two rounds then need no multiplication a lane and block: the
+// products of the walker id (round 1) and of round 1's word 0, which knows walker and sweep only
+// (round 2), are made once a sweep (PhiloxLane), and those of the group and of round 1's word 2 are
+// the same for the whole warp (uniform instructions).  Eight of ten rounds are left, and a block's
+// wide multiplications, 4 cycles each of a scheduler's multiply pipe, set the producers' pace.
+struct PhiloxLane {
+    uint32_t lo1, hi0, lo0;  // round 1: lo(M1 walker); round 2: hi and lo of M0 word 0
+};
+
+__device__ __forceinline__ PhiloxLane philox_lane(uint32_t sweep, uint32_t walker, const uint32_t (&rk)[20])
+{
+    const uint32_t w0 = __umulhi(kPhiloxM1, walker) ^ sweep ^ rk[0];
+    return PhiloxLane{kPhiloxM1 * walker, __umulhi(kPhiloxM0, w0), kPhiloxM0 * w0};
+}
+
+// W blocks (groups group, group + 1, ...) round by round together: a round is a chain of about 19
+// cycles (wide multiplication, xor) for 2 x 5.5 cycles of the scheduler's pipes, and a producer has
+// its scheduler with one other warp, so one block after the other left the pipes idle two thirds of
+// the time.
+template <int W>
+__device__ __forceinline__ void philox4x32_10_groups(uint32_t group, const PhiloxLane &l, const uint32_t (&rk)[20],
+                                                     uint4 (&c)[W])
+{
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const uint32_t w2 = __umulhi(kPhiloxM0, group + i) ^ kTagSweep ^ rk[1];
+        c[i] = make_uint4((__umulhi(kPhiloxM1, w2) ^ rk[2]) ^ l.lo1, kPhiloxM1 * w2,
+                          ((kPhiloxM0 * (group + i)) ^ rk[3]) ^ l.hi0, l.lo0);
+    }
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const uint32_t hi0 = __umulhi(kPhiloxM0, c[i].x), lo0 = kPhiloxM0 * c[i].x;
+            const uint32_t hi1 = __umulhi(kPhiloxM1, c[i].z), lo1 = kPhiloxM1 * c[i].z;
+            c[i] = make_uint4(hi1 ^ c[i].y ^ rk[2 * r], lo1, hi0 ^ c[i].w ^ rk[2 * r + 1], lo0);
+        }
+    }
+}
+
+__device__ __forceinline__ uint4 philox4x32_10_group(uint32_t group, const PhiloxLane &l, const uint32_t (&rk)[20])
+{
+    uint4 c[1];
+    philox4x32_10_groups<1>(group, l, rk, c);
+    return c[0];
+}
+
 // ---------------------------------------------------------------------------
 // Deterministic binary64 exp and log.
 // exp: Cody-Waite reduction x = k ln2 + r (ln 2 = HI + LO, HI with 32

@@ -9,35 +9,47 @@ namespace muca {
 
 // ---------------------------------------------------------------------------
 // Producer/consumer form with precomputed site codes (Ising and MUMA).
-// Shared memory holds the same threshold + histogram rows as above.  The
-// producer warp writes, per row, the walkers' random
+// Shared memory holds the thresholds and the histogram counters (column-major, see
+// below).  The producer warps write, per row, the walkers' random
 // words (clamped, see clamp_words), their old row and, for every site, two column
-// bytes holding 4 c (byte offsets into a threshold row): c0 for "left
+// bytes holding 4 c: c0 for "left
 // neighbour as it was" and c1 for "left neighbour flipped", both without the up
 // neighbour (which only the consumer knows: the row above is final only after
 // the consumer has swept it) and, for the last site, without its right
 // neighbour (site 0 of the same row).  Four sites are handled at once with
-// bytewise arithmetic.  The consumer subtracts the up term (and the right term of
-// the last site), derives the bin moves from the two columns and runs the same
-// speculative chain as above.  (A variant that stored (threshold, next-row) pairs
-// to save the moves was slower: its 8-byte random loads doubled the bank
-// conflicts on the critical chain.)
-__device__ __forceinline__ uint32_t nib_to_bytes(uint32_t n)  // 4 bits -> 4 bytes of 0/1
-{
-    return (n * 0x00204081u) & 0x01010101u;
-}
-
-template <int L, int WR>
-__device__ __forceinline__ uint32_t row_nibble(const uint32_t (&r)[WR], int x)  // bits x..x+3 (x % 4 == 0)
-{
-    return (r[x >> 5] >> (x & 31)) & 15u;
-}
-
+// bytewise arithmetic on the row's anti-aligned bits.  The consumer subtracts the up term
+// (and the right term of the last site), makes addresses and bin moves from the bytes
+// with byte dot products, and runs a speculative chain: both candidate thresholds of a
+// site are loaded while the site before it is decided.  (A variant that stored
+// (threshold, next-row) pairs to save the moves was slower: its 8-byte random loads
+// doubled the bank conflicts on the critical chain.)
+// Bound by that chain: 39 cycles a site, of which two shared-memory loads and their
+// selects and compares; the producers alone need 36 (L = 32).  Cycles a site, 8192
+// walkers spread over all bins, before / after the column-major table, the joined
+// rows and the shorter Philox rounds: Ising L = 32 50.7 / 42.6, MUMA 50.3 / 43.5;
+// Ising L = 64 (2048 walkers) 50.9 / 48.0, L = 16 59.4 / 48.6, L = 8 (64) 74.5 / 60.0.
 template <int L, int WR>
 __device__ __forceinline__ uint32_t row_bit(const uint32_t (&r)[WR], int x)
 {
     return (r[x >> 5] >> (x & 31)) & 1u;
 }
+
+// Sites x..x+3 (x % 4 == 0) of a packed row as bytes 4 [bit].
+template <int WR>
+__device__ __forceinline__ uint32_t nibble_fours(const uint32_t (&r)[WR], int x)
+{
+    return (((r[x >> 5] >> (x & 31)) & 15u) * (0x00204081u << 2)) & 0x04040404u;
+}
+
+// Code-form table of Ising and MUMA: column-major, T[c][b] at word c NB + b, the counters of the bins
+// behind the C columns.  A code byte is then worth NB bytes a unit of 4 c, and one dp2a makes a
+// threshold's address from the packed codes of four sites and the walker's bin address (NB in the
+// 16-bit half that meets the site's byte), where rows of C + 1 words a bin took an extraction and an
+// addition, and a multiplication for the bin's move.
+// Ising codes travel as 4 c + 0x78; the consumer flips the top bits behind the up neighbour's term,
+// which leaves the signed byte 4 (c - 2): the bin's move in bytes, added by one dp4a.
+template <int SYS>
+constexpr uint32_t kCodeBias = SYS == kIsing ? 0x78787878u : 0u;
 
 // The random words handed to a code-form consumer are min(u, 2^32 - 2).  With
 // that clamp the acceptance "T == always or u < T" becomes the single compare
@@ -94,198 +106,255 @@ __device__ __forceinline__ CodeRole code_role(int warp, int ncw)
 }
 constexpr int kCodeWarpsPerWalkerWarp = 4;
 
+// Lanes of a consumer warp that run the protocol (and arrive on EMPTY) when `left` walkers are left
+// for it: those with a walker, or all of a warp that has none.  (Lanes without a walker beside others
+// with one took a loop of their own, which the warp then ran after the walkers': 10 % at p = 1000.)
+__device__ __forceinline__ unsigned code_consumer_lanes(int left) { return left > 0 && left < 32 ? (unsigned)left : 32u; }
+
+// The producer's rows of nsw sweeps.
 template <int SYS, int L, int PART>
-__device__ __forceinline__ void produce_sweep_tn(uint32_t g, uint32_t wid, const uint32_t (&rk)[20],
-                                                 const uint32_t *__restrict__ lat, int ps, uint4 *ring_u,
-                                                 uint2 *ring_c, uint32_t *ring_r, unsigned long long *full,
-                                                 unsigned long long *empty, int &k, bool &bad, int drop_k)
+__device__ __forceinline__ void produce_tn(int64_t nsw, uint32_t g0, uint32_t wid, const uint32_t (&rk)[20],
+                                           const uint32_t *__restrict__ lat, int ps, uint4 *ring_u, uint2 *ring_c,
+                                           uint32_t *ring_r, unsigned long long *full, unsigned long long *empty, int &k,
+                                           bool &bad, int drop_k)
 {
     constexpr int WR = ising_words_per_row(L);
     constexpr int G = L / 4;
     constexpr size_t SU = (size_t)G * 32, SC = (size_t)G * 32, SR = (size_t)WR * 32;
     // Rolling rows: o = row y (old), d = row y+1 (old; row 0 final for y = L-1), nn = row y+2
-    // prefetched one row ahead.  The producer runs at most kRing rows ahead of the
-    // consumer and L >= 2 kRing, so every row it reads has its value for this sweep
-    // (rows y, y+1, y+2 not yet swept; row 0 already swept when it is the last row's
-    // down neighbour).  The first two rows of a sweep are read after the first wait.
+    // prefetched one row ahead, on into the next sweep.  The producer runs at most kRing rows ahead of
+    // the consumer and L >= 2 kRing, so every row it reads has its value for its sweep (rows y, y+1, y+2
+    // not yet swept; rows 0 and 1 already swept when they are read behind rows L-2 and L-1).  At the
+    // first sweep nothing is in flight.
     uint32_t o[WR], d[WR], nn[WR];
-#pragma unroll 1
-    for (int y = 0; y < L; ++y) {
-        const int slot = k % kRing;
-        if (!bad && !mbar_wait(&empty[slot], (unsigned)(((k / kRing) & 1) ^ 1))) bad = true;
-        if (y == 0) {
 #pragma unroll
-            for (int j = 0; j < WR; ++j) {
-                o[j] = lat[j * ps];
-                d[j] = lat[(WR + j) * ps];
+    for (int j = 0; j < WR; ++j) {
+        o[j] = lat[j * ps];
+        d[j] = lat[(WR + j) * ps];
+    }
+#pragma unroll 1
+    for (int64_t sw = 0; sw < nsw; ++sw) {
+        const PhiloxLane pl = philox_lane(g0 + (uint32_t)sw, wid, rk);
+#pragma unroll 1
+        for (int y = 0; y < L; ++y) {
+            const int slot = k % kRing;
+            // the row's random words are made while the answer about the slot is under way
+            constexpr int g_lo = PART * G / kCodeProducers, g_hi = (PART + 1) * G / kCodeProducers, NG = g_hi - g_lo;
+            bool free_slot = mbar_try(&empty[slot], (unsigned)(((k / kRing) & 1) ^ 1));
+            uint4 words[NG];
+            constexpr int PB = NG < 4 ? NG : 4;
+#pragma unroll
+            for (int i = 0; i + PB <= NG; i += PB) {
+                uint4 c[PB];
+                philox4x32_10_groups<PB>((uint32_t)(y * G + g_lo + i), pl, rk, c);
+#pragma unroll
+                for (int e = 0; e < PB; ++e) words[i + e] = clamp_words(c[e]);
             }
-        }
-        const int y2 = (y + 2 < L) ? y + 2 : y + 2 - L;
-        if (y + 1 < L) {
+            for (int i = NG / PB * PB; i < NG; ++i) words[i] = clamp_words(philox4x32_10_group((uint32_t)(y * G + g_lo + i), pl, rk));
+            if (!free_slot && !bad && !mbar_wait(&empty[slot], (unsigned)(((k / kRing) & 1) ^ 1))) bad = true;
+            const int y2 = (y + 2 < L) ? y + 2 : y + 2 - L;
 #pragma unroll
             for (int j = 0; j < WR; ++j) nn[j] = lat[(y2 * WR + j) * ps];
-        }
-        uint4 *wu = ring_u + slot * SU;
-        uint2 *wc = ring_c + slot * SC;
-        uint32_t *wr = ring_r + slot * SR;
-        if (PART == 0) {
+            uint4 *wu = ring_u + slot * SU;
+            uint2 *wc = ring_c + slot * SC;
+            uint32_t *wr = ring_r + slot * SR;
+            if (PART == 0) {
 #pragma unroll
-            for (int j = 0; j < WR; ++j) wr[j * 32] = o[j];
-        }
-        constexpr int g_lo = PART * G / kCodeProducers, g_hi = (PART + 1) * G / kCodeProducers;
-#pragma unroll
-        for (int gq = g_lo; gq < g_hi; ++gq) {
-            wu[gq * 32] = clamp_words(philox4x32_10_rk(make_uint4((uint32_t)(y * G + gq), g, wid, kTagSweep), rk));
-            const int x = 4 * gq;
-            const uint32_t s4 = row_nibble<L, WR>(o, x);
-            // left neighbours x-1..x+2 and right neighbours x+1..x+4 (periodic in x)
-            uint32_t l4 = (s4 << 1) & 15u, r4 = s4 >> 1;
-            l4 |= row_bit<L, WR>(o, (x + L - 1) % L);
-            if (x + 4 < L) r4 |= row_bit<L, WR>(o, x + 4) << 3;
-            else r4 |= ((s4 >> 3) & 1u) << 3;  // last site: right neighbour left out (anti = 0)
-            const uint32_t S = nib_to_bytes(s4);
-            const uint32_t A = nib_to_bytes(l4) ^ S;  // left anti-aligned
-            const uint32_t Bq = nib_to_bytes(r4) ^ S;
-            const uint32_t D = nib_to_bytes(row_nibble<L, WR>(d, x)) ^ S;
-            // columns as byte offsets (4 c) into a threshold row, per byte
-            const uint32_t k0 = (0x04040404u - (A + Bq + D)) << 2;  // 4 - anti-aligned (without up)
-            const uint32_t k1 = k0 + 8u * A - 0x04040404u;          // left neighbour flipped
-            if (SYS == kMuma) {
-                const uint32_t s5 = S * 20u;
-                wc[gq * 32] = make_uint2(s5 + k0, s5 + k1);
-            } else {
-                wc[gq * 32] = make_uint2(k0, k1);
+                for (int j = 0; j < WR; ++j) wr[j * 32] = o[j];
             }
-        }
-        if (k != drop_k) mbar_arrive(&full[slot]);
-        ++k;
+            // anti-aligned neighbours of the whole row at once: left, right (none for the last site: the
+            // consumer adds it) and down
+            uint32_t la[WR], ra[WR], da[WR];
 #pragma unroll
-        for (int j = 0; j < WR; ++j) {
-            o[j] = d[j];
-            d[j] = nn[j];
+            for (int j = 0; j < WR; ++j) {
+                constexpr int last = (L - 1) & 31;  // bit of the row's last site in its word
+                const uint32_t from_left = (j > 0) ? o[j - 1] >> 31 : (o[WR - 1] >> last) & 1u;
+                const uint32_t from_right = (j + 1 < WR) ? o[(j + 1) % WR] << 31 : o[j] & (1u << last);
+                la[j] = o[j] ^ ((o[j] << 1) | from_left);
+                ra[j] = o[j] ^ ((o[j] >> 1) | from_right);
+                da[j] = o[j] ^ d[j];
+            }
+#pragma unroll
+            for (int gq = g_lo; gq < g_hi; ++gq) {
+                wu[gq * 32] = words[gq - g_lo];
+                // per byte 4 [anti-aligned], and from them the columns as byte offsets 4 c: 4 (4 - count)
+                // without the up neighbour, for the left neighbour as it was (k0) and flipped (k1)
+                const int x = 4 * gq;
+                const uint32_t A = nibble_fours<WR>(la, x), BD = nibble_fours<WR>(ra, x) + nibble_fours<WR>(da, x);
+                uint32_t k0 = 0x10101010u - A - BD, k1 = 0x0C0C0C0Cu + A - BD;
+                // the row's first site does not see the site decided before it: one code for both outcomes
+                if (gq == 0) k1 = __byte_perm(k0, k1, 0x7650u);
+                if (SYS == kMuma) {
+                    const uint32_t s5 = nibble_fours<WR>(o, x) * 5u;
+                    k0 += s5;
+                    k1 += s5;
+                }
+                wc[gq * 32] = make_uint2(k0 + kCodeBias<SYS>, k1 + kCodeBias<SYS>);
+            }
+            if (k != drop_k) mbar_arrive(&full[slot]);
+            ++k;
+#pragma unroll
+            for (int j = 0; j < WR; ++j) {
+                o[j] = d[j];
+                d[j] = nn[j];
+            }
         }
     }
 }
 
+// The consumer's rows of nsw sweeps, one after the other without a break: the next row's hand-over,
+// its first codes and both candidates of its first threshold are taken up while the last four sites of
+// a row are decided (with a fresh start at every row a row cost 270 cycles beside 39 a site).
 template <int SYS, int L, int RECORD>
-__device__ __forceinline__ void ising_sweep_tc(uint32_t *__restrict__ lat, int ps, int &bR, uint32_t *__restrict__ sTH,
-                                               const uint4 *__restrict__ ring_u, const uint2 *__restrict__ ring_c,
-                                               const uint32_t *__restrict__ ring_r, unsigned long long *full,
-                                               unsigned long long *empty, int &k, bool &bad, unsigned long long *obs,
-                                               unsigned &nacc)
+__device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ lat, int ps, int &bR,
+                                           uint32_t *__restrict__ sTH, const uint4 *__restrict__ ring_u,
+                                           const uint2 *__restrict__ ring_c, const uint32_t *__restrict__ ring_r,
+                                           unsigned long long *full, unsigned long long *empty, int &k, bool &bad,
+                                           unsigned long long *obs, unsigned long long &nacc, int r_lo, int r_hi,
+                                           int &tst, unsigned &ev)
 {
-    int pc = 0;  // -1 spins of the final rows (observables)
     constexpr int WR = ising_words_per_row(L);
     constexpr int C = (SYS == kMuma) ? 10 : 5;
-    constexpr int RS = C + 1;
+    constexpr int NB = L * L + 1;
     constexpr int G = L / 4;
     constexpr size_t SU = (size_t)G * 32, SC = (size_t)G * 32, SR = (size_t)WR * 32;
-    // The chain works in 32-bit shared-window byte addresses: bB = table base + 4 RS bin and the
-    // producer's columns are 4 c, so a threshold address is one add and the bin's histogram
-    // counter an immediate offset from the (already updated) bin address.
+    // The chain works in 32-bit shared-window byte addresses: bB = table base + 4 bin.
     const int sbase = (int)__cvta_generic_to_shared(sTH);
+    constexpr int TOFF = (SYS == kMuma) ? 0 : 8 * NB;  // Ising: codes count from column 2
     auto th = [sbase](int addr) -> uint32_t {
         uint32_t v;
-        asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(checked_addr(addr, sbase)));
+        asm("ld.shared.u32 %0, [%1 + %2];" : "=r"(v) : "r"(checked_addr(addr + TOFF, sbase) - TOFF), "n"(TOFF));
         return v;
     };
-    // bin-row move of an accepted flip in bytes: Ising (c - 2) rows from the column,
-    // MUMA one row up for s = +1 and one down for s = -1 (the old spin of the site)
-    auto move = [](uint32_t cb) -> int { return ((int)cb - 8) * RS; };
-    int bB = sbase + bR * 4;
-    uint32_t up[WR], cur[WR], old[WR];
-#pragma unroll
-    for (int j = 0; j < WR; ++j) up[j] = lat[((L - 1) * WR + j) * ps];
-    // two rows an iteration from L = 32 up (2-4 % there; L = 16 rows are short enough that the
-    // larger body costs more than the loop overhead it saves)
-    constexpr int kRowUnroll = (L >= 32) ? 2 : 1;
-#pragma unroll kRowUnroll
-    for (int y = 0; y < L; ++y) {
+    // bB + NB x byte i of w (signed for Ising)
+    auto at = [](uint32_t w, int i, int b) -> int {
+        const int n = NB << (16 * (i & 1));
+        if (SYS == kMuma) return (int)(i < 2 ? __dp2a_lo((unsigned)n, w, (unsigned)b) : __dp2a_hi((unsigned)n, w, (unsigned)b));
+        return i < 2 ? __dp2a_lo(n, (int)w, b) : __dp2a_hi(n, (int)w, b);
+    };
+    // codes of four sites with the up neighbour's term (bytes 4 [anti-aligned])
+    auto settle = [](uint2 c, uint32_t up4) -> uint2 {
+        constexpr uint32_t flip = (SYS == kMuma) ? 0u : 0x80808080u;
+        return make_uint2((c.x - up4) ^ flip, (c.y - up4) ^ flip);
+    };
+
+    const int k_end = k + (int)(nsw * L);
+    int bB = sbase + 4 * bR;
+    uint32_t up[WR], cur[WR], nxt[WR];
+    uint2 cdn = make_uint2(0u, 0u);
+    uint32_t T0 = 0u, T1 = 0u;
+    bool accP = false;  // the site decided before
+    if (!bad && !mbar_wait(&full[k % kRing], (unsigned)((k / kRing) & 1))) bad = true;
+    if (!bad) {
         const int slot = k % kRing;
-        if (!bad && !mbar_wait(&full[slot], (unsigned)((k / kRing) & 1))) bad = true;
-        if (bad) {  // a wait gave up: the ring is out of step, so nothing more is computed
-            mbar_arrive(&empty[slot]);
-            ++k;
-            continue;
-        }
-        const uint4 *ru = ring_u + slot * SU;
-        const uint2 *rc = ring_c + slot * SC;
-        const uint32_t *rr = ring_r + slot * SR;
-        uint32_t ua[WR];
 #pragma unroll
         for (int j = 0; j < WR; ++j) {
-            cur[j] = rr[j * 32];
-            old[j] = cur[j];
-            ua[j] = up[j] ^ cur[j];  // up neighbour anti-aligned
+            up[j] = lat[((L - 1) * WR + j) * ps];
+            nxt[j] = ring_r[slot * SR + j * 32];
         }
-        const uint32_t sLast = row_bit<L, WR>(cur, L - 1);
-        uint2 cd = rc[0];
-        {
-            const uint32_t u4 = nib_to_bytes(row_nibble<L, WR>(ua, 0)) << 2;
-            cd.x -= u4;
-            cd.y -= u4;
-        }
-        uint2 cdn = cd;
-        const uint32_t c00 = cd.x & 0xffu;
-        uint32_t T0 = th(bB + (int)c00), T1 = 0u;
-        int d0 = move(c00), d1 = 0;
-        bool accP = false;
-        uint4 u = make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t ua0[1] = {up[0] ^ nxt[0]};
+        cdn = settle(ring_c[slot * SC], nibble_fours<1>(ua0, 0));
+        T0 = T1 = th(at(cdn.x, 0, bB));
+    }
+#pragma unroll 1
+    for (int64_t sw = 0; sw < nsw && !bad; ++sw) {
+        unsigned na = 0;
+        // two rows an iteration from L = 32 up (2-4 % there; L = 16 rows are short enough that the
+        // larger body costs more than the loop overhead it saves)
+        constexpr int kRowUnroll = (L >= 32) ? 2 : 1;
+#pragma unroll kRowUnroll
+        for (int y = 0; y < L; ++y) {
+            const int slot = k % kRing, slot_n = (k + 1) % kRing;
+            const uint4 *ru = ring_u + slot * SU;
+            const uint2 *rc = ring_c + slot * SC;
+            uint32_t ua[WR], old[WR];
 #pragma unroll
-        for (int x = 0; x < L; ++x) {
-            const int j4 = x & 3;
-            if (j4 == 0) {
-                u = ru[(x / 4) * 32];
-                cd = cdn;
-                if (x + 4 < L) {
-                    cdn = rc[(x / 4 + 1) * 32];
-                    const uint32_t u4 = nib_to_bytes(row_nibble<L, WR>(ua, x + 4)) << 2;
-                    cdn.x -= u4;
-                    cdn.y -= u4;
-                }
+            for (int j = 0; j < WR; ++j) {
+                old[j] = cur[j] = nxt[j];
+                ua[j] = up[j] ^ cur[j];  // up neighbour anti-aligned
             }
-            const uint32_t uw = word_of(u, j4);
-            const int dR = (SYS == kMuma) ? (row_bit<L, WR>(old, x) ? 4 * RS : -4 * RS) : (accP ? d1 : d0);
-            const uint32_t T = accP ? T1 : T0;
-            if (x + 1 < L) {
+            const uint32_t sLast = row_bit<L, WR>(cur, L - 1);
+            uint2 cd = cdn, cnext = cdn;
+            uint4 u = make_uint4(0u, 0u, 0u, 0u);
+            uint32_t mv = 0u;   // MUMA: the four sites' moves in bytes, +-4
+            bool next = false;  // the next row is there
+#pragma unroll
+            for (int x = 0; x < L; ++x) {
+                const int j4 = x & 3;
+                if (j4 == 0) {
+                    u = ru[(x / 4) * 32];
+                    cd = cdn;
+                    // s = -1 (bit set): one bin up, else one down; 0xFC = -4, 0xFC ^ 0xF8 = 4
+                    if (SYS == kMuma) mv = (nibble_fours<WR>(old, x) * 0x3Eu) ^ 0xFCFCFCFCu;
+                    if (x + 4 < L) cdn = settle(rc[(x / 4 + 1) * 32], nibble_fours<WR>(ua, x + 4));
+                    if (x + 8 == L) next = mbar_try(&full[slot_n], (unsigned)(((k + 1) / kRing) & 1));
+                    if (x + 4 == L) {
+                        // the next row; behind the last one (or a wait that gave up) an earlier row's codes
+                        // are read and not used
+                        if (!next && !(sw + 1 == nsw && y == L - 1))
+                            bad = !mbar_wait(&full[slot_n], (unsigned)(((k + 1) / kRing) & 1));
+#pragma unroll
+                        for (int j = 0; j < WR; ++j) nxt[j] = ring_r[slot_n * SR + j * 32];
+                        cnext = ring_c[slot_n * SC];
+                    }
+                }
+                if (x == L - 2) {
+                    // the last site's right neighbour is site 0 of this row, final by now (its code is the
+                    // top byte, so nothing is borrowed from)
+                    const uint32_t ra = (row_bit<L, WR>(cur, 0) ^ sLast) << 26;
+                    cd.x -= ra;
+                    cd.y -= ra;
+                }
+                if (x == L - 1) {
+                    const uint32_t ua0[1] = {cur[0] ^ nxt[0]};  // (sites 0..3 are final)
+                    cdn = settle(cnext, nibble_fours<1>(ua0, 0));
+                }
+                const uint32_t uw = word_of(u, j4);
+                // the bin's address if this site is accepted
+                const int bA = (SYS == kMuma) ? __dp4a((int)mv, 1 << (8 * j4), bB)
+                                              : __dp4a((int)(accP ? cd.y : cd.x), 1 << (8 * j4), bB);
+                const uint32_t T = accP ? T1 : T0;
+                // both candidates of the next site's threshold (behind the last site: of the next row's
+                // first, whose two codes are the same)
                 const int jn = (x + 1) & 3;
-                const uint32_t wx = (jn == 0) ? cdn.x : cd.x, wy = (jn == 0) ? cdn.y : cd.y;
-                // byte jn of the packed codes (selector bytes 4 pick zeros)
-                uint32_t c0 = __byte_perm(wx, 0u, 0x4440u | (uint32_t)jn);
-                uint32_t c1 = __byte_perm(wy, 0u, 0x4440u | (uint32_t)jn);
-                if (x + 1 == L - 1) {
-                    // the last site's right neighbour is site 0 of this row, final by now
-                    const uint32_t ra = (row_bit<L, WR>(cur, 0) ^ sLast) << 2;
-                    c0 -= ra;
-                    c1 -= ra;
-                }
-                T0 = th(bB + (int)c0);
-                T1 = th(bB + dR + (int)c1);
-                if (SYS != kMuma) {
-                    d0 = move(c0);
-                    d1 = move(c1);
-                }
+                T0 = th(at((jn == 0) ? cdn.x : cd.x, jn, bB));
+                T1 = th(at((jn == 0) ? cdn.y : cd.y, jn, bA));
+                const bool acc = uw < T;  // the producer's clamp makes this "always or u < T"
+                if (acc) cur[x >> 5] ^= 1u << (x & 31);
+                bB = acc ? bA : bB;
+                if (RECORD == 0)
+                    asm volatile("red.shared.add.u32 [%0 + %2], %1;" ::"r"(checked_addr(bB + 4 * C * NB, sbase) - 4 * C * NB),
+                                 "r"(1u), "n"(4 * C * NB)
+                                 : "memory");
+                accP = acc;
             }
-            const bool acc = uw < T;  // the producer's clamp makes this "always or u < T"
-            if (acc) cur[x >> 5] ^= 1u << (x & 31);
-            bB = acc ? bB + dR : bB;
-            if (RECORD == 0)
-                asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(checked_addr(bB + 4 * C, sbase)), "r"(1u) : "memory");
-            accP = acc;
-        }
 #pragma unroll
-        for (int j = 0; j < WR; ++j) {
-            lat[(y * WR + j) * ps] = cur[j];
-            pc += __popc(cur[j]);
-            nacc += __popc(old[j] ^ cur[j]);
-            up[j] = cur[j];
+            for (int j = 0; j < WR; ++j) {
+                lat[(y * WR + j) * ps] = cur[j];
+                na += (unsigned)__popc(old[j] ^ cur[j]);
+                up[j] = cur[j];
+            }
+            mbar_arrive(&empty[slot]);  // after the row is stored: the producer reads it later
+            ++k;
+            if (bad) break;
         }
-        mbar_arrive(&empty[slot]);  // after the row is stored: the producer reads it later
+        nacc += na;
+        if (bad) break;
+        const int bin = (bB - sbase) / 4;
+        if (RECORD == 1) atomicAdd(&sTH[checked_word(bin + C * NB)], 1u);
+        if (SYS == kIsing && obs) {
+            int pc = 0;  // -1 spins of the final rows
+#pragma unroll 1
+            for (int j = 0; j < L * WR; ++j) pc += __popc(lat[j * ps]);
+            record_observables(obs, bin, L * L, pc);
+        }
+        tunnel_step(bin, r_lo, r_hi, tst, ev);
+    }
+    while (k != k_end) {  // a wait gave up: the ring is out of step, so nothing more is computed
+        mbar_arrive(&empty[k % kRing]);
         ++k;
     }
     bR = (bB - sbase) / 4;
-    if (RECORD == 1) atomicAdd(&sTH[checked_word(bR + C)], 1u);
-    if (SYS == kIsing && obs && !bad) record_observables(obs, bR / RS, L * L, pc);
 }
 
 __host__ __device__ constexpr size_t tn_ring_bytes(int L)
@@ -297,7 +366,7 @@ template <int SYS, int L>
 __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, int slot_id, uint32_t *smem)
 {
     constexpr int C = num_cols(SYS);
-    constexpr int RS = C + 1;
+    constexpr int NB = L * L + 1;
     constexpr int G = L / 4;
     constexpr int NP = kCodeProducers;
     const int ncw = blockDim.x / (32 * kCodeWarpsPerWalkerWarp);
@@ -307,7 +376,7 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
     const int pair = role.pair, part = role.part;
     const int drop_k = (blockIdx.x == 0 && producer && pair == 0 && part == 0) ? a.debug_drop_row : -1;
     uint32_t *sTH = smem;
-    const size_t th_bytes = ((size_t)a.B * RS * 4 + 15) / 16 * 16;
+    const size_t th_bytes = ((size_t)NB * (C + 1) * 4 + 15) / 16 * 16;
     char *rbase = (char *)smem + th_bytes + (size_t)pair * tn_ring_bytes(L);
     uint4 *ring_u = (uint4 *)rbase + lane;
     uint2 *ring_c = (uint2 *)(rbase + (size_t)kRing * G * 32 * 16) + lane;
@@ -316,74 +385,76 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
     unsigned long long *full = bars + (size_t)pair * 2 * kRing, *empty = full + kRing;
 
     const int tid = threadIdx.x;
-    for (int i = tid; i < a.B * RS; i += blockDim.x) {
-        const int b = i / RS, c = i - (i / RS) * RS;
-        sTH[i] = (c < C) ? a.T[b * C + c] : 0u;
+    for (int i = tid; i < NB * C; i += blockDim.x) {
+        const int b = i / C, c = i - (i / C) * C;
+        sTH[c * NB + b] = a.T[i];
+    }
+    for (int b = tid; b < NB; b += blockDim.x) sTH[C * NB + b] = 0u;
+    // the rings' codes start on a middle column, so that codes read ahead of a row that never came
+    // (a wait that gave up, the end of the last sweep) still address the table
+    for (int i = tid; i < ncw * kRing * G * 32; i += blockDim.x) {
+        const int pr = i / (kRing * G * 32);
+        ((uint2 *)((char *)smem + th_bytes + (size_t)pr * tn_ring_bytes(L) + (size_t)kRing * G * 32 * 16))[i - pr * kRing * G * 32] =
+            make_uint2(0x08080808u + kCodeBias<SYS>, 0x08080808u + kCodeBias<SYS>);
     }
     if (tid == 0)  // per pair: FULL[kRing] (NP producer warps arrive), EMPTY[kRing] (the consumer)
-        for (int i = 0; i < ncw * 2 * kRing; ++i) mbar_init(bars + i, ((i / kRing) % 2 == 0) ? 32 * NP : 32);
+        for (int i = 0; i < ncw * 2 * kRing; ++i)
+            mbar_init(bars + i, ((i / kRing) % 2 == 0) ? 32 * NP : code_consumer_lanes(a.p - w0 - 32 * (i / (2 * kRing))));
     set_block_spin_limit(a.spin_limit);
-    checks_begin(a.B * RS, a.debug_check);
+    checks_begin(NB * (C + 1), a.debug_check);
     __syncthreads();
 
     const int w = w0 + pair * 32 + lane;
     const bool active = w < a.p;
+    const bool some = w - lane < a.p;  // this warp has walkers
     const uint32_t wid = (uint32_t)(w + a.walker_offset);
     const uint32_t g0 = (uint32_t)a.state->sweep_counter;
     uint32_t *lat = a.lattice + (active ? w : 0);
-    int bR = (active ? a.bin[w] : 0) * RS;
-    unsigned long long *Hb = a.Hpart + (size_t)slot_id * a.B;
+    int bR = active ? a.bin[w] : 0;
+    unsigned long long *Hb = a.Hpart + (size_t)slot_id * NB;
     int k = 0;
     bool bad = false;
-    const int r_lo = a.bin_lo * RS, r_hi = a.bin_hi * RS;
+    const int r_lo = a.bin_lo, r_hi = a.bin_hi;
     int tst = (consumer && active && a.tun) ? a.tun[w] : 0;
     unsigned ev = 0;
     unsigned long long nacc = 0;
     for (int64_t s0 = 0; s0 < a.sweeps; s0 += a.flush_every) {
-        const int64_t s1 = (a.sweeps < s0 + a.flush_every) ? a.sweeps : s0 + a.flush_every;
+        const int64_t nsw = (a.sweeps < s0 + a.flush_every) ? a.sweeps - s0 : (int64_t)a.flush_every;
+        const uint32_t g = g0 + (uint32_t)s0;
+        if (producer) {
+            if (part == 0)
+                produce_tn<SYS, L, 0>(nsw, g, wid, a.rk, lat, a.pstride, ring_u, ring_c, ring_r, full, empty, k, bad, drop_k);
+            else
+                produce_tn<SYS, L, 1>(nsw, g, wid, a.rk, lat, a.pstride, ring_u, ring_c, ring_r, full, empty, k, bad, -1);
+        } else if (consumer && !some) {  // a consumer warp with no walkers keeps the barrier protocol
 #pragma unroll 1
-        for (int64_t sw = s0; sw < s1; ++sw) {
-            const uint32_t g = g0 + (uint32_t)sw;
-            if (producer) {
-                if (part == 0)
-                    produce_sweep_tn<SYS, L, 0>(g, wid, a.rk, lat, a.pstride, ring_u, ring_c, ring_r, full, empty, k, bad,
-                                                drop_k);
-                else
-                    produce_sweep_tn<SYS, L, 1>(g, wid, a.rk, lat, a.pstride, ring_u, ring_c, ring_r, full, empty, k, bad,
-                                                -1);
-            } else if (consumer && active) {
-                unsigned na = 0;
-                if (a.record == 0)
-                    ising_sweep_tc<SYS, L, 0>(lat, a.pstride, bR, sTH, ring_u, ring_c, ring_r, full, empty, k, bad,
-                                              a.obs, na);
-                else
-                    ising_sweep_tc<SYS, L, 1>(lat, a.pstride, bR, sTH, ring_u, ring_c, ring_r, full, empty, k, bad,
-                                              a.obs, na);
-                nacc += na;
-                tunnel_step(bR, r_lo, r_hi, tst, ev);
-            } else if (consumer) {  // a consumer warp with no walkers keeps the barrier protocol
-#pragma unroll 1
-                for (int y = 0; y < L; ++y) {
-                    const int slot = k % kRing;
-                    if (!bad && !mbar_wait(&full[slot], (unsigned)((k / kRing) & 1))) bad = true;
-                    mbar_arrive(&empty[slot]);
-                    ++k;
-                }
+            for (int64_t r = 0; r < nsw * L; ++r) {
+                const int slot = k % kRing;
+                if (!bad && !mbar_wait(&full[slot], (unsigned)((k / kRing) & 1))) bad = true;
+                mbar_arrive(&empty[slot]);
+                ++k;
             }
+        } else if (consumer && active) {
+            if (a.record == 0)
+                consume_tn<SYS, L, 0>(nsw, lat, a.pstride, bR, sTH, ring_u, ring_c, ring_r, full, empty, k, bad,
+                                      a.obs, nacc, r_lo, r_hi, tst, ev);
+            else
+                consume_tn<SYS, L, 1>(nsw, lat, a.pstride, bR, sTH, ring_u, ring_c, ring_r, full, empty, k, bad,
+                                      a.obs, nacc, r_lo, r_hi, tst, ev);
         }
         __syncthreads();
-        for (int b = tid; b < a.B; b += blockDim.x) {
-            const uint32_t c = sTH[b * RS + C];
+        for (int b = tid; b < NB; b += blockDim.x) {
+            const uint32_t c = sTH[C * NB + b];
             if (c) {
                 Hb[b] += c;
-                sTH[b * RS + C] = 0u;
+                sTH[C * NB + b] = 0u;
             }
         }
         __syncthreads();
     }
     if (bad) atomicOr(const_cast<int *>(&a.state->err), 1);
     if (consumer && active) {
-        a.bin[w] = bR / RS;
+        a.bin[w] = bR;
         if (a.tun) a.tun[w] = (uint8_t)tst;
     }
     flush_metrics(a.metrics, nacc, ev);
@@ -519,6 +590,7 @@ __device__ __forceinline__ void produce_sweep_potts_tn(uint32_t g, uint32_t wid,
     constexpr int WR = L / 8;
     constexpr size_t S = (size_t)(L / 4) * 32;
     const uint32_t qm1 = q - 1u;
+    const PhiloxLane pl = philox_lane(g, wid, rk);
     uint32_t o[WR], d[WR], nn[WR];
 #pragma unroll 1
     for (int y = 0; y < L; ++y) {
@@ -552,7 +624,7 @@ __device__ __forceinline__ void produce_sweep_potts_tn(uint32_t g, uint32_t wid,
         if (i0 > 0 && i0 < i1) {
             // proposal of site 8 i0 - 1 (the second site of its Philox block): the c1
             // column of site 8 i0 has it as its recoloured left neighbour
-            const uint4 r = philox4x32_10_rk(make_uint4((uint32_t)(y * (L / 2) + 4 * i0 - 1), g, wid, kTagSweep), rk);
+            const uint4 r = philox4x32_10_group((uint32_t)(y * (L / 2) + 4 * i0 - 1), pl, rk);
             uint32_t v = (ob_prev >> 24) + 1u + __umulhi(r.z, qm1);
             v = (v >= q) ? v - q : v;
             pprev = v << 24;
@@ -568,8 +640,8 @@ __device__ __forceinline__ void produce_sweep_potts_tn(uint32_t g, uint32_t wid,
                 const uint32_t ob_next = nib_half_to_bytes(h == 0 ? o[0] : on, h ^ 1);
                 const uint32_t db = nib_half_to_bytes(d[0], h);
                 const uint32_t base = (uint32_t)(y * (L / 2) + 2 * j);
-                const uint4 r0 = philox4x32_10_rk(make_uint4(base, g, wid, kTagSweep), rk);
-                const uint4 r1 = philox4x32_10_rk(make_uint4(base + 1u, g, wid, kTagSweep), rk);
+                const uint4 r0 = philox4x32_10_group(base, pl, rk);
+                const uint4 r1 = philox4x32_10_group(base + 1u, pl, rk);
                 if (SPLIT)  // upper halves, clamped to 0xFFFE (split_hi)
                     wu16[j * 32] = make_uint2(__vminu2((r0.y >> 16) | (r0.w & 0xFFFF0000u), 0xFFFEFFFEu),
                                               __vminu2((r1.y >> 16) | (r1.w & 0xFFFF0000u), 0xFFFEFFFEu));
@@ -945,13 +1017,15 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
         }
     }
     if (tid == 0)  // per pair: FULL[RD] (NP producer warps arrive), EMPTY[RD] (the consumer)
-        for (int i = 0; i < ncw * 2 * RD; ++i) mbar_init(bars + i, ((i / RD) % 2 == 0) ? 32 * NP : 32);
+        for (int i = 0; i < ncw * 2 * RD; ++i)
+            mbar_init(bars + i, ((i / RD) % 2 == 0) ? 32 * NP : code_consumer_lanes(a.p - w0 - 32 * (i / (2 * RD))));
     set_block_spin_limit(a.spin_limit);
     checks_begin(a.B * RS, a.debug_check);
     __syncthreads();
 
     const int w = w0 + pair * 32 + lane;
     const bool active = w < a.p;
+    const bool some = w - lane < a.p;  // this warp has walkers
     const uint32_t wid = (uint32_t)(w + a.walker_offset);
     const uint32_t g0 = (uint32_t)a.state->sweep_counter;
     uint32_t *lat = a.lattice + (active ? w : 0);
@@ -997,7 +1071,7 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
                                              na, g, wid, a.key0, a.key1, a.T, Hb);
                 nacc += na;
                 tunnel_step(bR, r_lo, r_hi, tst, ev);
-            } else if (consumer) {
+            } else if (consumer && !some) {
 #pragma unroll 1
                 for (int y = 0; y < L; ++y) {
                     const int slot = k % RD;
@@ -1069,7 +1143,6 @@ template <int SYS>
 static cudaError_t launch_sys_tn(int L, const SpinSweepArgs &a, int block, cudaStream_t s)
 {
     switch (L) {
-    case 4: return launch_one_tn<SYS, 4>(a, block, s);
     case 8: return launch_one_tn<SYS, 8>(a, block, s);
     case 12: return launch_one_tn<SYS, 12>(a, block, s);
     case 16: return launch_one_tn<SYS, 16>(a, block, s);
