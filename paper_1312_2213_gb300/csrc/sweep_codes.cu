@@ -64,22 +64,12 @@ __device__ __forceinline__ uint4 clamp_words(uint4 u)
     return u;
 }
 
-// Producer warps per consumer warp in the Ising/MUMA code form (the Potts form
-// has kPottsProducers).  One Philox4x32-10 block costs a scheduler about 90
-// cycles of integer-multiply throughput and a single warp reaches about 134
-// cycles a block, so one producer cannot keep up with its consumer; the row's
+// Producer warps per consumer warp in the Ising/MUMA code form.  One Philox4x32-10 block costs a
+// scheduler 88 cycles of multiply and logic throughput and a single warp alone about 134
+// cycles, so one producer cannot keep up with its consumer; the row's
 // site groups are split over the producers (on other schedulers), which arrive
 // together on the row's FULL barrier.
 constexpr int kCodeProducers = 2;
-
-template <int WR>
-__device__ __forceinline__ void rotate_words(uint32_t (&o)[WR])  // o[e] <- o[e+1], cyclic
-{
-    const uint32_t t = o[0];
-#pragma unroll
-    for (int e = 0; e + 1 < WR; ++e) o[e] = o[e + 1];
-    o[WR - 1] = t;
-}
 
 // Warp roles of a code-form block of one or two walker warps (ncw).  The block
 // has 4 ncw warps, laid out so that, with warp w issuing from scheduler w mod 4,
@@ -87,8 +77,7 @@ __device__ __forceinline__ void rotate_words(uint32_t (&o)[WR])  // o[e] <- o[e+
 // pace) and the two producers of a consumer share another one:
 //   ncw = 1: [C0, idle, P0.0, P0.1]
 //   ncw = 2: [C0, C1, P0.0, P1.0, idle, idle, P0.1, P1.1]   (Pc.k: part k for consumer c)
-// Idle warps only take part in the block-wide barriers of the histogram flush
-// (the Potts form makes them a third producer part, see kPottsProducers).
+// Idle warps only take part in the block-wide barriers of the histogram flush.
 enum { kRoleConsumer = 0, kRoleProducer = 1, kRoleIdle = 2 };
 struct CodeRole {
     int kind, pair, part;
@@ -495,11 +484,6 @@ size_t spin_sweep_tn_smem_bytes(int system, int L, int B, int walkers_per_block)
 // of the same row, final by then) once a row.  The chain itself is the one of
 // the Ising code form.  RD is the ring depth in rows (4, or 2 where a deeper ring
 // does not fit next to the threshold table).
-__device__ __forceinline__ uint32_t ne_bytes(uint32_t a, uint32_t b)  // per byte [a != b], bytes < 16
-{
-    return (((a ^ b) + 0x0F0F0F0Fu) >> 4) & 0x01010101u;
-}
-
 __device__ __forceinline__ uint32_t nib_half_to_bytes(uint32_t w, int half)  // 4 nibbles -> 4 bytes
 {
     const uint32_t t = __byte_perm(w, 0u, half ? 0x3322u : 0x1100u);
@@ -511,22 +495,44 @@ __device__ __forceinline__ uint32_t bytes_to_nibs(uint32_t w0, uint32_t w1)  // 
     return __byte_perm(w0 | (w0 >> 4), w1 | (w1 >> 4), 0x6420u);
 }
 
-// Potts producers: kPottsProducers parts per consumer.  Parts 0 and 1 share a
-// scheduler; part 2 runs on the consumer's scheduler in the two-walker-warp
-// layout (the idle warps of the Ising layout) or on a scheduler of its own in
-// the one-walker-warp layout, and takes about a third of the row's nibble words.
-// A part may own no words; it still waits and arrives on every row.
-constexpr int kPottsProducers = 3;
-__host__ __device__ constexpr int potts_part_begin(int WR, int part)
+// Potts producers.  A Potts site takes two random words and eight neighbour comparisons, about 35
+// instructions against the consumer's 18; one warp issues an instruction every 2.5 cycles at best and
+// the multiply and logic pipes of a scheduler sustain a Philox block in 88 cycles, so production (not
+// the chain) bounds the blocks of two walker warps and is spread over more warps than the Ising
+// form's.  The block has 12 warps for two walker warps, 8 for one, warp w on scheduler w mod 4:
+//   ncw = 2: [C0, C1, P0.0, P1.0,  P0.3, P1.3, P0.1, P1.1,  -, -, P0.2, P1.2]
+//   ncw = 1: [C0, P0.0, P0.1, P0.2,  -, P0.3, P0.4, P0.5]
+// so a consumer shares its scheduler with one of its producers or with none.
+// Where the ring has four rows (L <= 32) four producers take whole rows in turn (produce_potts_rows).
+// With two rows (L = 48 and 64) all work on the same row: parts 0..n-1 own contiguous groups of four
+// sites, and a part beyond the first draws the block of the site left of its own once more.
+// Cycles a site with three producers on words of every row / as described: q = 8 L = 32, 8192
+// walkers 72.7 / 66.1 (4096 walkers 60.2 / 55.8), L = 24 77.6 / 66.9, L = 16 90.0 / 69.3, L = 8
+// 127 / 74; q = 10 L = 64, 4864 walkers or fewer 63.4 / 60.2, 8192 unchanged at 81 (five parts: 84).
+__host__ __device__ constexpr int potts_parts(int L, int ncw)  // parts with work
 {
-    // parts 0 / 1 / 2 own [0, n0), [n0, WR - n2), [WR - n2, WR) with n2 = (WR + 1) / 3
-    return part <= 0 ? 0 : part == 1 ? (WR - (WR + 1) / 3 + 1) / 2 : part == 2 ? WR - (WR + 1) / 3 : WR;
+    return ncw == 2 ? (L / 4 < 4 ? L / 4 : 4) : (L / 4 < 6 ? L / 4 : 6);
 }
+__host__ __device__ constexpr int potts_part_groups(int L, int ncw, int part)
+{
+    // as even as whole groups allow, the surplus with the first parts
+    return L / 4 / potts_parts(L, ncw) + (part < L / 4 % potts_parts(L, ncw) ? 1 : 0);
+}
+__host__ __device__ constexpr int potts_part_max(int L)  // most groups a part has, over both layouts
+{
+    return potts_part_groups(L, 2, 0) > potts_part_groups(L, 1, 0) ? potts_part_groups(L, 2, 0) : potts_part_groups(L, 1, 0);
+}
+__device__ __forceinline__ CodeRole potts_role(int warp, int ncw)
+{
+    if (ncw == 1)
+        return warp == 0 ? CodeRole{kRoleConsumer, 0, 0}
+                         : (warp == 4 ? CodeRole{kRoleIdle, 0, 0} : CodeRole{kRoleProducer, 0, warp < 4 ? warp - 1 : warp - 2});
+    if (warp < 2) return CodeRole{kRoleConsumer, warp, 0};
+    const int pair = warp & 1, row = warp >> 2;
+    return CodeRole{kRoleProducer, pair, (warp & 2) ? row : row + 2};
+}
+constexpr int potts_threads(int ncw) { return ncw == 2 ? 384 : 256; }
 
-// The producer runs a rolled loop over the row's nibble words (8 sites, 4
-// Philox blocks each); its old and down rows rotate through registers so that
-// word i is always element 0.  (A fully unrolled row was several times larger
-// than the instruction cache serves without fetch stalls.)
 // The split table (L = 64, see potts_split_full): the acceptance words travel as their
 // upper 16 bits, two to a 32-bit word (uint2 per 4 sites instead of uint4).
 template <int L>
@@ -576,121 +582,232 @@ __device__ __forceinline__ void split_scan(uint32_t *sTH, unsigned long long *Hb
     }
 }
 
-template <int L, int RD, int PART>
-__device__ __forceinline__ void produce_sweep_potts_tn(uint32_t g, uint32_t wid, const uint32_t (&rk)[20],
-                                                       const uint32_t *__restrict__ lat, int ps, uint32_t q,
-                                                       void *ring_u, uint2 *ring_c, uint2 *ring_op,
-                                                       unsigned long long *full, unsigned long long *empty, int &k,
-                                                       bool &bad, int drop_k, uint32_t *sTH, unsigned long long *Hb,
-                                                       int B, int F, int &since)
+// Codes travel as CSC c + bias with c = 4 + dE (without the up neighbour), CSC = 4 bytes a column (2
+// with the split table); the consumer flips the top bits behind the up neighbour's term, which leaves
+// the signed byte CSC (c - 4): the threshold's place in the bin's row, and RSW of it the bin's move.
+template <int L>
+struct PottsCode {
+    static constexpr int CSC = L > 48 ? 2 : 4;
+    static constexpr int SH = CSC == 4 ? 2 : 3;
+    static constexpr uint32_t BIAS = (0x80u - 4u * CSC) * 0x01010101u;
+    static constexpr uint32_t REST = 0x80808080u;  // dE = 0 at every site
+};
+__device__ __forceinline__ uint32_t ne16(uint32_t a, uint32_t b)  // per byte 16 [a != b], bytes < 16
+{
+    return ((a ^ b) + 0x0F0F0F0Fu) & 0x10101010u;
+}
+
+// Four sites of a row: bytes ob (old colours), those left (ob_prev, with its last proposal in the top
+// byte of pprev), right (ob_next) and below (db); r: the sites' two Philox blocks.  Returns the two
+// codes and the proposals in pb; last: the group holds the row's last site, whose right neighbour the
+// consumer adds; first: the row's first site does not see the site decided before it.
+template <int L>
+__device__ __forceinline__ uint2 potts_group(const uint4 (&r)[2], uint32_t q, uint32_t ob, uint32_t ob_prev, uint32_t ob_next,
+                                             uint32_t db, uint32_t pprev, bool first, uint32_t mask_last, uint32_t &pb)
+{
+    using PC = PottsCode<L>;
+    const uint32_t qm1 = q - 1u;
+    const uint32_t wrap = (0x80u - q) * 0x01010101u;  // per byte: top bit set iff v >= q
+    // proposals v = (s + 1 + mulhi(u, q - 1)) mod q, four bytes at once
+    const uint32_t t01 = __byte_perm(__umulhi(r[0].x, qm1), __umulhi(r[0].z, qm1), 0x0040u);
+    const uint32_t t23 = __byte_perm(__umulhi(r[1].x, qm1), __umulhi(r[1].z, qm1), 0x0040u);
+    pb = ob + 0x01010101u + __byte_perm(t01, t23, 0x5410u);
+    pb -= (((pb + wrap) & 0x80808080u) >> 7) * q;
+    const uint32_t R = __funnelshift_r(ob, ob_next, 8);   // right neighbours (old)
+    const uint32_t Lo = __funnelshift_l(ob_prev, ob, 8);  // left neighbours (old)
+    const uint32_t Lp = __funnelshift_l(pprev, pb, 8);    // left neighbours (recoloured)
+    const uint32_t nRp = ne16(R, pb) & mask_last, nRo = ne16(R, ob) & mask_last;
+    const uint32_t sp = 0x40404040u + nRp + ne16(db, pb);
+    const uint32_t so = nRo + ne16(db, ob);
+    // 16 c: every byte stays in [16, 112] and no partial result borrows across bytes
+    const uint32_t c0 = sp + ne16(Lo, pb) - so - ne16(Lo, ob);
+    uint32_t c1 = sp + ne16(Lp, pb) - so - ne16(Lp, ob);
+    if (first) c1 = __byte_perm(c0, c1, 0x7650u);
+    return make_uint2((c0 >> PC::SH) + PC::BIAS, (c1 >> PC::SH) + PC::BIAS);
+}
+
+// With a ring of RD = 4 rows, four producers: producer `part` makes every fourth row alone, always in
+// the ring's slot `part` (L is a multiple of four), so no block is drawn twice and three rows are on
+// the way while one is consumed.
+template <int L, int RD>
+__device__ __forceinline__ void produce_potts_rows(int64_t nsw, uint32_t sweep0, uint32_t wid, const uint32_t (&rk)[20],
+                                                   const uint32_t *__restrict__ lat, int ps, uint32_t q, int part,
+                                                   void *ring_u, uint2 *ring_c, uint2 *ring_op, unsigned long long *full,
+                                                   unsigned long long *empty, int &k, bool &bad, int drop_k)
+{
+    static_assert(L % 8 == 0 && L % RD == 0 && !PottsSplit<L>::on, "whole nibble words a row, whole turns of the ring");
+    constexpr int WR = L / 8;
+    constexpr size_t S = (size_t)(L / 4) * 32;
+    // Rows as in produce_tn: when slot `part` is free the consumer has finished the row four before, so
+    // from L = 16 up the two rows of the next turn (y + 4, y + 5) have their values for it and are
+    // loaded a turn ahead.
+    constexpr bool AHEAD = L >= 16;
+    uint32_t o[WR], d[WR], on[WR], dn[WR];
+    auto load = [&](int y, uint32_t (&a)[WR], uint32_t (&b)[WR]) {
+        const int y0 = y < L ? y : y - L, y1 = y + 1 < L ? y + 1 : y + 1 - L;
+#pragma unroll
+        for (int e = 0; e < WR; ++e) {
+            a[e] = lat[(y0 * WR + e) * ps];
+            b[e] = lat[(y1 * WR + e) * ps];
+        }
+    };
+    if (AHEAD) load(part, on, dn);
+    uint4 *wu = (uint4 *)ring_u + part * S;
+    uint2 *wc = ring_c + part * S;
+    uint2 *wop = ring_op + part * S;
+    k += part;
+#pragma unroll 1
+    for (int64_t sw = 0; sw < nsw; ++sw) {
+        const PhiloxLane pl = philox_lane(sweep0 + (uint32_t)sw, wid, rk);
+#pragma unroll 1
+        for (int y = part; y < L; y += RD) {
+            if (!bad && !mbar_wait(&empty[part], (unsigned)(((k / RD) & 1) ^ 1))) bad = true;
+            if (AHEAD) {
+#pragma unroll
+                for (int e = 0; e < WR; ++e) {
+                    o[e] = on[e];
+                    d[e] = dn[e];
+                }
+                load(y + RD, on, dn);
+            } else {
+                load(y, o, d);
+            }
+            uint32_t ob_prev = nib_half_to_bytes(o[WR - 1], 1), pprev = 0u;
+            uint32_t ob = nib_half_to_bytes(o[0], 0);
+#pragma unroll 1
+            for (int i = 0; i < WR; ++i) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int j = 2 * i + h;
+                    uint4 rr[2];
+                    philox4x32_10_groups<2>((uint32_t)(y * (L / 2) + 2 * j), pl, rk, rr);
+                    const uint32_t ob_next = nib_half_to_bytes(h == 0 ? o[0] : o[1 % WR], h ^ 1);
+                    uint32_t pb;
+                    const uint2 c = potts_group<L>(rr, q, ob, ob_prev, ob_next, nib_half_to_bytes(d[0], h), pprev, j == 0,
+                                                   (h == 1 && i == WR - 1) ? 0x00FFFFFFu : 0xFFFFFFFFu, pb);
+                    wu[j * 32] = clamp_words(make_uint4(rr[0].y, rr[0].w, rr[1].y, rr[1].w));
+                    wc[j * 32] = c;
+                    wop[j * 32] = make_uint2(ob, pb);
+                    ob_prev = ob;
+                    ob = ob_next;
+                    pprev = pb;
+                }
+                // the next word becomes word 0
+                const uint32_t t0 = o[0], t1 = d[0];
+#pragma unroll
+                for (int e = 0; e + 1 < WR; ++e) {
+                    o[e] = o[e + 1];
+                    d[e] = d[e + 1];
+                }
+                o[WR - 1] = t0;
+                d[WR - 1] = t1;
+            }
+            if (k != drop_k) mbar_arrive(&full[part]);
+            k += RD;
+        }
+    }
+    k -= part;
+}
+
+// The producer's rows of nsw sweeps: groups [g0, g0 + ng) of every row, the same code for every part.
+template <int L, int RD>
+__device__ __forceinline__ void produce_potts_tn(int64_t nsw, uint32_t sweep0, uint32_t wid, const uint32_t (&rk)[20],
+                                                 const uint32_t *__restrict__ lat, int ps, uint32_t q, int part, int g0,
+                                                 int ng, void *ring_u, uint2 *ring_c, uint2 *ring_op,
+                                                 unsigned long long *full, unsigned long long *empty, int &k, bool &bad,
+                                                 int drop_k, uint32_t *sTH, unsigned long long *Hb, int B, int F, int &since)
 {
     constexpr bool SPLIT = PottsSplit<L>::on;
     constexpr int RSW = 5;  // words a split row (only the split table is scanned)
     static_assert(L % 8 == 0, "whole nibble words a row");
     constexpr int WR = L / 8;
+    constexpr int NGM = potts_part_max(L);
+    constexpr int NA = (2 + NGM) / 2 + 1;  // words of the part's groups and one group on either side
     constexpr size_t S = (size_t)(L / 4) * 32;
     const uint32_t qm1 = q - 1u;
-    const PhiloxLane pl = philox_lane(g, wid, rk);
-    uint32_t o[WR], d[WR], nn[WR];
+    // Rolling rows as in produce_tn, of this part's words: word e is word g0 / 2 - 1 + e of the row,
+    // cyclic.
+    int off[NA + 1];
+#pragma unroll
+    for (int e = 0; e <= NA; ++e) off[e] = (g0 / 2 - 1 + e + WR * 4) % WR * ps;
+    const int odd = 16 * (g0 & 1);
+    uint32_t o[NA + 1], d[NA + 1], nn[NA + 1];
+#pragma unroll
+    for (int e = 0; e <= NA; ++e) {
+        o[e] = lat[off[e]];
+        d[e] = lat[WR * ps + off[e]];
+    }
+    const uint32_t mask_last = (g0 + ng == L / 4) ? 0x00FFFFFFu : 0xFFFFFFFFu;
 #pragma unroll 1
-    for (int y = 0; y < L; ++y) {
-        const int slot = k % RD;
-        if (!bad && !mbar_wait(&empty[slot], (unsigned)(((k / RD) & 1) ^ 1))) bad = true;
-        if (y == 0) {
-#pragma unroll
-            for (int j = 0; j < WR; ++j) {
-                o[j] = lat[j * ps];
-                d[j] = lat[(WR + j) * ps];
-            }
-        }
-        const int y2 = (y + 2 < L) ? y + 2 : y + 2 - L;
-        if (y + 1 < L) {
-#pragma unroll
-            for (int j = 0; j < WR; ++j) nn[j] = lat[(y2 * WR + j) * ps];
-        }
-        uint4 *wu = (uint4 *)ring_u + slot * S;
-        uint2 *wu16 = (uint2 *)ring_u + slot * S;
-        uint2 *wc = ring_c + slot * S;
-        uint2 *wop = ring_op + slot * S;
-        // this producer's nibble words [i0, i1); the arrays are rotated so that word i0 is element 0
-        constexpr int i0 = potts_part_begin(WR, PART), i1 = potts_part_begin(WR, PART + 1);
-#pragma unroll
-        for (int e = 0; e < i0; ++e) {
-            rotate_words<WR>(o);
-            rotate_words<WR>(d);
-        }
-        uint32_t ob_prev = nib_half_to_bytes(o[WR - 1], 1);  // the four sites left of word i0 (cyclic)
-        uint32_t pprev = 0u;                                  // site 0's c1 is never used
-        if (i0 > 0 && i0 < i1) {
-            // proposal of site 8 i0 - 1 (the second site of its Philox block): the c1
-            // column of site 8 i0 has it as its recoloured left neighbour
-            const uint4 r = philox4x32_10_group((uint32_t)(y * (L / 2) + 4 * i0 - 1), pl, rk);
-            uint32_t v = (ob_prev >> 24) + 1u + __umulhi(r.z, qm1);
-            v = (v >= q) ? v - q : v;
-            pprev = v << 24;
-        }
+    for (int64_t sw = 0; sw < nsw; ++sw) {
+        const PhiloxLane pl = philox_lane(sweep0 + (uint32_t)sw, wid, rk);
 #pragma unroll 1
-        for (int i = i0; i < i1; ++i) {
-            const uint32_t on = o[1 % WR];  // next nibble word, cyclic
-            const uint32_t mask_last = (i == WR - 1) ? 0x00FFFFFFu : 0xFFFFFFFFu;
+        for (int y = 0; y < L; ++y) {
+            const int slot = k % RD;
+            bool free_slot = mbar_try(&empty[slot], (unsigned)(((k / RD) & 1) ^ 1));
+            // the part's groups at even halves of words: group g0 + i is half i & 1 of word 1 + i / 2
+            uint32_t ow[NA], dw[NA];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = 2 * i + h;
-                const uint32_t ob = nib_half_to_bytes(o[0], h);
-                const uint32_t ob_next = nib_half_to_bytes(h == 0 ? o[0] : on, h ^ 1);
-                const uint32_t db = nib_half_to_bytes(d[0], h);
-                const uint32_t base = (uint32_t)(y * (L / 2) + 2 * j);
-                const uint4 r0 = philox4x32_10_group(base, pl, rk);
-                const uint4 r1 = philox4x32_10_group(base + 1u, pl, rk);
-                if (SPLIT)  // upper halves, clamped to 0xFFFE (split_hi)
-                    wu16[j * 32] = make_uint2(__vminu2((r0.y >> 16) | (r0.w & 0xFFFF0000u), 0xFFFEFFFEu),
-                                              __vminu2((r1.y >> 16) | (r1.w & 0xFFFF0000u), 0xFFFEFFFEu));
-                else
-                    wu[j * 32] = clamp_words(make_uint4(r0.y, r0.w, r1.y, r1.w));
-                const uint32_t up4[4] = {r0.x, r0.z, r1.x, r1.z};
-                uint32_t pb = 0u;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    uint32_t v = ((ob >> (8 * e)) & 0xffu) + 1u + __umulhi(up4[e], qm1);
-                    v = (v >= q) ? v - q : v;
-                    pb |= v << (8 * e);
-                }
-                const uint32_t R = __funnelshift_r(ob, ob_next, 8);   // right neighbours (old)
-                const uint32_t Lo = __funnelshift_l(ob_prev, ob, 8);  // left neighbours (old)
-                const uint32_t Lp = __funnelshift_l(pprev, pb, 8);    // left neighbours (recoloured)
-                uint32_t nRp = ne_bytes(R, pb), nRo = ne_bytes(R, ob);
-                if (h == 1) {  // the row's last site: its right neighbour is added by the consumer
-                    nRp &= mask_last;
-                    nRo &= mask_last;
-                }
-                const uint32_t sp = 0x04040404u + nRp + ne_bytes(db, pb);
-                const uint32_t so = nRo + ne_bytes(db, ob);
-                // every byte stays in [1, 7] and no partial result borrows across bytes
-                const uint32_t c0 = sp + ne_bytes(Lo, pb) - so - ne_bytes(Lo, ob);
-                const uint32_t c1 = sp + ne_bytes(Lp, pb) - so - ne_bytes(Lp, ob);
-                wc[j * 32] = make_uint2(c0, c1);
-                wop[j * 32] = make_uint2(ob, pb);
-                ob_prev = ob;
-                pprev = pb;
+            for (int e = 0; e < NA; ++e) {
+                ow[e] = __funnelshift_r(o[e], o[e + 1], odd);
+                dw[e] = __funnelshift_r(d[e], d[e + 1], odd);
             }
-            rotate_words<WR>(o);
-            rotate_words<WR>(d);
-        }
+            uint32_t ob_prev = nib_half_to_bytes(ow[0], 1);  // the four sites left of group g0 (cyclic)
+            uint32_t pprev = 0u;
+            if (g0 > 0) {
+                // proposal of site 4 g0 - 1 (the second site of its Philox block): the c1
+                // column of site 4 g0 has it as its recoloured left neighbour
+                const uint4 r = philox4x32_10_group((uint32_t)(y * (L / 2) + 2 * g0 - 1), pl, rk);
+                uint32_t v = (ob_prev >> 24) + 1u + __umulhi(r.z, qm1);
+                v = (v >= q) ? v - q : v;
+                pprev = v << 24;
+            }
+            uint32_t ob = nib_half_to_bytes(ow[1], 0);
+            uint4 *wu = (uint4 *)ring_u + slot * S;
+            uint2 *wu16 = (uint2 *)ring_u + slot * S;
+            uint2 *wc = ring_c + slot * S;
+            uint2 *wop = ring_op + slot * S;
 #pragma unroll
-        for (int e = i1; e < WR; ++e) {  // back to word 0 first (WR rotations in all)
-            rotate_words<WR>(o);
-            rotate_words<WR>(d);
-        }
-        if (k != drop_k) mbar_arrive(&full[slot]);
-        ++k;
-        if (SPLIT && PART == 1) {  // empty one F-th of the 16-bit counters (split_scan)
-            split_scan<RSW>(sTH, Hb, B, (int)(threadIdx.x & 31), since, F);
-            if (++since == F) since = 0;
-        }
+            for (int i = 0; i < NGM; ++i) {
+                if (i < ng) {
+                    const int j = g0 + i;
+                    uint4 r[2];
+                    philox4x32_10_groups<2>((uint32_t)(y * (L / 2) + 2 * j), pl, rk, r);
+                    const uint32_t ob_next = nib_half_to_bytes(ow[(3 + i) / 2], (3 + i) & 1);
+                    const uint32_t db = nib_half_to_bytes(dw[(2 + i) / 2], i & 1);
+                    uint32_t pb;
+                    const uint2 c = potts_group<L>(r, q, ob, ob_prev, ob_next, db, pprev, j == 0,
+                                                   i == ng - 1 ? mask_last : 0xFFFFFFFFu, pb);
+                    if (i == 0) {
+                        if (!free_slot && !bad && !mbar_wait(&empty[slot], (unsigned)(((k / RD) & 1) ^ 1))) bad = true;
+                        // (also behind the last row: rows 0 and 1 as this sweep leaves them)
+                        const int y2 = (y + 2 < L) ? y + 2 : y + 2 - L;
 #pragma unroll
-        for (int j = 0; j < WR; ++j) {
-            o[j] = d[j];
-            d[j] = nn[j];
+                        for (int e = 0; e <= NA; ++e) nn[e] = lat[y2 * WR * ps + off[e]];
+                    }
+                    if (SPLIT)  // upper halves, clamped to 0xFFFE (split_hi)
+                        wu16[j * 32] = make_uint2(__vminu2((r[0].y >> 16) | (r[0].w & 0xFFFF0000u), 0xFFFEFFFEu),
+                                                  __vminu2((r[1].y >> 16) | (r[1].w & 0xFFFF0000u), 0xFFFEFFFEu));
+                    else
+                        wu[j * 32] = clamp_words(make_uint4(r[0].y, r[0].w, r[1].y, r[1].w));
+                    wc[j * 32] = c;
+                    wop[j * 32] = make_uint2(ob, pb);
+                    ob_prev = ob;
+                    ob = ob_next;
+                    pprev = pb;
+                }
+            }
+            if (k != drop_k) mbar_arrive(&full[slot]);
+            ++k;
+            if (SPLIT && part == 1) {  // empty one F-th of the 16-bit counters (split_scan)
+                split_scan<RSW>(sTH, Hb, B, (int)(threadIdx.x & 31), since, F);
+                if (++since == F) since = 0;
+            }
+#pragma unroll
+            for (int e = 0; e <= NA; ++e) {
+                o[e] = d[e];
+                d[e] = nn[e];
+            }
         }
     }
 }
@@ -760,8 +877,8 @@ __device__ __forceinline__ void potts_redo_row(uint32_t *__restrict__ lat, int p
     for (int j = 0; j < W4; ++j) {
         const uint2 op = rop[j * 32];
         const uint32_t ubw = uOld[j * 32];
-        const uint32_t np = ne_bytes(ubw, op.y), no = ne_bytes(ubw, op.x);
-        const uint32_t cx = (rc[j * 32].x + np - no) << 1, cy = (rc[j * 32].y + np - no) << 1;
+        const uint32_t np = ne16(ubw, op.y) >> PottsCode<L>::SH, no = ne16(ubw, op.x) >> PottsCode<L>::SH;
+        const uint32_t cx = rc[j * 32].x + np - no - PottsCode<L>::BIAS, cy = rc[j * 32].y + np - no - PottsCode<L>::BIAS;
         const uint2 h = ru16[j * 32];
         uint32_t amw = 0u, amr = 0u;
 #pragma unroll 1
@@ -810,25 +927,27 @@ __device__ __forceinline__ void potts_redo_row(uint32_t *__restrict__ lat, int p
     nacc += nar - naw;  // modulo 2^32, like the count itself
 }
 
-// The consumer runs a loop over the row's byte words (4 sites each), unrolled
-// by two (rolled it lost 16-20 % to loop overhead between the words' chains;
-// fully unrolled, L = 48 stalled on instruction fetch), and peels the last
-// word, which holds the last site's right-neighbour term.  The final row above
+// The consumer's rows of nsw sweeps, joined as in consume_tn: the next row is asked for two byte words
+// ahead, and its first site's threshold is loaded for both outcomes of the row's last.  A row is a
+// loop over its byte words (4 sites each), unrolled by two (rolled it lost 16-20 % to loop overhead
+// between the words' chains; fully unrolled, L = 48 stalled on instruction fetch), with the last
+// word, which holds the last site's right-neighbour term, peeled.  The final row above
 // lives in a per-lane shared-memory row (bytes).  With the split table there are
 // two such rows, read and written in turn (the row being decided reads one and
 // writes the other), so that a redo still has the row above; otherwise one row
 // is rewritten word by word as the current row completes.
 template <int L, int RD, int RECORD>
-__device__ __forceinline__ void potts_sweep_tc(uint32_t *__restrict__ lat, int ps, int &bR,
-                                               uint32_t *__restrict__ sTH, const void *__restrict__ ring_u_,
-                                               const uint2 *__restrict__ ring_c, const uint2 *__restrict__ ring_op,
-                                               uint32_t *__restrict__ sU, unsigned long long *full,
-                                               unsigned long long *empty, int &k, bool &bad, unsigned &nacc,
-                                               uint32_t g, uint32_t wid, uint32_t key0, uint32_t key1,
-                                               const uint32_t *__restrict__ Tg, unsigned long long *Hb)
+__device__ __forceinline__ void consume_potts_tn(int64_t nsw, uint32_t sweep0, uint32_t *__restrict__ lat, int ps, int &bR,
+                                                 uint32_t *__restrict__ sTH, const void *__restrict__ ring_u_,
+                                                 const uint2 *__restrict__ ring_c, const uint2 *__restrict__ ring_op,
+                                                 uint32_t *__restrict__ sU, unsigned long long *full,
+                                                 unsigned long long *empty, int &k, bool &bad, unsigned long long &nacc,
+                                                 int r_lo, int r_hi, int &tst, unsigned &ev, uint32_t wid, uint32_t key0,
+                                                 uint32_t key1, const uint32_t *__restrict__ Tg, unsigned long long *Hb)
 {
     static_assert(L % 8 == 0, "whole nibble words a row");
     using R = PottsRow<L>;
+    using PC = PottsCode<L>;
     constexpr bool SPLIT = R::split;
     constexpr int WR = L / 8;
     constexpr int W4 = L / 4;
@@ -836,130 +955,149 @@ __device__ __forceinline__ void potts_sweep_tc(uint32_t *__restrict__ lat, int p
     static_assert(!SPLIT || L % 2 == 0, "the up rows alternate: row L - 1 must leave its values in the first");
     const uint4 *ring_u = (const uint4 *)ring_u_;
     const uint2 *ring_u16 = (const uint2 *)ring_u_;
-    // byte i of a packed word (selector bytes 4 pick zeros)
-    auto byte_of = [](uint32_t w, int i) -> int { return (int)__byte_perm(w, 0u, 0x4440u | (uint32_t)i); };
-    // As in the Ising consumer: 32-bit shared-window byte addresses (bB = table base + 4 RSW bin,
-    // codes scaled to CSC c), clamped acceptance words, one compare (split: upper halves).
+    // As in the Ising consumer: 32-bit shared-window byte addresses (bB = table base + 4 RSW bin),
+    // clamped acceptance words, one compare (split: upper halves).
     const int sbase = (int)__cvta_generic_to_shared(sTH);
+    constexpr int TOFF = R::C4;  // signed codes count from column 4
     auto th = [sbase](int addr) -> uint32_t {
         uint32_t v;
         if (SPLIT)
-            asm("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(checked_addr(addr, sbase)));
+            asm("ld.shared.u16 %0, [%1 + %2];" : "=r"(v) : "r"(checked_addr(addr + TOFF, sbase) - TOFF), "n"(TOFF));
         else
-            asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(checked_addr(addr, sbase)));
+            asm("ld.shared.u32 %0, [%1 + %2];" : "=r"(v) : "r"(checked_addr(addr + TOFF, sbase) - TOFF), "n"(TOFF));
         return v;
     };
     auto hist = [sbase](int addr) {
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(checked_addr(addr, sbase)), "r"(R::ONE) : "memory");
+        asm volatile("red.shared.add.u32 [%0 + %2], %1;" ::"r"(checked_addr(addr + 4 * R::HW, sbase) - 4 * R::HW),
+                     "r"(R::ONE), "n"(4 * R::HW)
+                     : "memory");
     };
+    // threshold address and bin move of byte i of settled codes
+    auto at = [](uint32_t c, int i, int b) -> int { return __dp4a((int)c, 1 << (8 * i), b); };
+    constexpr int MOVE = 4 * R::RSW / PC::CSC;
+    auto moved = [](uint32_t c, int i, int b) -> int { return __dp4a((int)c, MOVE << (8 * i), b); };
+    // codes with the up neighbour's term added (bytes CSC (c - 4))
+    auto settle = [](uint2 c, uint2 op, uint32_t ubw) -> uint2 {
+        const uint32_t np = ne16(ubw, op.y) >> PC::SH, no = ne16(ubw, op.x) >> PC::SH;
+        return make_uint2((c.x + np - no) ^ PC::REST, (c.y + np - no) ^ PC::REST);
+    };
+    const int k_end = k + (int)(nsw * L);
     int bB = sbase + bR * 4;
-#pragma unroll 1
-    for (int y = 0; y < L; ++y) {
+    uint2 opn = make_uint2(0u, 0u), cdn = opn;
+    uint32_t T0 = 0u, T1 = 0u;
+    bool accP = false;  // the site decided before
+    bool tie = false;
+    // decide the current site (codes of its word c, byte i; threshold T0 or T1 by the previous
+    // decision) and load both candidates of the next site, byte jn of the codes n
+    auto site = [&](uint32_t uw, const uint2 &c, int i, const uint2 &n, int jn, uint32_t &am) {
+        const int bA = moved(accP ? c.y : c.x, i, bB);
+        const uint32_t T = accP ? T1 : T0;
+        T0 = th(at(n.x, jn, bB));
+        T1 = th(at(n.y, jn, bA));
+        const bool acc = uw < T;  // the producer's clamp makes this "always or u < T"
+        if (SPLIT) tie |= uw == T;  // upper halves equal: the row is redone (potts_redo_row)
+        if (acc) am |= 0xffu << (8 * i);
+        bB = acc ? bA : bB;
+        if (RECORD == 0) hist(bB);
+        accP = acc;
+    };
+    if (!bad && !mbar_wait(&full[k % RD], (unsigned)((k / RD) & 1))) bad = true;
+    if (!bad) {
         const int slot = k % RD;
-        if (!bad && !mbar_wait(&full[slot], (unsigned)((k / RD) & 1))) bad = true;
-        if (bad) {  // a wait gave up: the ring is out of step, so nothing more is computed
-            mbar_arrive(&empty[slot]);
-            ++k;
-            continue;
-        }
-        const uint4 *ru = ring_u + slot * S;
-        const uint2 *ru16 = ring_u16 + slot * S;
-        const uint2 *rc = ring_c + slot * S;
-        const uint2 *rop = ring_op + slot * S;
-        const uint32_t *uOld = (SPLIT && (y & 1)) ? sU + S : sU;  // the row above
-        uint32_t *uNew = (SPLIT && !(y & 1)) ? sU + S : sU;       // this row, as it is decided
-        const int b0 = bB;
-        bool tie = false;
-        // the acceptance words of byte word j (split: their upper halves)
-        auto words = [&](int j) -> uint4 {
-            if (SPLIT) {
-                const uint2 h = ru16[j * 32];
-                return make_uint4(h.x & 0xFFFFu, h.x >> 16, h.y & 0xFFFFu, h.y >> 16);
-            }
-            return ru[j * 32];
-        };
-        // code bytes of word j with the up neighbour's term added (bytes stay in [0, 8]),
-        // scaled to byte offsets CSC c
-        auto codes = [&](int j, uint2 op, uint32_t ubw) -> uint2 {
-            uint2 c = rc[j * 32];
-            const uint32_t np = ne_bytes(ubw, op.y), no = ne_bytes(ubw, op.x);
-            c.x = (c.x + np - no) << (SPLIT ? 1 : 2);
-            c.y = (c.y + np - no) << (SPLIT ? 1 : 2);
-            return c;
-        };
-        uint2 opn = rop[0];
-        uint2 cdn = codes(0, opn, uOld[0]);
-        const int c00 = byte_of(cdn.x, 0);
-        uint32_t T0 = th(bB + c00), T1 = 0u;
-        int d0 = (c00 - R::C4) * R::MS, d1 = 0;  // bin-row move (c - 4) rows, in bytes
-        bool accP = false;
-        // decide the current site (threshold T0 or T1 by the previous decision) and
-        // load both candidates of the next site, whose code bytes are n0 / n1
-        auto site = [&](uint32_t uw, int n0, int n1, uint32_t &am, int i) {
-            const int dR = accP ? d1 : d0;
-            const uint32_t T = accP ? T1 : T0;
-            T0 = th(bB + n0);
-            T1 = th(bB + dR + n1);
-            d0 = (n0 - R::C4) * R::MS;
-            d1 = (n1 - R::C4) * R::MS;
-            const bool acc = uw < T;  // the producer's clamp makes this "always or u < T"
-            if (SPLIT) tie |= uw == T;  // upper halves equal: the row is redone (potts_redo_row)
-            if (acc) am |= 0xffu << (8 * i);
-            bB = acc ? bB + dR : bB;
-            if (RECORD == 0) hist(bB + 4 * R::HW);
-            accP = acc;
-        };
-        uint32_t fprev = 0u;
+        opn = ring_op[slot * S];
+        cdn = settle(ring_c[slot * S], opn, sU[0]);
+        T0 = T1 = th(at(cdn.x, 0, bB));
+    }
+#pragma unroll 1
+    for (int64_t sw = 0; sw < nsw && !bad; ++sw) {
+        unsigned na = 0;
+#pragma unroll 1
+        for (int y = 0; y < L; ++y) {
+            const int slot = k % RD, slot_n = (k + 1) % RD;
+            const uint4 *ru = ring_u + slot * S;
+            const uint2 *ru16 = ring_u16 + slot * S;
+            const uint2 *rc = ring_c + slot * S;
+            const uint2 *rop = ring_op + slot * S;
+            const uint32_t *uOld = (SPLIT && (y & 1)) ? sU + S : sU;  // the row above
+            uint32_t *uNew = (SPLIT && !(y & 1)) ? sU + S : sU;       // this row, as it is decided
+            const int b0 = bB;
+            // the acceptance words of byte word j (split: their upper halves)
+            auto words = [&](int j) -> uint4 {
+                if (SPLIT) {
+                    const uint2 h = ru16[j * 32];
+                    return make_uint4(h.x & 0xFFFFu, h.x >> 16, h.y & 0xFFFFu, h.y >> 16);
+                }
+                return ru[j * 32];
+            };
+            uint32_t fprev = 0u;
 #pragma unroll 2
-        for (int j = 0; j < W4 - 1; ++j) {
-            const uint2 op = opn, cd = cdn;
-            const uint4 u = words(j);
-            opn = rop[(j + 1) * 32];
-            cdn = codes(j + 1, opn, uOld[(j + 1) * 32]);
-            uint32_t am = 0u;
-            site(u.x, byte_of(cd.x, 1), byte_of(cd.y, 1), am, 0);
-            site(u.y, byte_of(cd.x, 2), byte_of(cd.y, 2), am, 1);
-            site(u.z, byte_of(cd.x, 3), byte_of(cd.y, 3), am, 2);
-            site(u.w, byte_of(cdn.x, 0), byte_of(cdn.y, 0), am, 3);
-            nacc += (unsigned)__popc(am);  // 0xff per accepted site: 8 x accepted (divided at the end)
-            const uint32_t f = op.x ^ ((op.x ^ op.y) & am);
-            uNew[j * 32] = f;
-            if (j & 1) lat[(y * WR + (j >> 1)) * ps] = bytes_to_nibs(fprev, f);
-            fprev = f;
+            for (int j = 0; j < W4 - 1; ++j) {
+                const uint2 op = opn, cd = cdn;
+                const uint4 u = words(j);
+                opn = rop[(j + 1) * 32];
+                cdn = settle(rc[(j + 1) * 32], opn, uOld[(j + 1) * 32]);
+                uint32_t am = 0u;
+                site(u.x, cd, 0, cd, 1, am);
+                site(u.y, cd, 1, cd, 2, am);
+                site(u.z, cd, 2, cd, 3, am);
+                site(u.w, cd, 3, cdn, 0, am);
+                na += (unsigned)__popc(am);  // 0xff per accepted site: 8 x accepted (divided at the end)
+                const uint32_t f = op.x ^ ((op.x ^ op.y) & am);
+                uNew[j * 32] = f;
+                if (j & 1) lat[(y * WR + (j >> 1)) * ps] = bytes_to_nibs(fprev, f);
+                fprev = f;
+            }
+            {
+                constexpr int j = W4 - 1;
+                bool next = mbar_try(&full[slot_n], (unsigned)(((k + 1) / RD) & 1));
+                const uint2 op = opn;
+                uint2 cd = cdn;
+                const uint4 u = words(j);
+                uint32_t am = 0u;
+                site(u.x, cd, 0, cd, 1, am);
+                site(u.y, cd, 1, cd, 2, am);
+                // the last site's right neighbour is site 0 of this row, final by now (word 0 is written);
+                // its code is the top byte
+                const uint32_t f0 = uNew[0];
+                const uint32_t t = (PC::CSC << 24) * (uint32_t)((int)((f0 & 0xffu) != (op.y >> 24)) - (int)((f0 & 0xffu) != (op.x >> 24)));
+                cd.x += t;
+                cd.y += t;
+                // the next row; behind the last one (or a wait that gave up) an earlier row's codes
+                // are read and not used
+                if (!next && !(sw + 1 == nsw && y == L - 1))
+                    bad = !mbar_wait(&full[slot_n], (unsigned)(((k + 1) / RD) & 1));
+                opn = ring_op[slot_n * S];
+                const uint2 rcn = ring_c[slot_n * S];
+                site(u.z, cd, 2, cd, 3, am);
+                cdn = settle(rcn, opn, f0);
+                site(u.w, cd, 3, cdn, 0, am);
+                na += (unsigned)__popc(am);
+                const uint32_t f = op.x ^ ((op.x ^ op.y) & am);
+                uNew[j * 32] = f;
+                lat[(y * WR + WR - 1) * ps] = bytes_to_nibs(fprev, f);
+                if (SPLIT && tie) {
+                    potts_redo_row<L>(lat, ps, y, sbase, b0, bB, ru16, rc, rop, uOld, uNew, Hb, RECORD, na, sweep0 + (uint32_t)sw,
+                                      wid, key0, key1, Tg);
+                    cdn = settle(rcn, opn, uNew[0]);
+                    T0 = T1 = th(at(cdn.x, 0, bB));
+                    tie = false;
+                }
+            }
+            mbar_arrive(&empty[slot]);  // after the row is stored: the producer reads it later
+            ++k;
+            if (bad) break;
         }
-        {
-            constexpr int j = W4 - 1;
-            const uint2 op = opn, cd = cdn;
-            const uint4 u = words(j);
-            uint32_t am = 0u;
-            site(u.x, byte_of(cd.x, 1), byte_of(cd.y, 1), am, 0);
-            site(u.y, byte_of(cd.x, 2), byte_of(cd.y, 2), am, 1);
-            // the last site's right neighbour is site 0 of this row, final by now (word 0 is written)
-            const uint32_t f0 = uNew[0] & 0xffu;
-            const int t = (int)(f0 != (op.y >> 24)) - (int)(f0 != (op.x >> 24));
-            site(u.z, byte_of(cd.x, 3) + R::CSC * t, byte_of(cd.y, 3) + R::CSC * t, am, 2);
-            // the last site: decision only
-            const int dR = accP ? d1 : d0;
-            const uint32_t T = accP ? T1 : T0;
-            const bool acc = u.w < T;
-            if (SPLIT) tie |= u.w == T;
-            if (acc) am |= 0xff000000u;
-            bB = acc ? bB + dR : bB;
-            if (RECORD == 0) hist(bB + 4 * R::HW);
-            nacc += (unsigned)__popc(am);
-            const uint32_t f = op.x ^ ((op.x ^ op.y) & am);
-            uNew[j * 32] = f;
-            lat[(y * WR + WR - 1) * ps] = bytes_to_nibs(fprev, f);
-        }
-        if (SPLIT && tie)
-            potts_redo_row<L>(lat, ps, y, sbase, b0, bB, ru16, rc, rop, uOld, uNew, Hb, RECORD, nacc, g, wid, key0,
-                              key1, Tg);
-        mbar_arrive(&empty[slot]);  // after the row is stored: the producer reads it later
+        nacc += na >> 3;
+        if (bad) break;
+        const int word = (bB - sbase) / 4;
+        if (RECORD == 1) atomicAdd(&sTH[checked_word(word + R::HW)], R::ONE);
+        tunnel_step(word, r_lo, r_hi, tst, ev);
+    }
+    while (k != k_end) {  // a wait gave up: the ring is out of step, so nothing more is computed
+        mbar_arrive(&empty[k % RD]);
         ++k;
     }
     bR = (bB - sbase) / 4;
-    nacc >>= 3;
-    if (RECORD == 1) atomicAdd(&sTH[checked_word(bR + R::HW)], R::ONE);
 }
 
 // Shared memory a consumer warp owns: RD ring rows (acceptance words 16 B, or their
@@ -984,14 +1122,21 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
     constexpr int C = 9;
     constexpr int RS = R::RSW;  // words a table row
     constexpr size_t S = (size_t)(L / 4) * 32;
-    constexpr int NP = kPottsProducers;
-    const int ncw = blockDim.x / (32 * kCodeWarpsPerWalkerWarp);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    CodeRole role = code_role(warp, ncw);
-    if (role.kind == kRoleIdle) role = CodeRole{kRoleProducer, ncw == 1 ? 0 : (warp & 1), 2};
-    const bool producer = role.kind == kRoleProducer, consumer = role.kind == kRoleConsumer;
+    const int ncw = blockDim.x == (unsigned)potts_threads(2) ? 2 : 1;
+    // (from lane 0, so that the compiler knows it is the same for the warp)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const CodeRole role = potts_role(warp, ncw);
+    constexpr bool ROWS = RD == 4;            // producers take whole rows in turn, else groups of every row
+    const int NP = ROWS ? RD : potts_parts(L, ncw);  // further producers are idle
     const int pair = role.pair, part = role.part;
-    const int drop_k = (blockIdx.x == 0 && producer && pair == 0 && part == 0) ? a.debug_drop_row : -1;
+    const bool producer = role.kind == kRoleProducer && part < NP, consumer = role.kind == kRoleConsumer;
+    int g0 = 0, ng = 0;  // a producer's groups of the row
+    for (int i = 0; i <= part && producer && !ROWS; ++i) {
+        g0 += ng;
+        ng = potts_part_groups(L, ncw, i);
+    }
+    // (the test hook's row: with whole rows in turn, of the producer whose turn it is)
+    const int drop_k = (blockIdx.x == 0 && producer && pair == 0 && (ROWS || part == 0)) ? a.debug_drop_row : -1;
     uint32_t *sTH = smem;
     const size_t th_bytes = tnp_table_bytes(L, a.B);
     constexpr size_t UB = R::split ? 8 : 16;  // ring bytes of a group's acceptance words
@@ -1016,9 +1161,16 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
             sTH[i] = (c < C) ? a.T[b * C + c] : 0u;
         }
     }
+    // as in the Ising form: codes read ahead of a row that never came address the table
+    for (int i = tid; i < ncw * RD * (int)S; i += blockDim.x) {
+        char *rb = (char *)smem + th_bytes + (size_t)(i / (RD * (int)S)) * tnp_warp_bytes(L, RD) + (size_t)RD * S * UB;
+        const int e = i % (RD * (int)S);
+        ((uint2 *)rb)[e] = make_uint2(PottsCode<L>::REST, PottsCode<L>::REST);
+        ((uint2 *)(rb + (size_t)RD * S * 8))[e] = make_uint2(0u, 0u);
+    }
     if (tid == 0)  // per pair: FULL[RD] (NP producer warps arrive), EMPTY[RD] (the consumer)
         for (int i = 0; i < ncw * 2 * RD; ++i)
-            mbar_init(bars + i, ((i / RD) % 2 == 0) ? 32 * NP : code_consumer_lanes(a.p - w0 - 32 * (i / (2 * RD))));
+            mbar_init(bars + i, ((i / RD) % 2 == 0) ? (ROWS ? 32 : 32 * NP) : code_consumer_lanes(a.p - w0 - 32 * (i / (2 * RD))));
     set_block_spin_limit(a.spin_limit);
     checks_begin(a.B * RS, a.debug_check);
     __syncthreads();
@@ -1027,7 +1179,7 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
     const bool active = w < a.p;
     const bool some = w - lane < a.p;  // this warp has walkers
     const uint32_t wid = (uint32_t)(w + a.walker_offset);
-    const uint32_t g0 = (uint32_t)a.state->sweep_counter;
+    const uint32_t g_first = (uint32_t)a.state->sweep_counter;
     uint32_t *lat = a.lattice + (active ? w : 0);
     int bR = (active ? a.bin[w] : 0) * RS;
     unsigned long long *Hb = a.Hpart + (size_t)slot_id * a.B;
@@ -1047,39 +1199,30 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
             sU[j * 32] = nib_half_to_bytes(lat[((L - 1) * WR + (j >> 1)) * a.pstride], j & 1);
     }
     for (int64_t s0 = 0; s0 < a.sweeps; s0 += a.flush_every) {
-        const int64_t s1 = (a.sweeps < s0 + a.flush_every) ? a.sweeps : s0 + a.flush_every;
+        const int64_t nsw = (a.sweeps < s0 + a.flush_every) ? a.sweeps - s0 : (int64_t)a.flush_every;
+        const uint32_t g = g_first + (uint32_t)s0;
+        if (producer) {
+            if constexpr (ROWS)
+                produce_potts_rows<L, RD>(nsw, g, wid, a.rk, lat, a.pstride, (uint32_t)a.q, part, ring_u, ring_c, ring_op, full,
+                                          empty, k, bad, drop_k);
+            else
+                produce_potts_tn<L, RD>(nsw, g, wid, a.rk, lat, a.pstride, (uint32_t)a.q, part, g0, ng, ring_u, ring_c, ring_op,
+                                    full, empty, k, bad, drop_k, sTH, Hb, a.B, F, since);
+        } else if (consumer && !some) {  // a consumer warp with no walkers keeps the barrier protocol
 #pragma unroll 1
-        for (int64_t sw = s0; sw < s1; ++sw) {
-            const uint32_t g = g0 + (uint32_t)sw;
-            if (producer) {
-                if (part == 0)
-                    produce_sweep_potts_tn<L, RD, 0>(g, wid, a.rk, lat, a.pstride, (uint32_t)a.q, ring_u, ring_c,
-                                                     ring_op, full, empty, k, bad, drop_k, sTH, Hb, a.B, F, since);
-                else if (part == 1)
-                    produce_sweep_potts_tn<L, RD, 1>(g, wid, a.rk, lat, a.pstride, (uint32_t)a.q, ring_u, ring_c,
-                                                     ring_op, full, empty, k, bad, -1, sTH, Hb, a.B, F, since);
-                else
-                    produce_sweep_potts_tn<L, RD, 2>(g, wid, a.rk, lat, a.pstride, (uint32_t)a.q, ring_u, ring_c,
-                                                     ring_op, full, empty, k, bad, -1, sTH, Hb, a.B, F, since);
-            } else if (consumer && active) {
-                unsigned na = 0;
-                if (a.record == 0)
-                    potts_sweep_tc<L, RD, 0>(lat, a.pstride, bR, sTH, ring_u, ring_c, ring_op, sU, full, empty, k, bad,
-                                             na, g, wid, a.key0, a.key1, a.T, Hb);
-                else
-                    potts_sweep_tc<L, RD, 1>(lat, a.pstride, bR, sTH, ring_u, ring_c, ring_op, sU, full, empty, k, bad,
-                                             na, g, wid, a.key0, a.key1, a.T, Hb);
-                nacc += na;
-                tunnel_step(bR, r_lo, r_hi, tst, ev);
-            } else if (consumer && !some) {
-#pragma unroll 1
-                for (int y = 0; y < L; ++y) {
-                    const int slot = k % RD;
-                    if (!bad && !mbar_wait(&full[slot], (unsigned)((k / RD) & 1))) bad = true;
-                    mbar_arrive(&empty[slot]);
-                    ++k;
-                }
+            for (int64_t r = 0; r < nsw * L; ++r) {
+                const int slot = k % RD;
+                if (!bad && !mbar_wait(&full[slot], (unsigned)((k / RD) & 1))) bad = true;
+                mbar_arrive(&empty[slot]);
+                ++k;
             }
+        } else if (consumer && active) {
+            if (a.record == 0)
+                consume_potts_tn<L, RD, 0>(nsw, g, lat, a.pstride, bR, sTH, ring_u, ring_c, ring_op, sU, full, empty, k, bad,
+                                           nacc, r_lo, r_hi, tst, ev, wid, a.key0, a.key1, a.T, Hb);
+            else
+                consume_potts_tn<L, RD, 1>(nsw, g, lat, a.pstride, bR, sTH, ring_u, ring_c, ring_op, sU, full, empty, k, bad,
+                                           nacc, r_lo, r_hi, tst, ev, wid, a.key0, a.key1, a.T, Hb);
         }
         __syncthreads();
         for (int b = tid; b < a.B; b += blockDim.x) {
@@ -1101,12 +1244,12 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
 }
 
 template <int L, int RD>
-// At most 64 walkers (256 threads) a block: the L = 48 and 64 forms need more than the 128
+// At most 64 walkers (384 threads) a block: the L = 48 and 64 forms need more than the 128
 // registers a thread that 512-thread blocks would leave.
-__global__ void __launch_bounds__(kCodeWarpsPerWalkerWarp * 64, 1) k_sweep_potts_tn(const SpinSweepArgs a)
+__global__ void __launch_bounds__(potts_threads(2), 1) k_sweep_potts_tn(const SpinSweepArgs a)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    sweep_block_tnp<L, RD>(a, blockIdx.x * (blockDim.x / kCodeWarpsPerWalkerWarp), blockIdx.x, smem);
+    sweep_block_tnp<L, RD>(a, blockIdx.x * (blockDim.x == (unsigned)potts_threads(2) ? 64 : 32), blockIdx.x, smem);
 }
 
 static size_t potts_tn_smem_bytes(int L, int RD, int B, int walkers_per_block)
@@ -1170,7 +1313,7 @@ static cudaError_t launch_one_tnp(const SpinSweepArgs &a, int block, cudaStream_
     cudaError_t e = cudaFuncSetAttribute(k_sweep_potts_tn<L, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    k_sweep_potts_tn<L, RD><<<nblk, kCodeWarpsPerWalkerWarp * block, smem, s>>>(a);
+    k_sweep_potts_tn<L, RD><<<nblk, potts_threads(block / 32), smem, s>>>(a);
     return cudaGetLastError();
 }
 
