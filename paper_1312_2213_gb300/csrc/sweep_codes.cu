@@ -500,18 +500,20 @@ __device__ __forceinline__ uint32_t bytes_to_nibs(uint32_t w0, uint32_t w1)  // 
 // the multiply and logic pipes of a scheduler sustain a Philox block in 88 cycles, so production (not
 // the chain) bounds the blocks of two walker warps and is spread over more warps than the Ising
 // form's.  The block has 12 warps for two walker warps, 8 for one, warp w on scheduler w mod 4:
-//   ncw = 2: [C0, C1, P0.0, P1.0,  P0.3, P1.3, P0.1, P1.1,  -, -, P0.2, P1.2]
+//   ncw = 2: [C0, C1, P0.0, P1.0,  P0.3, P1.3, P0.1, P1.1,  P0.4, P1.4, P0.2, P1.2]
 //   ncw = 1: [C0, P0.0, P0.1, P0.2,  -, P0.3, P0.4, P0.5]
-// so a consumer shares its scheduler with one of its producers or with none.
+// so a consumer shares its scheduler with one or two of its producers or with none.
 // Where the ring has four rows (L <= 32) four producers take whole rows in turn (produce_potts_rows).
 // With two rows (L = 48 and 64) all work on the same row: parts 0..n-1 own contiguous groups of four
 // sites, and a part beyond the first draws the block of the site left of its own once more.
-// Cycles a site with three producers on words of every row / as described: q = 8 L = 32, 8192
-// walkers 72.7 / 66.1 (4096 walkers 60.2 / 55.8), L = 24 77.6 / 66.9, L = 16 90.0 / 69.3, L = 8
-// 127 / 74; q = 10 L = 64, 4864 walkers or fewer 63.4 / 60.2, 8192 unchanged at 81 (five parts: 84).
+// Cycles a site with three producers on words of every row / as described (the consumer's unrolled
+// loop included, which pays since all producers run one code): q = 8 L = 32, 8192 walkers 72.7 / 57.8
+// (4096 walkers 60.2 / 47.6), L = 24 77.6 / 61.0, L = 16 90.0 / 63.9 (q = 10, 2048 walkers 71.3 / 52.8),
+// L = 8 127 / 74; q = 10 L = 48, 2048 walkers 56.1 / 48.9; L = 64, 8192 walkers 81.5 / 77.6 (four parts
+// 81.4: production bounds it, two rows being all that fits beside the table), 4096 walkers 63.4 / 54.0.
 __host__ __device__ constexpr int potts_parts(int L, int ncw)  // parts with work
 {
-    return ncw == 2 ? (L / 4 < 4 ? L / 4 : 4) : (L / 4 < 6 ? L / 4 : 6);
+    return ncw == 2 ? (L / 4 < 5 ? L / 4 : 5) : (L / 4 < 6 ? L / 4 : 6);
 }
 __host__ __device__ constexpr int potts_part_groups(int L, int ncw, int part)
 {
@@ -929,8 +931,9 @@ __device__ __forceinline__ void potts_redo_row(uint32_t *__restrict__ lat, int p
 
 // The consumer's rows of nsw sweeps, joined as in consume_tn: the next row is asked for two byte words
 // ahead, and its first site's threshold is loaded for both outcomes of the row's last.  A row is a
-// loop over its byte words (4 sites each), unrolled by two (rolled it lost 16-20 % to loop overhead
-// between the words' chains; fully unrolled, L = 48 stalled on instruction fetch), with the last
+// loop over its byte words (4 sites each), unrolled (by two it took 55.8 cycles a site at L = 32 with
+// 4096 walkers, in full 47.6; the longer rows of the split table by four: by two 60.2, in full 59.7,
+// by four 54.0), with the last
 // word, which holds the last site's right-neighbour term, peeled.  The final row above
 // lives in a per-lane shared-memory row (bytes).  With the split table there are
 // two such rows, read and written in turn (the row being decided reads one and
@@ -953,6 +956,7 @@ __device__ __forceinline__ void consume_potts_tn(int64_t nsw, uint32_t sweep0, u
     constexpr int W4 = L / 4;
     constexpr size_t S = (size_t)W4 * 32;
     static_assert(!SPLIT || L % 2 == 0, "the up rows alternate: row L - 1 must leave its values in the first");
+    constexpr int kWordUnroll = SPLIT ? 4 : W4;
     const uint4 *ring_u = (const uint4 *)ring_u_;
     const uint2 *ring_u16 = (const uint2 *)ring_u_;
     // As in the Ising consumer: 32-bit shared-window byte addresses (bB = table base + 4 RSW bin),
@@ -1030,7 +1034,7 @@ __device__ __forceinline__ void consume_potts_tn(int64_t nsw, uint32_t sweep0, u
                 return ru[j * 32];
             };
             uint32_t fprev = 0u;
-#pragma unroll 2
+#pragma unroll kWordUnroll
             for (int j = 0; j < W4 - 1; ++j) {
                 const uint2 op = opn, cd = cdn;
                 const uint4 u = words(j);
