@@ -509,6 +509,13 @@ int check_ctx(const muca_ctx *c)
     return MUCA_OK;
 }
 
+int device_flag_status(int err)
+{
+    if (err & 2) return fail(MUCA_ERR_CHECK, "a device bounds check failed (checked build); the last iterations are invalid");
+    if (err) return fail(MUCA_ERR_TIMEOUT, "a bounded device wait gave up; the last iterations are invalid");
+    return MUCA_OK;
+}
+
 // Device-side checks (bounded waits) leave a flag in the device state; every
 // call that synchronises reports it.
 int check_device_flag(muca_ctx *c)
@@ -516,8 +523,18 @@ int check_device_flag(muca_ctx *c)
     int err = 0;
     MUCA_CUDA(cudaMemcpyAsync(&err, &c->state->err, sizeof err, cudaMemcpyDeviceToHost, c->stream));
     MUCA_CUDA(cudaStreamSynchronize(c->stream));
-    if (err & 2) return fail(MUCA_ERR_CHECK, "a device bounds check failed (checked build); the last iterations are invalid");
-    if (err) return fail(MUCA_ERR_TIMEOUT, "a bounded device wait gave up; the last iterations are invalid");
+    return device_flag_status(err);
+}
+
+// The flatness flag and the error word behind it, in one copy and one wait.
+int read_flat(muca_ctx *c, int *is_flat)
+{
+    static_assert(offsetof(DevState, err) == offsetof(DevState, flat) + sizeof(int), "flat and err side by side");
+    int v[2] = {0, 0};
+    MUCA_CUDA(cudaMemcpyAsync(v, &c->state->flat, sizeof v, cudaMemcpyDeviceToHost, c->stream));
+    MUCA_CUDA(cudaStreamSynchronize(c->stream));
+    if (int rc = device_flag_status(v[1])) return rc;
+    *is_flat = v[0];
     return MUCA_OK;
 }
 
@@ -887,12 +904,7 @@ int muca_merge_and_update(muca_ctx *c, int *is_flat)
     }
     c->started = true;
     c->open = false;
-    if (is_flat) {
-        int f = 0;
-        if (int rc = d2h(c, &f, &c->state->flat, sizeof(int))) return rc;
-        *is_flat = f;
-    }
-    return MUCA_OK;
+    return is_flat ? read_flat(c, is_flat) : MUCA_OK;
 }
 
 int muca_merge_open(muca_ctx *c, uint64_t *dev_H_out)
@@ -926,12 +938,7 @@ int muca_update_with(muca_ctx *c, const uint64_t *dev_H, int *is_flat)
     }
     c->started = true;
     c->open = false;
-    if (is_flat) {
-        int f = 0;
-        if (int rc = d2h(c, &f, &c->state->flat, sizeof(int))) return rc;
-        *is_flat = f;
-    }
-    return MUCA_OK;
+    return is_flat ? read_flat(c, is_flat) : MUCA_OK;
 }
 
 int muca_set_lnW(muca_ctx *c, const double *host_lnW, int nbins)

@@ -27,7 +27,7 @@ namespace muca {
 // selects and compares; the producers alone need 36 (L = 32).  Cycles a site, 8192
 // walkers spread over all bins, before / after the column-major table, the joined
 // rows and the shorter Philox rounds: Ising L = 32 50.7 / 42.6, MUMA 50.3 / 43.5;
-// Ising L = 64 (2048 walkers) 50.9 / 48.0, L = 16 59.4 / 48.6, L = 8 (64) 74.5 / 60.0.
+// Ising L = 64 (2048 walkers) 50.9 / 42.9, L = 16 59.4 / 48.6, L = 8 (64) 74.5 / 60.0.
 template <int L, int WR>
 __device__ __forceinline__ uint32_t row_bit(const uint32_t (&r)[WR], int x)
 {
@@ -227,9 +227,12 @@ __device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ l
         return make_uint2((c.x - up4) ^ flip, (c.y - up4) ^ flip);
     };
 
+    // A row is decided in units of U sites (one word): the whole row up to L = 32, halves at L = 64,
+    // where 64 unrolled sites stalled on instruction fetch (48.0 cycles a site, 42.9 in halves).
+    constexpr int U = (L % 32 == 0) ? 32 : L, NU = L / U, WU = (U + 31) / 32;
     const int k_end = k + (int)(nsw * L);
     int bB = sbase + 4 * bR;
-    uint32_t up[WR], cur[WR], nxt[WR];
+    uint32_t up[WR], cur[WU], nxt[WU];
     uint2 cdn = make_uint2(0u, 0u);
     uint32_t T0 = 0u, T1 = 0u;
     bool accP = false;  // the site decided before
@@ -237,10 +240,9 @@ __device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ l
     if (!bad) {
         const int slot = k % kRing;
 #pragma unroll
-        for (int j = 0; j < WR; ++j) {
-            up[j] = lat[((L - 1) * WR + j) * ps];
-            nxt[j] = ring_r[slot * SR + j * 32];
-        }
+        for (int j = 0; j < WR; ++j) up[j] = lat[((L - 1) * WR + j) * ps];
+#pragma unroll
+        for (int j = 0; j < WU; ++j) nxt[j] = ring_r[slot * SR + j * 32];
         const uint32_t ua0[1] = {up[0] ^ nxt[0]};
         cdn = settle(ring_c[slot * SC], nibble_fours<1>(ua0, 0));
         T0 = T1 = th(at(cdn.x, 0, bB));
@@ -251,51 +253,57 @@ __device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ l
         // two rows an iteration from L = 32 up (2-4 % there; L = 16 rows are short enough that the
         // larger body costs more than the loop overhead it saves)
         constexpr int kRowUnroll = (L >= 32) ? 2 : 1;
+        uint32_t s0 = 0u;  // site 0 of the row, decided
 #pragma unroll kRowUnroll
-        for (int y = 0; y < L; ++y) {
-            const int slot = k % kRing, slot_n = (k + 1) % kRing;
-            const uint4 *ru = ring_u + slot * SU;
-            const uint2 *rc = ring_c + slot * SC;
-            uint32_t ua[WR], old[WR];
+        for (int yu = 0; yu < L * NU; ++yu) {
+            const int y = yu / NU, h = yu % NU;  // row and unit (constants of the unrolled pair at NU = 2)
+            const bool row_end = h == NU - 1;
+            const int slot = k % kRing, slot_n = row_end ? (k + 1) % kRing : slot;
+            const uint4 *ru = ring_u + slot * SU + (size_t)h * (U / 4) * 32;
+            const uint2 *rc = ring_c + slot * SC + (size_t)h * (U / 4) * 32;
+            uint32_t ua[WU], old[WU];
 #pragma unroll
-            for (int j = 0; j < WR; ++j) {
+            for (int j = 0; j < WU; ++j) {
                 old[j] = cur[j] = nxt[j];
-                ua[j] = up[j] ^ cur[j];  // up neighbour anti-aligned
+                ua[j] = up[h * WU + j] ^ cur[j];  // up neighbour anti-aligned
             }
-            const uint32_t sLast = row_bit<L, WR>(cur, L - 1);
+            const uint32_t sLast = row_bit<U, WU>(cur, U - 1);
             uint2 cd = cdn, cnext = cdn;
             uint4 u = make_uint4(0u, 0u, 0u, 0u);
             uint32_t mv = 0u;   // MUMA: the four sites' moves in bytes, +-4
             bool next = false;  // the next row is there
 #pragma unroll
-            for (int x = 0; x < L; ++x) {
+            for (int x = 0; x < U; ++x) {
                 const int j4 = x & 3;
                 if (j4 == 0) {
                     u = ru[(x / 4) * 32];
                     cd = cdn;
                     // s = -1 (bit set): one bin up, else one down; 0xFC = -4, 0xFC ^ 0xF8 = 4
-                    if (SYS == kMuma) mv = (nibble_fours<WR>(old, x) * 0x3Eu) ^ 0xFCFCFCFCu;
-                    if (x + 4 < L) cdn = settle(rc[(x / 4 + 1) * 32], nibble_fours<WR>(ua, x + 4));
-                    if (x + 8 == L) next = mbar_try(&full[slot_n], (unsigned)(((k + 1) / kRing) & 1));
-                    if (x + 4 == L) {
-                        // the next row; behind the last one (or a wait that gave up) an earlier row's codes
+                    if (SYS == kMuma) mv = (nibble_fours<WU>(old, x) * 0x3Eu) ^ 0xFCFCFCFCu;
+                    if (x + 4 < U) cdn = settle(rc[(x / 4 + 1) * 32], nibble_fours<WU>(ua, x + 4));
+                    if (x + 8 == U && row_end) next = mbar_try(&full[slot_n], (unsigned)(((k + 1) / kRing) & 1));
+                    if (x + 4 == U) {
+                        // the next unit; behind the last row (or a wait that gave up) an earlier row's codes
                         // are read and not used
-                        if (!next && !(sw + 1 == nsw && y == L - 1))
+                        if (row_end && !next && !(sw + 1 == nsw && y == L - 1))
                             bad = !mbar_wait(&full[slot_n], (unsigned)(((k + 1) / kRing) & 1));
+                        const int hn = row_end ? 0 : h + 1;
 #pragma unroll
-                        for (int j = 0; j < WR; ++j) nxt[j] = ring_r[slot_n * SR + j * 32];
-                        cnext = ring_c[slot_n * SC];
+                        for (int j = 0; j < WU; ++j) nxt[j] = ring_r[slot_n * SR + (hn * WU + j) * 32];
+                        cnext = ring_c[slot_n * SC + (size_t)hn * (U / 4) * 32];
                     }
                 }
-                if (x == L - 2) {
+                if (h == 0 && x == 4) s0 = row_bit<U, WU>(cur, 0);
+                if (row_end && x == U - 2) {
                     // the last site's right neighbour is site 0 of this row, final by now (its code is the
                     // top byte, so nothing is borrowed from)
-                    const uint32_t ra = (row_bit<L, WR>(cur, 0) ^ sLast) << 26;
+                    const uint32_t ra = (s0 ^ sLast) << 26;
                     cd.x -= ra;
                     cd.y -= ra;
                 }
-                if (x == L - 1) {
-                    const uint32_t ua0[1] = {cur[0] ^ nxt[0]};  // (sites 0..3 are final)
+                if (x == U - 1) {
+                    // (the first four sites of this row's first unit, or of the row above's next unit)
+                    const uint32_t ua0[1] = {((NU == 1) ? cur[0] : up[row_end ? 0 : h + 1]) ^ nxt[0]};
                     cdn = settle(cnext, nibble_fours<1>(ua0, 0));
                 }
                 const uint32_t uw = word_of(u, j4);
@@ -318,14 +326,16 @@ __device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ l
                 accP = acc;
             }
 #pragma unroll
-            for (int j = 0; j < WR; ++j) {
-                lat[(y * WR + j) * ps] = cur[j];
+            for (int j = 0; j < WU; ++j) {
+                lat[(y * WR + h * WU + j) * ps] = cur[j];
                 na += (unsigned)__popc(old[j] ^ cur[j]);
-                up[j] = cur[j];
+                up[h * WU + j] = cur[j];
             }
-            mbar_arrive(&empty[slot]);  // after the row is stored: the producer reads it later
-            ++k;
-            if (bad) break;
+            if (row_end) {
+                mbar_arrive(&empty[slot]);  // after the row is stored: the producer reads it later
+                ++k;
+                if (bad) break;
+            }
         }
         nacc += na;
         if (bad) break;
@@ -351,6 +361,23 @@ __host__ __device__ constexpr size_t tn_ring_bytes(int L)
     return (size_t)kRing * ((size_t)(L / 4) * 32 * 16 + (size_t)(L / 4) * 32 * 8 + (size_t)((L + 31) / 32) * 32 * 4);
 }
 
+// put(i, T[i]) for i < n by the whole block, eight loads a thread in flight (one after the other they
+// took an L2 round trip each: 46,000 thresholds of q-Potts at L = 48 by 256 threads).
+template <class PUT>
+__device__ __forceinline__ void stage_table(const uint32_t *__restrict__ T, int n, PUT put)
+{
+    constexpr int U = 8;
+    int i = threadIdx.x;
+    for (; i + (U - 1) * (int)blockDim.x < n; i += U * blockDim.x) {
+        uint32_t t[U];
+#pragma unroll
+        for (int e = 0; e < U; ++e) t[e] = T[i + e * (int)blockDim.x];
+#pragma unroll
+        for (int e = 0; e < U; ++e) put(i + e * (int)blockDim.x, t[e]);
+    }
+    for (; i < n; i += blockDim.x) put(i, T[i]);
+}
+
 template <int SYS, int L>
 __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, int slot_id, uint32_t *smem)
 {
@@ -374,10 +401,10 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
     unsigned long long *full = bars + (size_t)pair * 2 * kRing, *empty = full + kRing;
 
     const int tid = threadIdx.x;
-    for (int i = tid; i < NB * C; i += blockDim.x) {
+    stage_table(a.T, NB * C, [&](int i, uint32_t t) {
         const int b = i / C, c = i - (i / C) * C;
-        sTH[c * NB + b] = a.T[i];
-    }
+        sTH[c * NB + b] = t;
+    });
     for (int b = tid; b < NB; b += blockDim.x) sTH[C * NB + b] = 0u;
     // the rings' codes start on a middle column, so that codes read ahead of a row that never came
     // (a wait that gave up, the end of the last sweep) still address the table
@@ -1155,15 +1182,12 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
     const int tid = threadIdx.x;
     if (R::split) {  // halfword rows: 9 upper halves (split_hi), the 16-bit counter
         uint16_t *h = (uint16_t *)smem;
-        for (int i = tid; i < a.B * 10; i += blockDim.x) {
-            const int b = i / 10, c = i - (i / 10) * 10;
-            h[i] = (c < C) ? split_hi(a.T[b * C + c]) : (uint16_t)0;
-        }
+        stage_table(a.T, a.B * C, [&](int i, uint32_t t) { h[i + i / C] = split_hi(t); });
+        for (int b = tid; b < a.B; b += blockDim.x) h[b * 10 + C] = (uint16_t)0;
     } else {
-        for (int i = tid; i < a.B * RS; i += blockDim.x) {
-            const int b = i / RS, c = i - (i / RS) * RS;
-            sTH[i] = (c < C) ? a.T[b * C + c] : 0u;
-        }
+        stage_table(a.T, a.B * C, [&](int i, uint32_t t) { sTH[i + (RS - C) * (i / C)] = t; });
+        for (int b = tid; b < a.B; b += blockDim.x)
+            for (int c = C; c < RS; ++c) sTH[b * RS + c] = 0u;
     }
     // as in the Ising form: codes read ahead of a row that never came address the table
     for (int i = tid; i < ncw * RD * (int)S; i += blockDim.x) {
