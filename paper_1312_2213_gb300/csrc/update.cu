@@ -14,6 +14,8 @@
 // All binary64 arithmetic of the recursion and the thresholds uses explicit
 // round-to-nearest intrinsics (this file is also built with -fmad=false), so
 // the results are the same bits on every run and every compiler.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 
 #include "muca_device.cuh"
@@ -541,12 +543,42 @@ __global__ void k_unpack_spins(int system, int L, int p, int pstride, const uint
 
 // Eq. (2) with O a function of the binned variable; ln Omega(b) = ln H(b) -
 // ln W(b), W being the weights H was sampled with.  Fixed-order tree
-// reductions in one block, so repeated calls give identical results.
-__global__ void __launch_bounds__(1024) k_reweight(const UpdateArgs a, double beta, double *out4, double *lnP)
+// reductions, so repeated calls give identical results.
+// One log and three exponentials a bin in binary64, of which an SM does two lanes a clock: 8193 bins
+// on one SM took 214 us.  So a cluster of kReweightCtas blocks works as one block of 1024 threads
+// would, thread t on bins t, t + 1024, ...: the partial results of all threads go to every block through
+// distributed shared memory, and each makes the same tree of 1024 (the sums keep their order).
+constexpr int kReweightCtas = 8, kReweightThreads = 128, kReweightAll = kReweightCtas * kReweightThreads;
+
+template <class OP>
+__device__ double reweight_reduce(double v, double *red, OP op)
 {
-    extern __shared__ double sx[];  // B values of x_b
-    __shared__ double red[1024];
-    const int tid = threadIdx.x, bs = blockDim.x, B = a.B, N = a.N;
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int t = (int)cl.block_rank() * kReweightThreads + threadIdx.x;
+    cl.sync();  // the last reduction has been read everywhere
+    for (int r = 0; r < kReweightCtas; ++r) cl.map_shared_rank(red, r)[t] = v;
+    cl.sync();
+    for (int s = kReweightAll / 2; s > 0; s >>= 1) {
+        for (int i = threadIdx.x; i < s; i += kReweightThreads) red[i] = op(red[i], red[i + s]);
+        __syncthreads();
+    }
+    return red[0];
+}
+
+__global__ void __cluster_dims__(kReweightCtas, 1, 1) __launch_bounds__(kReweightThreads)
+    k_reweight(const UpdateArgs a, double beta, double *out4, double *lnP)
+{
+    extern __shared__ double sx[];  // this block's values of x_b: bin t + 1024 i at 128 i + its thread
+    __shared__ double red[kReweightAll];
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = rank * kReweightThreads + threadIdx.x, bs = kReweightAll, B = a.B, N = a.N;
+    auto own = [](int b) { return b / kReweightAll * kReweightThreads + b % kReweightThreads; };
+    auto energy = [&](int b) {
+        if (a.system == kPolymer) return a.e_lo + a.bin_w * (b + 0.5);
+        return (a.system == kIsing) ? (double)(4 * b - 2 * N) : (double)(b - 2 * N);
+    };
+    auto plus = [](double x, double y) { return x + y; };
+    auto larger = [](double x, double y) { return fmax(x, y); };
     const double NEG_INF = kNegInf;
     double m = NEG_INF;
     for (int b = tid; b < B; b += bs) {
@@ -554,91 +586,43 @@ __global__ void __launch_bounds__(1024) k_reweight(const UpdateArgs a, double be
         const unsigned long long h = a.H[b];
         if (a.reach[b] && h) {
             const double lnOmega = log((double)h) - a.lnW_sampled[b];
-            if (a.system == kMuma) {
-                x = lnOmega;
-            } else if (a.system == kPolymer) {
-                x = lnOmega - beta * (a.e_lo + a.bin_w * (b + 0.5));
-            } else {
-                const double E = (a.system == kIsing) ? (double)(4 * b - 2 * N) : (double)(b - 2 * N);
-                x = lnOmega - beta * E;
-            }
+            x = (a.system == kMuma) ? lnOmega : lnOmega - beta * energy(b);
         }
-        sx[b] = x;
+        sx[own(b)] = x;
         m = fmax(m, x);
     }
-    red[tid] = m;
-    __syncthreads();
-    for (int s = bs / 2; s > 0; s >>= 1) {
-        if (tid < s) red[tid] = fmax(red[tid], red[tid + s]);
-        __syncthreads();
-    }
-    m = red[0];
-    __syncthreads();
+    m = reweight_reduce(m, red, larger);
     double z = 0.0;
     for (int b = tid; b < B; b += bs)
-        if (sx[b] > NEG_INF) z += exp(sx[b] - m);
-    red[tid] = z;
-    __syncthreads();
-    for (int s = bs / 2; s > 0; s >>= 1) {
-        if (tid < s) red[tid] += red[tid + s];
-        __syncthreads();
-    }
-    const double lse = m + log(red[0]);
-    __syncthreads();
+        if (sx[own(b)] > NEG_INF) z += exp(sx[own(b)] - m);
+    const double lse = m + log(reweight_reduce(z, red, plus));
     double a1 = 0.0, a2 = 0.0;
     for (int b = tid; b < B; b += bs) {
-        const double x = sx[b];
+        const double x = sx[own(b)];
         const double lp = (x > NEG_INF) ? x - lse : NEG_INF;
         if (lnP) lnP[b] = lp;
         if (x > NEG_INF) {
             const double P = exp(lp);
-            double v;
-            if (a.system == kMuma) v = fabs((double)(2 * b - N));
-            else if (a.system == kPolymer) v = a.e_lo + a.bin_w * (b + 0.5);
-            else v = (a.system == kIsing) ? (double)(4 * b - 2 * N) : (double)(b - 2 * N);
+            const double v = (a.system == kMuma) ? fabs((double)(2 * b - N)) : energy(b);
             a1 += P * v;
             a2 += P * v * v;
         }
     }
-    __shared__ double red2[1024];
-    red[tid] = a1;
-    red2[tid] = a2;
-    __syncthreads();
-    for (int s = bs / 2; s > 0; s >>= 1) {
-        if (tid < s) {
-            red[tid] += red[tid + s];
-            red2[tid] += red2[tid + s];
-        }
-        __syncthreads();
-    }
-    a1 = red[0];
-    a2 = red2[0];
+    a1 = reweight_reduce(a1, red, plus);
+    a2 = reweight_reduce(a2, red, plus);
     // polymer: log-sum-exp of ln Omega itself (the normalisation of ln Z)
     double lnNorm = 0.0;
     if (a.system == kPolymer) {
-        __syncthreads();
         double m2 = NEG_INF;
         for (int b = tid; b < B; b += bs)
-            if (sx[b] > NEG_INF) m2 = fmax(m2, sx[b] + beta * (a.e_lo + a.bin_w * (b + 0.5)));
-        red2[tid] = m2;
-        __syncthreads();
-        for (int st = bs / 2; st > 0; st >>= 1) {
-            if (tid < st) red2[tid] = fmax(red2[tid], red2[tid + st]);
-            __syncthreads();
-        }
-        m2 = red2[0];
-        __syncthreads();
+            if (sx[own(b)] > NEG_INF) m2 = fmax(m2, sx[own(b)] + beta * energy(b));
+        m2 = reweight_reduce(m2, red, larger);
         double z2 = 0.0;
         for (int b = tid; b < B; b += bs)
-            if (sx[b] > NEG_INF) z2 += exp(sx[b] + beta * (a.e_lo + a.bin_w * (b + 0.5)) - m2);
-        red2[tid] = z2;
-        __syncthreads();
-        for (int st = bs / 2; st > 0; st >>= 1) {
-            if (tid < st) red2[tid] += red2[tid + st];
-            __syncthreads();
-        }
-        lnNorm = m2 + log(red2[0]);
+            if (sx[own(b)] > NEG_INF) z2 += exp(sx[own(b)] + beta * energy(b) - m2);
+        lnNorm = m2 + log(reweight_reduce(z2, red, plus));
     }
+    auto x_of = [&](int b) -> double { return cl.map_shared_rank(sx, b % kReweightAll / kReweightThreads)[own(b)]; };
     if (tid == 0) {
         if (a.system == kPolymer) {
             out4[0] = a1;
@@ -650,16 +634,17 @@ __global__ void __launch_bounds__(1024) k_reweight(const UpdateArgs a, double be
             out4[1] = a2 / ((double)N * N);
             out4[2] = a.beta * N * (out4[1] - out4[0] * out4[0]);
             const int b0 = N / 2, bm = N;
-            out4[3] = (sx[b0] > NEG_INF && sx[bm] > NEG_INF) ? sx[b0] - sx[bm] : __longlong_as_double(0x7ff8000000000000LL);
+            out4[3] = (x_of(b0) > NEG_INF && x_of(bm) > NEG_INF) ? x_of(b0) - x_of(bm) : __longlong_as_double(0x7ff8000000000000LL);
         } else {
             out4[0] = a1;
             out4[1] = a2;
             out4[2] = beta * beta * (a2 - a1 * a1) / N;
             const double g0 = (a.system == kIsing) ? 2.0 : (double)a.q;
-            if (sx[0] > NEG_INF) out4[3] = lse + log(g0) - (sx[0] - beta * (double)(2 * N));
+            if (x_of(0) > NEG_INF) out4[3] = lse + log(g0) - (x_of(0) - beta * (double)(2 * N));
             else out4[3] = __longlong_as_double(0x7ff8000000000000LL);
         }
     }
+    cl.sync();  // no block leaves while its shared memory may be read
 }
 
 __global__ void k_det_math(int fn, const double *in, double *out, long long n)
@@ -767,10 +752,9 @@ cudaError_t launch_unpack_spins(int system, int L, int p, int pstride, const uin
 
 cudaError_t launch_reweight(const UpdateArgs &a, double beta, double *out4, double *lnP, cudaStream_t s)
 {
-    const size_t smem = (size_t)a.B * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_reweight, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_reweight<<<1, 1024, smem, s>>>(a, beta, out4, lnP);
+    // (at most 12288 bins: 12 KB a block, within what a launch may ask for without an attribute)
+    const size_t smem = (size_t)((a.B + kReweightAll - 1) / kReweightAll) * kReweightThreads * sizeof(double);
+    k_reweight<<<kReweightCtas, kReweightThreads, smem, s>>>(a, beta, out4, lnP);
     return cudaGetLastError();
 }
 
