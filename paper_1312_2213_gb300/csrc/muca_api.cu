@@ -325,6 +325,16 @@ cudaError_t launch_system_sweep(const muca_ctx *c, const SpinSweepArgs &a, cudaS
     return launch_spin_sweep(c->system, c->L, a, block, s);
 }
 
+// Shared memory of one block of that launch.
+size_t system_sweep_smem(const muca_ctx *c, int block)
+{
+    if (c->pipeline >= 2 && spin_sweep_tn_fits(c->system, c->L, c->B, block))
+        return spin_sweep_tn_smem_bytes(c->system, c->L, c->B, block);
+    if (c->pipeline >= 1 && spin_sweep_pc_fits(c->system, c->L, c->B, block))
+        return spin_sweep_pc_smem_bytes(c->system, c->L, c->B, block);
+    return spin_sweep_smem_bytes(c->system, c->B);
+}
+
 PolyArgs poly_args(const muca_ctx *c, int64_t sweeps)
 {
     PolyArgs a{};
@@ -1341,26 +1351,70 @@ struct muca_batch {
     bool tiles_fit = true;             // every system's table fits the form-0 kernel's shared memory
     std::vector<int64_t> sw;           // per-system sweeps of an iteration (empty: the run's argument)
     std::vector<int> blk;              // form 1: each system's walkers per block in this batch
+    int nsm = 152;                     // SMs of the device
     std::vector<int64_t> g_sw;         // per-system sweeps the captured graph was made with
 };
 
 namespace {
 
-// Systems heaviest first (sites x sweeps, Potts sites counted 2.5 times), so that their
-// blocks or tiles start in the first wave.
-std::vector<int> batch_order(const muca_batch *b)
+// A system's sweep in units of an Ising attempt of its form: a q-Potts site takes 1.2 times as long in
+// the code form (48 against 43 cycles at L = 48 / 64), 2.5 times in the one-warp form of the tiles; a
+// polymer bead attempt counts as about 40 (its pair terms).
+double batch_cost(const muca_batch *b, int i, int form)
+{
+    const muca_ctx *c = b->sys[i];
+    const double w = c->system == kPotts ? (form == 1 ? 1.2 : 2.5) : (c->system == kPolymer ? 40.0 : 1.0);
+    return (double)c->N * w * (b->sw.empty() ? 1.0 : (double)b->sw[i]);
+}
+
+// Systems heaviest first, so that their blocks or tiles start in the first wave.
+std::vector<int> batch_order(const muca_batch *b, int form)
 {
     const int n = (int)b->sys.size();
     std::vector<int> order(n);
     for (int i = 0; i < n; ++i) order[i] = i;
-    auto cost = [&](int i) {  // a polymer bead attempt counted as ~40 spin attempts (its pair terms)
-        const muca_ctx *c = b->sys[i];
-        const double w = c->system == kPotts ? 2.5 : (c->system == kPolymer ? 40.0 : 1.0);
-        return (double)c->N * w * (b->sw.empty() ? 1.0 : (double)b->sw[i]);
-    };
     for (int i = 1; i < n; ++i)
-        for (int j = i; j > 0 && cost(order[j]) > cost(order[j - 1]); --j) std::swap(order[j], order[j - 1]);
+        for (int j = i; j > 0 && batch_cost(b, order[j], form) > batch_cost(b, order[j - 1], form); --j)
+            std::swap(order[j], order[j - 1]);
     return order;
+}
+
+// Form 1: which of the batch's streams each system's sweep goes to, by its place in the order.  A
+// system whose blocks find SMs beside the heavier ones' gets a stream of its own; when the SMs are
+// taken, it queues behind the system that ends first.  (With every system on a stream of its own the
+// light systems' small blocks could be placed first, in a graph above all, and an L = 64 block, which
+// takes an SM's whole shared memory, had to wait for them: 27 ms for 20 iterations of 10 sweeps of the
+// mix as a graph, where the L = 64 chain and the updates take 19.)  Polymers fill the GPU
+// by themselves and gain from lying side by side, so each keeps its own stream.
+std::vector<int> batch_lanes(const muca_batch *b)
+{
+    const int n = (int)b->sys.size();
+    std::vector<int> lane(n);
+    std::vector<double> end;
+    double free_sms = (double)b->nsm;
+    for (int r = 0; r < n; ++r) {
+        const int i = b->order[r];
+        const muca_ctx *c = b->sys[i];
+        double sms = 0.0;
+        if (c->system != kPolymer) {
+            const size_t smem = std::max(system_sweep_smem(c, b->blk[i]), (size_t)1);
+            const int per_sm = std::max(1, std::min((int)(kMaxSmem / smem), 4));
+            sms = (double)((c->p + b->blk[i] - 1) / b->blk[i]) / per_sm;
+        }
+        // (a system that mostly fits starts too: its last blocks follow the first that end)
+        if (end.empty() || sms <= 1.5 * free_sms) {
+            lane[r] = (int)end.size();
+            end.push_back(batch_cost(b, i, 1));
+            free_sms -= sms;
+        } else {
+            int best = 0;
+            for (int l = 1; l < (int)end.size(); ++l)
+                if (end[l] < end[best]) best = l;
+            lane[r] = best;
+            end[best] += batch_cost(b, i, 1);
+        }
+    }
+    return lane;
 }
 
 int batch_enqueue_iteration(muca_batch *b, int64_t sweeps)
@@ -1369,17 +1423,22 @@ int batch_enqueue_iteration(muca_batch *b, int64_t sweeps)
     if (b->form == 1) {
         MUCA_CUDA(cudaEventRecord(b->ev_fork, b->stream));
         // heaviest first, so that their blocks take the SMs before the light systems' blocks
-        for (int i : b->order) {
-            MUCA_CUDA(cudaStreamWaitEvent(b->sub[i], b->ev_fork, 0));
+        const std::vector<int> lane = batch_lanes(b);
+        std::vector<char> forked(n, 0);
+        for (int r = 0; r < n; ++r) {
+            const int i = b->order[r];
+            const cudaStream_t sub = b->sub[lane[r]];
+            if (!forked[lane[r]]) MUCA_CUDA(cudaStreamWaitEvent(sub, b->ev_fork, 0));
+            forked[lane[r]] = 1;
             muca_ctx *c = b->sys[i];
             if (c->system == kPolymer) {  // as muca_iterate: the sweeps, then the energies from scratch
                 const PolyArgs pa = poly_args(c, b->h_sys[i].sweeps);
-                MUCA_CUDA(launch_poly_sweep(pa, c->block_set ? c->block : 0, b->sub[i]));
-                MUCA_CUDA(launch_poly_energy(pa, 1, b->sub[i]));
+                MUCA_CUDA(launch_poly_sweep(pa, c->block_set ? c->block : 0, sub));
+                MUCA_CUDA(launch_poly_energy(pa, 1, sub));
             } else {
-                MUCA_CUDA(launch_system_sweep(c, b->h_own[i], b->sub[i], b->blk[i]));
+                MUCA_CUDA(launch_system_sweep(c, b->h_own[i], sub, b->blk[i]));
             }
-            MUCA_CUDA(cudaEventRecord(b->ev_join[i], b->sub[i]));
+            MUCA_CUDA(cudaEventRecord(b->ev_join[i], sub));
         }
         for (int i = 0; i < n; ++i) MUCA_CUDA(cudaStreamWaitEvent(b->stream, b->ev_join[i], 0));
     } else {
@@ -1427,7 +1486,7 @@ int muca_batch_create(muca_ctx *const *systems, int n, muca_batch **out)
         delete b;
         return fail(MUCA_ERR_CUDA, "muca_batch_create: cannot create stream/events");
     }
-    const std::vector<int> order = batch_order(b);
+    const std::vector<int> order = batch_order(b, 0);  // of the tiles
     // Form 1 runs each system in its own block size, except that q-Potts systems given 32-walker
     // blocks because every block would have an SM to itself go back to 64 when the batch's
     // systems together have more such blocks than the GPU has SMs (they share the SMs then).
@@ -1438,6 +1497,7 @@ int muca_batch_create(muca_ctx *const *systems, int n, muca_batch **out)
         const bool shared = cudaGetDevice(&dev) == cudaSuccess &&
                             cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
                             blocks32 > nsm;
+        if (nsm > 0) b->nsm = nsm;
         b->blk.resize(n);
         for (int i = 0; i < n; ++i) {
             const muca_ctx *c = b->sys[i];
@@ -1466,7 +1526,7 @@ int muca_batch_create(muca_ctx *const *systems, int n, muca_batch **out)
     for (int i : order)
         if (b->sys[i]->system != kPolymer)
             for (int w0 = 0; w0 < b->sys[i]->p; w0 += b->block) tiles.push_back(make_int2(i, w0));
-    b->order = order;
+    b->order = batch_order(b, 1);
     b->ntiles = (int)tiles.size();
     b->h_sys.resize(n);
     const size_t sz_sys = align_up(sizeof(SpinSweepArgs) * n), sz_tiles = align_up(sizeof(int2) * tiles.size()),
@@ -1617,9 +1677,9 @@ int muca_batch_set_sweeps(muca_batch *b, const int64_t *sweeps, int n)
     }
     MUCA_CUDA(cudaStreamSynchronize(b->stream));  // the tile list may be in use
     b->sw = sw;
-    b->order = batch_order(b);
+    b->order = batch_order(b, 1);
     std::vector<int2> tiles;
-    for (int i : b->order)
+    for (int i : batch_order(b, 0))
         if (b->sys[i]->system != kPolymer)
             for (int w0 = 0; w0 < b->sys[i]->p; w0 += b->block) tiles.push_back(make_int2(i, w0));
     if (!tiles.empty())
