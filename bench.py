@@ -46,12 +46,11 @@ N = L * L
 # (10 rounds x 4 ops / 4 = 10), neighbour bits and count 8, table column and address 2,
 # threshold load 1, integer compare 2, flip/select 3, bin update 2, histogram atomic 1, loop 1.
 INSTR_PER_ATTEMPT = 30
-# Cycles an attempt of one walker's chain in this design's sweep with its scheduler to itself
-# (one consumer warp an SM, p = 4096 in 32-walker blocks, measured on GB300 at 2.07 GHz): Ising
-# 42.9, multimagnetic 49.1, averaged over the step's two systems.  p f / CHAIN_CYCLES bounds the
+# Cycles an attempt of one walker's chain in this design's sweep inside a row, from clock reads in
+# the Ising consumer (L = 32, GB300 at 2.07 GHz).  p f / CHAIN_CYCLES bounds the
 # attempts/s of the sweep kernel, and its rate is reported against it as well (the issue-peak
 # fraction counts all schedulers, which one chain per walker cannot fill at p = 8192).
-CHAIN_CYCLES = (42.9 + 49.1) / 2
+CHAIN_CYCLES = 39.7
 # DRAM bytes (read + write) per launch of the timed sweep kernel, from one ncu capture of the current
 # k_sweep_spin_tn build (dram__bytes_read.sum + dram__bytes_write.sum; mean of the Ising and MUMA
 # launches: 1.25 MB and 2.17 MB read, nothing written).  It is the walker state and does not grow
@@ -520,7 +519,7 @@ def run_ours(args):
     kernel_rate = P * sweeps * N / (sweep_ms / 1e3)
     roofline["chain_bound"] = {"cycles_per_attempt": CHAIN_CYCLES, "attempts_per_s": chain_rate,
                                "achieved_attempts_per_s": kernel_rate, "frac": kernel_rate / chain_rate,
-                               "basis": "p x f_SM / cycles of one walker's chain with its scheduler to itself"}
+                               "basis": "p x f_SM / cycles of one walker's chain inside a row"}
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "u32", "data": "synthetic",

@@ -89,10 +89,11 @@ int muca_init_ex(muca_ctx **out, int system, int L_or_N, int q, int p, uint64_t 
  *                 multiple of 32; default 64, or 32 where only that fits the
  *                 code form, and 32 for q-Potts when p <= 32 x the SM count;
  *                 the code form runs for 32 or 64);
- *                 polymer: threads per block (default 256).  Before the first
+ *                 polymer: threads per block (default: as many as spread the
+ *                 walkers evenly over the SMs, at most 256).  Before the first
  *                 iterate.
  *   "pipeline"    spins: 2 (default) pairs every warp of walkers with
- *                 producer warps (two; three for Potts) that compute their
+ *                 producer warps (two; four to six for Potts) that compute their
  *                 random numbers and each site's neighbour code (Potts: also
  *                 the proposal) into a shared-memory ring; 1 does the same
  *                 with random numbers only, one producer warp; 0 runs one
