@@ -244,7 +244,6 @@ __device__ __forceinline__ void produce_sweep(uint32_t g, uint32_t wid, const ui
                                               int drop_k)
 {
     constexpr int G = (SYS == kPotts) ? L / 2 : L / 4;
-    const PhiloxLane pl = philox_lane(g, wid, rk);
 #pragma unroll 1
     for (int y = 0; y < L; ++y) {
         const int slot = k % kRing;
@@ -252,7 +251,7 @@ __device__ __forceinline__ void produce_sweep(uint32_t g, uint32_t wid, const ui
         uint4 *wu = ring + (size_t)slot * G * 32;
 #pragma unroll
         for (int gq = 0; gq < G; ++gq)
-            wu[gq * 32] = philox4x32_10_group((uint32_t)(y * G + gq), pl, rk);
+            wu[gq * 32] = philox4x32_10_rk(make_uint4((uint32_t)(y * G + gq), g, wid, kTagSweep), rk);
         if (k != drop_k) mbar_arrive(&full[slot]);
         ++k;
     }

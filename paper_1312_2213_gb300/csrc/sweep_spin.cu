@@ -55,8 +55,7 @@ __device__ __forceinline__ void ising_sweep(uint32_t *__restrict__ lat, int ps, 
         first[j] = 0u;
         nxt[j] = 0u;
     }
-    const PhiloxLane pl = philox_lane(g, wid, rk);
-    uint4 u_next = philox4x32_10_group(0u, pl, rk);
+    uint4 u_next = philox4x32_10_rk(make_uint4(0u, g, wid, kTagSweep), rk);
 #pragma unroll 1
     for (int y = 0; y < L; ++y) {
         if (y + 2 < L) {
@@ -97,7 +96,7 @@ __device__ __forceinline__ void ising_sweep(uint32_t *__restrict__ lat, int ps, 
         for (int x = 0; x < L; ++x) {
             if ((x & 3) == 0) {
                 u = u_next;
-                u_next = philox4x32_10_group((uint32_t)((y * L + x) / 4 + 1), pl, rk);
+                u_next = philox4x32_10_rk(make_uint4((uint32_t)((y * L + x) / 4 + 1), g, wid, kTagSweep), rk);
             }
             const uint32_t uw = word_of(u, x & 3);
             bR = accP ? bR + dRp : bR;
