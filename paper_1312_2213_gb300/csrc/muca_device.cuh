@@ -65,14 +65,15 @@ __device__ __forceinline__ uint4 philox4x32_10_rk(uint4 c, const uint32_t (&rk)[
     return c;
 }
 
-// Blocks of the code form and of the one-warp q-Potts sweep: counter (word group, sweep, walker,
-// kTagSweep), the group the same for every lane of a warp.  The first two rounds then need no
-// multiplication a lane and block: the products of the walker id (round 1) and of round 1's word 0,
-// which knows walker and sweep only (round 2), are made once a sweep (PhiloxLane), and those of the
-// group and of round 1's word 2 are the same for the whole warp (uniform instructions).  Eight of ten
-// rounds are left, and a block's wide multiplications, 4 cycles each of a scheduler's multiply pipe,
-// set the producers' pace.  (The one-warp Ising sweep ran 9 % slower with it, the producer/consumer
-// form of random words alone 1-4 %: those keep philox4x32_10_rk.)
+// Blocks of the code form: counter (word group, sweep, walker, kTagSweep), the group the same for
+// every lane of a warp.  The first two rounds then need no multiplication a lane and block: the
+// products of the walker id (round 1) and of round 1's word 0, which knows walker and sweep only
+// (round 2), are made once a sweep (PhiloxLane), and those of the group and of round 1's word 2 are
+// the same for the whole warp (uniform instructions).  Eight of ten rounds are left, and a block's
+// wide multiplications, 4 cycles each of a scheduler's multiply pipe, set the producers' pace.  (The
+// one-warp Ising sweep ran 9 % slower with it, the one-warp q-Potts sweep 7 % faster at L = 16 and
+// 2 % slower at L = 24 and 48, the producer/consumer form of random words alone 1-4 % slower: those
+// keep philox4x32_10_rk.)
 struct PhiloxLane {
     uint32_t lo1, hi0, lo0;  // round 1: lo(M1 walker); round 2: hi and lo of M0 word 0
 };

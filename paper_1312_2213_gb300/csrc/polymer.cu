@@ -985,10 +985,11 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
 // weight lookups, the decision) is shared by the 32/G walkers of a warp, the pair
 // terms are spread over G lanes.  A request for a grouping whose warp does not fit
 // the shared memory of a block falls back to the next larger G.  Measured on GB300
-// with 4096 walkers (pilot windows), 16 lanes is the fastest at N = 13, 32, 64 and
-// 128: fewer lanes share the fixed cost among more walkers but leave 4096 G / 32
-// warps to hide latency (G = 4: 2.1e9 against 3.0e9 attempts/s at N = 13; G = 1:
-// 1.1e9), so 16 stays the default.
+// with 2048 walkers (pilot window, N = 13, 46 sweeps): 1.54, 1.07, 0.68, 0.46, 0.30 and
+// 0.47 ms with 1, 2, 4, 8, 16 and 32 lanes.  Fewer lanes share the fixed cost among more
+// walkers but leave 2048 G / 32 warps to hide latency and prepare more beads one after
+// the other, and only 16 has the loops unrolled by the partners of a lane; so 16 is the
+// default.
 // (What fits is still counted in the bytes of a slot that holds a whole sweep's random words: the
 // lanes decide the rounding of the FP32 sums, so a request keeps the grouping it always had.  The
 // slots above are smaller where this line matters.)

@@ -172,8 +172,7 @@ __device__ __forceinline__ void potts_sweep(uint32_t *__restrict__ lat, int ps, 
         nxt[j] = 0u;
     }
     const uint32_t qm1 = q - 1u;
-    const PhiloxLane pl = philox_lane(g, wid, rk);
-    uint4 u_next = philox4x32_10_group(0u, pl, rk);
+    uint4 u_next = philox4x32_10_rk(make_uint4(0u, g, wid, kTagSweep), rk);
 #pragma unroll 1
     for (int y = 0; y < L; ++y) {
         if (y + 2 < L) {
@@ -212,7 +211,7 @@ __device__ __forceinline__ void potts_sweep(uint32_t *__restrict__ lat, int ps, 
         for (int x = 0; x < L; ++x) {
             if ((x & 1) == 0) {
                 u = u_next;
-                u_next = philox4x32_10_group((uint32_t)((y * L + x) / 2 + 1), pl, rk);
+                u_next = philox4x32_10_rk(make_uint4((uint32_t)((y * L + x) / 2 + 1), g, wid, kTagSweep), rk);
             }
             const uint32_t u_acc = (x & 1) ? u.w : u.y;
             bR = accP ? bR + dRp : bR;
