@@ -121,20 +121,23 @@ __device__ __forceinline__ int poly_bin_rel(long long r, const PolyArgs &a)
     return min(max(v, -1), a.B);
 }
 
-// llrint(v 2^32) for |v| < 2^26.  Conversion instructions have twice the latency of additions, and
-// this is on the attempt's chain, so v is cut into integers by adding 1.5 2^23 (the integer then
-// sits in the low mantissa bits): v = 16 h + r, 2^12 r = m + x, q = 2^36 h + 2^20 m + rint(2^20 x),
+// llrint(v 2^32) for the sum of G lanes, each below 2^22: |v| <= 2^26 up to 16 lanes, 2^27 for 32.
+// Conversion instructions have twice the latency of additions, and this is on the attempt's chain, so
+// v is cut into integers by adding 1.5 2^23 (the integer, at most 2^22, then sits in the low mantissa
+// bits): v = U h + r with U = 16 (32 for 32 lanes), 2^12 r = m + x, q = U 2^32 h + 2^20 m + rint(2^20 x),
 // every difference exact (a multiple of v's last place that is no longer than v).  Only the last
 // step rounds, to nearest even beside even terms, as the conversion of v would.
+template <int G>
 __device__ __forceinline__ long long float_to_q32(float v)
 {
     const float M = 12582912.0f;
     const int MB = 0x4B400000;
-    const float th = fmaf(v, 0.0625f, M), r = fmaf(th - M, -16.0f, v);
+    constexpr int U = G > 16 ? 32 : 16;
+    const float th = fmaf(v, 1.0f / U, M), r = fmaf(th - M, (float)-U, v);
     const float tm = fmaf(r, 4096.0f, M), x = fmaf(r, 4096.0f, -(tm - M));
     const float tl = fmaf(x, 1048576.0f, M);
     const int h = __float_as_int(th) - MB, m = __float_as_int(tm) - MB, l = __float_as_int(tl) - MB;
-    return (long long)m * (1 << 20) + l + ((long long)(h * 16) << 32);
+    return (long long)m * (1 << 20) + l + ((long long)(h * U) << 32);
 }
 
 // n visits of a bin: a shared-memory reduction without a returned value, so nothing
@@ -683,7 +686,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                     float lane_sum = fabsf(s) < 4194304.0f ? s - c : __int_as_float(0x7fffffff);
 #pragma unroll
                     for (int off = G / 2; off; off >>= 1) lane_sum += __shfl_xor_sync(0xffffffffu, lane_sum, off);
-                    const long long En = E + float_to_q32(lane_sum);
+                    const long long En = E + float_to_q32<G>(lane_sum);
                     const int bn = poly_bin_rel(En, a);
                     const bool lands = (unsigned)bn < (unsigned)a.B && lane_sum == lane_sum;
                     const long long lwn = __ldg(a.lnWq + (lands ? bn : 0));
@@ -787,7 +790,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 float lane_sum = s - c;
 #pragma unroll
                 for (int off = G / 2; off; off >>= 1) lane_sum += __shfl_xor_sync(0xffffffffu, lane_sum, off);
-                const long long q = float_to_q32(lane_sum);  // (a refused move's is not used)
+                const long long q = float_to_q32<G>(lane_sum);  // (a refused move's is not used)
                 const long long En = E + q;
                 const int bn = poly_bin_rel(En, a);
                 const bool lands = (unsigned)bn < (unsigned)a.B;
