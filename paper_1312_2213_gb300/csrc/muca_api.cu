@@ -1547,8 +1547,8 @@ int muca_batch_create(muca_ctx *const *systems, int n, muca_batch **out)
     e = cudaMemcpy(b->d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_upd, upd.data(), sizeof(UpdateArgs) * n, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b->d_states, states.data(), sizeof(DevState *) * n, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && b->tiles_fit) e = prepare_sweep_batch(b->smem);
-    if (e == cudaSuccess) e = prepare_recursion_batch(b->max_nreach);
+    if (e == cudaSuccess && b->tiles_fit) e = prepare_sweep_batch();
+    if (e == cudaSuccess) e = prepare_recursion_batch();
     if (e != cudaSuccess) {
         cudaFree(b->dmem);
         cudaStreamDestroy(b->stream);

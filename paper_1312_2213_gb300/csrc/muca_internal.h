@@ -27,6 +27,17 @@ struct DevState {
     unsigned long long drift_max_q;    // polymer: largest |E_running - E_scratch| at a refresh (2^-32 units)
 };
 
+// Lets launches of `kernel` ask for up to `most` bytes of dynamic shared memory.  The limit belongs to
+// the kernel, not to the launch: all contexts, batches and threads of the process share it.  So `most`
+// is always the most any launch of that kernel asks for, whatever the launch at hand needs -- a limit
+// that followed the last caller's size refused a larger one prepared before it (a batch of q-Potts
+// L = 64 next to a batch of small lattices; two threads with blocks of 32 and 64 walkers).
+template <class KERNEL>
+inline cudaError_t allow_dynamic_smem(KERNEL kernel, size_t most)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Everything one spin sweep launch needs.  All pointers are device pointers.
 struct SpinSweepArgs {
     const uint32_t *T;       // [B][C] thresholds
@@ -90,7 +101,7 @@ bool spin_sweep_tn_fits(int system, int L, int B, int walkers_per_block);
 size_t spin_sweep_tn_smem_bytes(int system, int L, int B, int walkers_per_block);
 cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s);
 // Batched sweep: tiles[k] = (system index, first walker); all tiles use `block` threads.
-cudaError_t prepare_sweep_batch(size_t smem);
+cudaError_t prepare_sweep_batch();
 cudaError_t launch_sweep_batch(const SpinSweepArgs *d_sys, const int2 *d_tiles, int ntiles, int block, size_t smem,
                                cudaStream_t s);
 
@@ -170,7 +181,7 @@ cudaError_t launch_merge(const UpdateArgs &a, cudaStream_t s);
 // Batched update kernels over n systems (argument arrays in device memory).
 cudaError_t launch_merge_batch(const UpdateArgs *d_args, int n, int max_bins, cudaStream_t s);
 cudaError_t launch_recursion_batch(const UpdateArgs *d_args, int n, int max_nreach, cudaStream_t s);
-cudaError_t prepare_recursion_batch(int max_nreach);
+cudaError_t prepare_recursion_batch();
 cudaError_t launch_thresholds_batch(const UpdateArgs *d_args, int n, int max_cells, cudaStream_t s);
 cudaError_t launch_advance_batch(DevState *const *d_states, const SpinSweepArgs *d_sys, int n, cudaStream_t s);
 cudaError_t launch_recursion(const UpdateArgs &a, cudaStream_t s);

@@ -967,7 +967,7 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
     const int spb = wpb * (32 / G);
     const size_t smem = (size_t)wpb * per_warp + hist;
     const int nblk = (a.p + spb - 1) / spb;
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_polymer<G, MOVES, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_sweep_polymer<G, MOVES, NP>, kPolySmemMax);
     if (e != cudaSuccess) return e;
     // one launch per chunk of sweeps whose visits fit the block's 32-bit counters (spb N a sweep
     // at most), or fewer ("flush_every")

@@ -1303,7 +1303,8 @@ template <int SYS, int L>
 static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s)
 {
     const size_t smem = spin_sweep_tn_smem_bytes(SYS, L, a.B, block);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_spin_tn<SYS, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int largest = spin_sweep_tn_fits(SYS, L, a.B, 64) ? 64 : 32;
+    cudaError_t e = allow_dynamic_smem(k_sweep_spin_tn<SYS, L>, spin_sweep_tn_smem_bytes(SYS, L, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
     k_sweep_spin_tn<SYS, L><<<nblk, kCodeWarpsPerWalkerWarp * block, smem, s>>>(a);
@@ -1338,7 +1339,8 @@ template <int L, int RD>
 static cudaError_t launch_one_tnp(const SpinSweepArgs &a, int block, cudaStream_t s)
 {
     const size_t smem = potts_tn_smem_bytes(L, RD, a.B, block);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_potts_tn<L, RD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int largest = potts_tn_depth(L, a.B, 64) == RD ? 64 : 32;
+    cudaError_t e = allow_dynamic_smem(k_sweep_potts_tn<L, RD>, potts_tn_smem_bytes(L, RD, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
     k_sweep_potts_tn<L, RD><<<nblk, potts_threads(block / 32), smem, s>>>(a);

@@ -381,7 +381,9 @@ template <int SYS, int L>
 static cudaError_t launch_one_pc(const SpinSweepArgs &a, int block, cudaStream_t s)
 {
     const size_t smem = spin_sweep_pc_smem_bytes(SYS, L, a.B, block);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_spin_pc<SYS, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    size_t most = smem;  // of the largest block that fits
+    for (int w = block + 32; spin_sweep_pc_fits(SYS, L, a.B, w); w += 32) most = spin_sweep_pc_smem_bytes(SYS, L, a.B, w);
+    cudaError_t e = allow_dynamic_smem(k_sweep_spin_pc<SYS, L>, most);
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
     k_sweep_spin_pc<SYS, L><<<nblk, 2 * block, smem, s>>>(a);

@@ -35,6 +35,8 @@
 #include "muca_checks.cuh"
 #include "sweep_common.cuh"
 
+#include <algorithm>
+
 namespace muca {
 
 template <int SYS, int L, int RECORD>
@@ -443,15 +445,20 @@ cudaError_t launch_sweep_batch(const SpinSweepArgs *d_sys, const int2 *d_tiles, 
     return cudaGetLastError();
 }
 
-cudaError_t prepare_sweep_batch(size_t smem)
-{
-    return cudaFuncSetAttribute(k_sweep_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 size_t spin_sweep_smem_bytes(int system, int B) { return (size_t)B * (num_cols(system) + 1) * sizeof(uint32_t); }
 
 // The global-table Potts form (L = 64).
 static bool potts_gt(int system, int L) { return system == kPotts && L == 64; }
+
+cudaError_t prepare_sweep_batch()
+{
+    size_t most = 0;  // the largest table of the tiles' systems
+    for (int system : {(int)kIsing, (int)kPotts, (int)kMuma})
+        for (int L = 4; L <= 64; L += 4)
+            if (spin_sweep_supported(system, L) && !potts_gt(system, L))
+                most = std::max(most, spin_sweep_smem_bytes(system, (system == kPotts ? 2 : 1) * L * L + 1));
+    return allow_dynamic_smem(k_sweep_batch, most);
+}
 
 bool spin_sweep_supported(int system, int L)
 {
@@ -467,7 +474,7 @@ template <int SYS, int L>
 static cudaError_t launch_one(const SpinSweepArgs &a, int block, cudaStream_t s)
 {
     const size_t smem = spin_sweep_smem_bytes(SYS, a.B);
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_spin<SYS, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k_sweep_spin<SYS, L>, smem);  // (the same for every launch)
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
     k_sweep_spin<SYS, L><<<nblk, block, smem, s>>>(a);
@@ -497,7 +504,7 @@ cudaError_t launch_spin_sweep(int system, int L, const SpinSweepArgs &a, int blo
     if (!spin_sweep_supported(system, L)) return cudaErrorInvalidValue;
     if (potts_gt(system, L)) {
         const size_t smem = (size_t)a.B * sizeof(uint32_t);
-        cudaError_t e = cudaFuncSetAttribute(k_sweep_potts_gt<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_dynamic_smem(k_sweep_potts_gt<64>, smem);  // (the same for every launch)
         if (e != cudaSuccess) return e;
         k_sweep_potts_gt<64><<<(a.p + block - 1) / block, block, smem, s>>>(a);
         return cudaGetLastError();

@@ -679,7 +679,7 @@ cudaError_t launch_recursion(const UpdateArgs &a, cudaStream_t s)
 {
     const size_t smem = recursion_smem(a.nreach);
     if (smem > 40u * 1024u) {  // above what a launch may ask for without the attribute
-        const cudaError_t e = cudaFuncSetAttribute(k_recursion, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_dynamic_smem(k_recursion, recursion_smem(kPolyMaxBins));
         if (e != cudaSuccess) return e;
     }
     k_recursion<<<recursion_grid(a.nreach), kRecThreads, smem, s>>>(a);
@@ -705,10 +705,9 @@ cudaError_t launch_recursion_batch(const UpdateArgs *d_args, int n, int max_nrea
     return cudaGetLastError();
 }
 
-cudaError_t prepare_recursion_batch(int max_nreach)
+cudaError_t prepare_recursion_batch()
 {
-    return cudaFuncSetAttribute(k_recursion_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)recursion_smem(max_nreach));
+    return allow_dynamic_smem(k_recursion_batch, recursion_smem(kPolyMaxBins));  // (no system has more bins)
 }
 
 cudaError_t launch_thresholds_batch(const UpdateArgs *d_args, int n, int max_cells, cudaStream_t s)
