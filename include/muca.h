@@ -145,7 +145,8 @@ int muca_init_ex(muca_ctx **out, int system, int L_or_N, int q, int p, uint64_t 
  *                 uint64 slot (the polymer: to the uint64 histogram); 0
  *                 (default) = the largest count that cannot overflow a
  *                 counter (floor((2^32 - 1) / (block walkers * N)), or
- *                 / block with "record" = 1).  Results do not depend on it;
+ *                 / block with "record" = 1; lattices at most 2^30 / L, for
+ *                 the row counters).  Results do not depend on it;
  *                 a small value makes short runs cross the flush between
  *                 chunks of sweeps (tests).  Any time.
  *   "model"       polymer, before the first iterate: 0 (default) = the benchmark

@@ -17,6 +17,7 @@
 
 #include "muca.h"
 #include "muca_internal.h"
+#include "ring_rows.h"
 
 using namespace muca;
 
@@ -296,10 +297,8 @@ SpinSweepArgs sweep_args(const muca_ctx *c, int64_t sweeps, int block)
     a.sweeps = sweeps;
     const unsigned long long per_sweep = (unsigned long long)block * (c->record == 0 ? (unsigned)c->N : 1u);
     unsigned long long fe = 0xFFFFFFFFull / per_sweep;
-    if (fe < 1) fe = 1;
     if (c->flush_cap > 0 && fe > (unsigned long long)c->flush_cap) fe = (unsigned long long)c->flush_cap;
-    if (fe > (unsigned long long)sweeps) fe = (unsigned long long)sweeps;
-    a.flush_every = (int)(fe > 0x7fffffffull ? 0x7fffffffull : fe);
+    a.flush_every = chunk_sweeps(fe, sweeps, c->L);
     fill_round_keys(a, c->seed);
     a.record = c->record;
     a.walker_offset = c->walker_offset;

@@ -390,7 +390,7 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
     const CodeRole role = code_role(warp, ncw);
     const bool producer = role.kind == kRoleProducer, consumer = role.kind == kRoleConsumer;
     const int pair = role.pair, part = role.part;
-    const int drop_k = (blockIdx.x == 0 && producer && pair == 0 && part == 0) ? a.debug_drop_row : -1;
+    int drop_k = (blockIdx.x == 0 && producer && pair == 0 && part == 0) ? a.debug_drop_row : -1;
     uint32_t *sTH = smem;
     const size_t th_bytes = ((size_t)NB * (C + 1) * 4 + 15) / 16 * 16;
     char *rbase = (char *)smem + th_bytes + (size_t)pair * tn_ring_bytes(L);
@@ -466,6 +466,7 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
                 sTH[C * NB + b] = 0u;
             }
         }
+        rebase_rows(k, drop_k, kRing);
         __syncthreads();
     }
     if (bad) atomicOr(const_cast<int *>(&a.state->err), 1);
@@ -1167,7 +1168,7 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
         ng = potts_part_groups(L, ncw, i);
     }
     // (the test hook's row: with whole rows in turn, of the producer whose turn it is)
-    const int drop_k = (blockIdx.x == 0 && producer && pair == 0 && (ROWS || part == 0)) ? a.debug_drop_row : -1;
+    int drop_k = (blockIdx.x == 0 && producer && pair == 0 && (ROWS || part == 0)) ? a.debug_drop_row : -1;
     uint32_t *sTH = smem;
     const size_t th_bytes = tnp_table_bytes(L, a.B);
     constexpr size_t UB = R::split ? 8 : 16;  // ring bytes of a group's acceptance words
@@ -1260,6 +1261,7 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
                 sTH[b * RS + R::HW] -= c << R::CSH;
             }
         }
+        rebase_rows(k, drop_k, RD);
         __syncthreads();
     }
     if (bad) atomicOr(const_cast<int *>(&a.state->err), 1);

@@ -5,6 +5,7 @@
 #pragma once
 #include "muca_device.cuh"
 #include "muca_internal.h"
+#include "ring_rows.h"
 
 namespace muca {
 

@@ -274,7 +274,7 @@ __device__ __forceinline__ void sweep_block_pc(const SpinSweepArgs &a, int w0, i
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool producer = warp >= ncw;
     const int pair = producer ? warp - ncw : warp;
-    const int drop_k = (blockIdx.x == 0 && producer && pair == 0) ? a.debug_drop_row : -1;
+    int drop_k = (blockIdx.x == 0 && producer && pair == 0) ? a.debug_drop_row : -1;
     uint32_t *sTH = smem;
     const size_t th_bytes = ((size_t)a.B * RS * 4 + 15) / 16 * 16;
     uint4 *ring = (uint4 *)((char *)smem + th_bytes) + (size_t)pair * kRing * G * 32 + lane;
@@ -350,6 +350,7 @@ __device__ __forceinline__ void sweep_block_pc(const SpinSweepArgs &a, int w0, i
                 sTH[b * RS + C] = 0u;
             }
         }
+        rebase_rows(k, drop_k, kRing);
         __syncthreads();
     }
     if (bad) atomicOr(const_cast<int *>(&a.state->err), 1);
