@@ -100,6 +100,11 @@ constexpr int kCodeWarpsPerWalkerWarp = 4;
 // with one took a loop of their own, which the warp then ran after the walkers': 10 % at p = 1000.)
 __device__ __forceinline__ unsigned code_consumer_lanes(int left) { return left > 0 && left < 32 ? (unsigned)left : 32u; }
 
+// A lane whose wait gives up (`bad`) takes no further part in the launch's hand-overs: it writes no slot,
+// reads none and arrives nowhere, so its partners' waits run out as well, within the same bound, and no
+// lane ever decides on a slot that is being rewritten (its codes need not fit its lattice and bin, which
+// could walk off the table).
+
 // The producer's rows of nsw sweeps.
 template <int SYS, int L, int PART>
 __device__ __forceinline__ void produce_tn(int64_t nsw, uint32_t g0, uint32_t wid, const uint32_t (&rk)[20],
@@ -140,7 +145,10 @@ __device__ __forceinline__ void produce_tn(int64_t nsw, uint32_t g0, uint32_t wi
                 for (int e = 0; e < PB; ++e) words[i + e] = clamp_words(c[e]);
             }
             for (int i = NG / PB * PB; i < NG; ++i) words[i] = clamp_words(philox4x32_10_group((uint32_t)(y * G + g_lo + i), pl, rk));
-            if (!free_slot && !bad && !mbar_wait(&empty[slot], (unsigned)(((k / kRing) & 1) ^ 1))) bad = true;
+            if (!free_slot && !mbar_wait(&empty[slot], (unsigned)(((k / kRing) & 1) ^ 1))) {
+                bad = true;
+                return;
+            }
             const int y2 = (y + 2 < L) ? y + 2 : y + 2 - L;
 #pragma unroll
             for (int j = 0; j < WR; ++j) nn[j] = lat[(y2 * WR + j) * ps];
@@ -236,7 +244,7 @@ __device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ l
     uint2 cdn = make_uint2(0u, 0u);
     uint32_t T0 = 0u, T1 = 0u;
     bool accP = false;  // the site decided before
-    if (!bad && !mbar_wait(&full[k % kRing], (unsigned)((k / kRing) & 1))) bad = true;
+    if (!mbar_wait(&full[k % kRing], (unsigned)((k / kRing) & 1))) bad = true;
     if (!bad) {
         const int slot = k % kRing;
 #pragma unroll
@@ -349,10 +357,7 @@ __device__ __forceinline__ void consume_tn(int64_t nsw, uint32_t *__restrict__ l
         }
         tunnel_step(bin, r_lo, r_hi, tst, ev);
     }
-    while (k != k_end) {  // a wait gave up: the ring is out of step, so nothing more is computed
-        mbar_arrive(&empty[k % kRing]);
-        ++k;
-    }
+    k = k_end;
     bR = (bB - sbase) / 4;
 }
 
@@ -437,7 +442,8 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
     for (int64_t s0 = 0; s0 < a.sweeps; s0 += a.flush_every) {
         const int64_t nsw = (a.sweeps < s0 + a.flush_every) ? a.sweeps - s0 : (int64_t)a.flush_every;
         const uint32_t g = g0 + (uint32_t)s0;
-        if (producer) {
+        if (bad) {  // (a wait of this lane gave up: see code_consumer_lanes)
+        } else if (producer) {
             if (part == 0)
                 produce_tn<SYS, L, 0>(nsw, g, wid, a.rk, lat, a.pstride, ring_u, ring_c, ring_r, full, empty, k, bad, drop_k);
             else
@@ -446,7 +452,10 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
 #pragma unroll 1
             for (int64_t r = 0; r < nsw * L; ++r) {
                 const int slot = k % kRing;
-                if (!bad && !mbar_wait(&full[slot], (unsigned)((k / kRing) & 1))) bad = true;
+                if (!mbar_wait(&full[slot], (unsigned)((k / kRing) & 1))) {
+                    bad = true;
+                    break;
+                }
                 mbar_arrive(&empty[slot]);
                 ++k;
             }
@@ -691,7 +700,10 @@ __device__ __forceinline__ void produce_potts_rows(int64_t nsw, uint32_t sweep0,
         const PhiloxLane pl = philox_lane(sweep0 + (uint32_t)sw, wid, rk);
 #pragma unroll 1
         for (int y = part; y < L; y += RD) {
-            if (!bad && !mbar_wait(&empty[part], (unsigned)(((k / RD) & 1) ^ 1))) bad = true;
+            if (!mbar_wait(&empty[part], (unsigned)(((k / RD) & 1) ^ 1))) {
+                bad = true;
+                return;
+            }
             if (AHEAD) {
 #pragma unroll
                 for (int e = 0; e < WR; ++e) {
@@ -809,7 +821,10 @@ __device__ __forceinline__ void produce_potts_tn(int64_t nsw, uint32_t sweep0, u
                     const uint2 c = potts_group<L>(r, q, ob, ob_prev, ob_next, db, pprev, j == 0,
                                                    i == ng - 1 ? mask_last : 0xFFFFFFFFu, pb);
                     if (i == 0) {
-                        if (!free_slot && !bad && !mbar_wait(&empty[slot], (unsigned)(((k / RD) & 1) ^ 1))) bad = true;
+                        if (!free_slot && !mbar_wait(&empty[slot], (unsigned)(((k / RD) & 1) ^ 1))) {
+                            bad = true;
+                            return;
+                        }
                         // (also behind the last row: rows 0 and 1 as this sweep leaves them)
                         const int y2 = (y + 2 < L) ? y + 2 : y + 2 - L;
 #pragma unroll
@@ -1033,7 +1048,7 @@ __device__ __forceinline__ void consume_potts_tn(int64_t nsw, uint32_t sweep0, u
         if (RECORD == 0) hist(bB);
         accP = acc;
     };
-    if (!bad && !mbar_wait(&full[k % RD], (unsigned)((k / RD) & 1))) bad = true;
+    if (!mbar_wait(&full[k % RD], (unsigned)((k / RD) & 1))) bad = true;
     if (!bad) {
         const int slot = k % RD;
         opn = ring_op[slot * S];
@@ -1125,10 +1140,7 @@ __device__ __forceinline__ void consume_potts_tn(int64_t nsw, uint32_t sweep0, u
         if (RECORD == 1) atomicAdd(&sTH[checked_word(word + R::HW)], R::ONE);
         tunnel_step(word, r_lo, r_hi, tst, ev);
     }
-    while (k != k_end) {  // a wait gave up: the ring is out of step, so nothing more is computed
-        mbar_arrive(&empty[k % RD]);
-        ++k;
-    }
+    k = k_end;
     bR = (bB - sbase) / 4;
 }
 
@@ -1230,7 +1242,8 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
     for (int64_t s0 = 0; s0 < a.sweeps; s0 += a.flush_every) {
         const int64_t nsw = (a.sweeps < s0 + a.flush_every) ? a.sweeps - s0 : (int64_t)a.flush_every;
         const uint32_t g = g_first + (uint32_t)s0;
-        if (producer) {
+        if (bad) {  // (a wait of this lane gave up: see code_consumer_lanes)
+        } else if (producer) {
             if constexpr (ROWS)
                 produce_potts_rows<L, RD>(nsw, g, wid, a.rk, lat, a.pstride, (uint32_t)a.q, part, ring_u, ring_c, ring_op, full,
                                           empty, k, bad, drop_k);
@@ -1241,7 +1254,10 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
 #pragma unroll 1
             for (int64_t r = 0; r < nsw * L; ++r) {
                 const int slot = k % RD;
-                if (!bad && !mbar_wait(&full[slot], (unsigned)((k / RD) & 1))) bad = true;
+                if (!mbar_wait(&full[slot], (unsigned)((k / RD) & 1))) {
+                    bad = true;
+                    break;
+                }
                 mbar_arrive(&empty[slot]);
                 ++k;
             }
