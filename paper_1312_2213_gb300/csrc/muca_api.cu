@@ -16,6 +16,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "muca.h"
+#include "batch_lanes.h"
 #include "muca_internal.h"
 #include "ring_rows.h"
 
@@ -314,24 +315,15 @@ SpinSweepArgs sweep_args(const muca_ctx *c, int64_t sweeps, int block)
 
 // The context's sweep in its configured form (code form, producer/consumer or one warp), falling
 // back to the next lower form where one does not fit the system, L, bin count or block.
-cudaError_t launch_system_sweep(const muca_ctx *c, const SpinSweepArgs &a, cudaStream_t s, int block = 0)
+cudaError_t launch_system_sweep(const muca_ctx *c, const SpinSweepArgs &a, cudaStream_t s, int block = 0,
+                                int *per_sm = nullptr)
 {
     if (block <= 0) block = c->block;
     if (c->pipeline >= 2 && spin_sweep_tn_fits(c->system, c->L, c->B, block))
-        return launch_spin_sweep_tn(c->system, c->L, a, block, s);
+        return launch_spin_sweep_tn(c->system, c->L, a, block, s, per_sm);
     if (c->pipeline >= 1 && spin_sweep_pc_fits(c->system, c->L, c->B, block))
-        return launch_spin_sweep_pc(c->system, c->L, a, block, s);
-    return launch_spin_sweep(c->system, c->L, a, block, s);
-}
-
-// Shared memory of one block of that launch.
-size_t system_sweep_smem(const muca_ctx *c, int block)
-{
-    if (c->pipeline >= 2 && spin_sweep_tn_fits(c->system, c->L, c->B, block))
-        return spin_sweep_tn_smem_bytes(c->system, c->L, c->B, block);
-    if (c->pipeline >= 1 && spin_sweep_pc_fits(c->system, c->L, c->B, block))
-        return spin_sweep_pc_smem_bytes(c->system, c->L, c->B, block);
-    return spin_sweep_smem_bytes(c->system, c->B);
+        return launch_spin_sweep_pc(c->system, c->L, a, block, s, per_sm);
+    return launch_spin_sweep(c->system, c->L, a, block, s, per_sm);
 }
 
 PolyArgs poly_args(const muca_ctx *c, int64_t sweeps)
@@ -1351,6 +1343,8 @@ struct muca_batch {
     std::vector<int64_t> sw;           // per-system sweeps of an iteration (empty: the run's argument)
     std::vector<int> blk;              // form 1: each system's walkers per block in this batch
     int nsm = 152;                     // SMs of the device
+    std::vector<LaneSystem> lane_sys;  // form 1: what the streams were planned for (in order)
+    std::vector<int> lane;             // and the stream of each
     std::vector<int64_t> g_sw;         // per-system sweeps the captured graph was made with
 };
 
@@ -1378,57 +1372,40 @@ std::vector<int> batch_order(const muca_batch *b, int form)
     return order;
 }
 
-// Form 1: which of the batch's streams each system's sweep goes to, by its place in the order.  A
-// system whose blocks find SMs beside the heavier ones' gets a stream of its own; when the SMs are
-// taken, it queues behind the system that ends first.  (With every system on a stream of its own the
-// light systems' small blocks could be placed first, in a graph above all, and an L = 64 block, which
-// takes an SM's whole shared memory, had to wait for them: 27 ms for 20 iterations of 10 sweeps of the
-// mix as a graph, where the L = 64 chain and the updates take 19.)  Polymers fill the GPU
-// by themselves and gain from lying side by side, so each keeps its own stream.
-std::vector<int> batch_lanes(const muca_batch *b)
+// Form 1: the batch's stream of each system's sweep, by its place in the order (batch_lanes.h).
+int batch_lanes(muca_batch *b)
 {
-    const int n = (int)b->sys.size();
-    std::vector<int> lane(n);
-    std::vector<double> end;
-    double free_sms = (double)b->nsm;
-    for (int r = 0; r < n; ++r) {
-        const int i = b->order[r];
+    std::vector<LaneSystem> sys;
+    for (int i : b->order) {
         const muca_ctx *c = b->sys[i];
-        double sms = 0.0;
-        if (c->system != kPolymer) {
-            const size_t smem = std::max(system_sweep_smem(c, b->blk[i]), (size_t)1);
-            const int per_sm = std::max(1, std::min((int)(kMaxSmem / smem), 4));
-            sms = (double)((c->p + b->blk[i] - 1) / b->blk[i]) / per_sm;
+        LaneSystem s{0, 1, batch_cost(b, i, 1), c->system == kPolymer};
+        if (!s.polymer) {
+            s.blocks = (c->p + b->blk[i] - 1) / b->blk[i];
+            MUCA_CUDA(launch_system_sweep(c, b->h_own[i], nullptr, b->blk[i], &s.per_sm));
+            s.per_sm = std::max(s.per_sm, 1);
         }
-        // (a system that mostly fits starts too: its last blocks follow the first that end)
-        if (end.empty() || sms <= 1.5 * free_sms) {
-            lane[r] = (int)end.size();
-            end.push_back(batch_cost(b, i, 1));
-            free_sms -= sms;
-        } else {
-            int best = 0;
-            for (int l = 1; l < (int)end.size(); ++l)
-                if (end[l] < end[best]) best = l;
-            lane[r] = best;
-            end[best] += batch_cost(b, i, 1);
-        }
+        sys.push_back(s);
     }
-    return lane;
+    if (sys != b->lane_sys) {
+        b->lane = plan_lanes(sys, b->nsm);
+        b->lane_sys = sys;
+    }
+    return MUCA_OK;
 }
 
-int batch_enqueue_iteration(muca_batch *b, int64_t sweeps)
+int batch_enqueue_iteration(muca_batch *b)
 {
     const int n = (int)b->sys.size();
     if (b->form == 1) {
         MUCA_CUDA(cudaEventRecord(b->ev_fork, b->stream));
         // heaviest first, so that their blocks take the SMs before the light systems' blocks
-        const std::vector<int> lane = batch_lanes(b);
         std::vector<char> forked(n, 0);
         for (int r = 0; r < n; ++r) {
             const int i = b->order[r];
-            const cudaStream_t sub = b->sub[lane[r]];
-            if (!forked[lane[r]]) MUCA_CUDA(cudaStreamWaitEvent(sub, b->ev_fork, 0));
-            forked[lane[r]] = 1;
+            const int l = b->lane[r];
+            const cudaStream_t sub = b->sub[l];
+            if (!forked[l]) MUCA_CUDA(cudaStreamWaitEvent(sub, b->ev_fork, 0));
+            forked[l] = 1;
             muca_ctx *c = b->sys[i];
             if (c->system == kPolymer) {  // as muca_iterate: the sweeps, then the energies from scratch
                 const PolyArgs pa = poly_args(c, b->h_sys[i].sweeps);
@@ -1443,7 +1420,6 @@ int batch_enqueue_iteration(muca_batch *b, int64_t sweeps)
     } else {
         MUCA_CUDA(launch_sweep_batch(b->d_sys, b->d_tiles, b->ntiles, b->block, b->smem, b->stream));
     }
-    (void)sweeps;
     MUCA_CUDA(launch_advance_batch(b->d_states, b->d_sys, n, b->stream));
     MUCA_CUDA(launch_merge_batch(b->d_upd, n, b->max_bins, b->stream));
     MUCA_CUDA(launch_recursion_batch(b->d_upd, n, b->max_nreach, b->stream));
@@ -1612,9 +1588,11 @@ int muca_batch_run(muca_batch *b, int n_iter, int64_t sweeps, int use_graph)
             }
             // the host-side copies above stay outside the captured region
             MUCA_CUDA(cudaStreamSynchronize(b->stream));
+            if (b->form == 1)
+                if (int rc = batch_lanes(b)) return rc;
             MUCA_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
             int rc = MUCA_OK;
-            for (int it = 0; it < n_iter && rc == MUCA_OK; ++it) rc = batch_enqueue_iteration(b, sweeps);
+            for (int it = 0; it < n_iter && rc == MUCA_OK; ++it) rc = batch_enqueue_iteration(b);
             cudaGraph_t graph = nullptr;
             cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
             if (rc != MUCA_OK) {
@@ -1634,8 +1612,10 @@ int muca_batch_run(muca_batch *b, int n_iter, int64_t sweeps, int use_graph)
         }
         MUCA_CUDA(cudaGraphLaunch(b->exec, b->stream));
     } else {
+        if (b->form == 1)
+            if (int rc = batch_lanes(b)) return rc;
         for (int it = 0; it < n_iter; ++it)
-            if (int rc = batch_enqueue_iteration(b, sweeps)) return rc;
+            if (int rc = batch_enqueue_iteration(b)) return rc;
     }
     // and the systems' later work after the batch
     MUCA_CUDA(cudaEventRecord(b->ev_out, b->stream));

@@ -87,19 +87,28 @@ __host__ __device__ constexpr int words_per_walker(int system, int L)
 __host__ __device__ constexpr int num_cols(int system) { return system == kPotts ? 9 : (system == kMuma ? 10 : 5); }
 
 // Launchers (return cudaSuccess or the launch error; cudaErrorInvalidValue for
-// an unsupported lattice size).
+// an unsupported lattice size).  With `per_sm` nothing is launched: it receives
+// how many blocks of that launch an SM holds at a time.
+template <class KERNEL>
+inline cudaError_t launch_sweep_kernel(KERNEL kernel, const SpinSweepArgs &a, int blocks, int threads, size_t smem,
+                                       cudaStream_t s, int *per_sm)
+{
+    if (per_sm) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kernel, threads, smem);
+    kernel<<<blocks, threads, smem, s>>>(a);
+    return cudaGetLastError();
+}
 bool spin_sweep_supported(int system, int L);
 size_t spin_sweep_smem_bytes(int system, int B);
-cudaError_t launch_spin_sweep(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s);
+cudaError_t launch_spin_sweep(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm = nullptr);
 int sweep_kind(int system, int L);
 // Producer/consumer form: `block` walkers a block, run by 2*block threads.
 bool spin_sweep_pc_fits(int system, int L, int B, int walkers_per_block);
 size_t spin_sweep_pc_smem_bytes(int system, int L, int B, int walkers_per_block);
-cudaError_t launch_spin_sweep_pc(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s);
+cudaError_t launch_spin_sweep_pc(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm = nullptr);
 // Producer/consumer form with precomputed site codes (Ising, MUMA).
 bool spin_sweep_tn_fits(int system, int L, int B, int walkers_per_block);
 size_t spin_sweep_tn_smem_bytes(int system, int L, int B, int walkers_per_block);
-cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s);
+cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm = nullptr);
 // Batched sweep: tiles[k] = (system index, first walker); all tiles use `block` threads.
 cudaError_t prepare_sweep_batch();
 cudaError_t launch_sweep_batch(const SpinSweepArgs *d_sys, const int2 *d_tiles, int ntiles, int block, size_t smem,

@@ -1318,28 +1318,27 @@ static int potts_tn_depth(int L, int B, int walkers_per_block)
 
 
 template <int SYS, int L>
-static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     const size_t smem = spin_sweep_tn_smem_bytes(SYS, L, a.B, block);
     const int largest = spin_sweep_tn_fits(SYS, L, a.B, 64) ? 64 : 32;
     cudaError_t e = allow_dynamic_smem(k_sweep_spin_tn<SYS, L>, spin_sweep_tn_smem_bytes(SYS, L, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    k_sweep_spin_tn<SYS, L><<<nblk, kCodeWarpsPerWalkerWarp * block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_sweep_kernel(k_sweep_spin_tn<SYS, L>, a, nblk, kCodeWarpsPerWalkerWarp * block, smem, s, per_sm);
 }
 
 template <int SYS>
-static cudaError_t launch_sys_tn(int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_sys_tn(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     switch (L) {
-    case 8: return launch_one_tn<SYS, 8>(a, block, s);
-    case 12: return launch_one_tn<SYS, 12>(a, block, s);
-    case 16: return launch_one_tn<SYS, 16>(a, block, s);
-    case 24: return launch_one_tn<SYS, 24>(a, block, s);
-    case 32: return launch_one_tn<SYS, 32>(a, block, s);
-    case 48: return launch_one_tn<SYS, 48>(a, block, s);
-    case 64: return launch_one_tn<SYS, 64>(a, block, s);
+    case 8: return launch_one_tn<SYS, 8>(a, block, s, per_sm);
+    case 12: return launch_one_tn<SYS, 12>(a, block, s, per_sm);
+    case 16: return launch_one_tn<SYS, 16>(a, block, s, per_sm);
+    case 24: return launch_one_tn<SYS, 24>(a, block, s, per_sm);
+    case 32: return launch_one_tn<SYS, 32>(a, block, s, per_sm);
+    case 48: return launch_one_tn<SYS, 48>(a, block, s, per_sm);
+    case 64: return launch_one_tn<SYS, 64>(a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -1354,47 +1353,46 @@ bool spin_sweep_tn_fits(int system, int L, int B, int walkers_per_block)
 }
 
 template <int L, int RD>
-static cudaError_t launch_one_tnp(const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_one_tnp(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     const size_t smem = potts_tn_smem_bytes(L, RD, a.B, block);
     const int largest = potts_tn_depth(L, a.B, 64) == RD ? 64 : 32;
     cudaError_t e = allow_dynamic_smem(k_sweep_potts_tn<L, RD>, potts_tn_smem_bytes(L, RD, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    k_sweep_potts_tn<L, RD><<<nblk, potts_threads(block / 32), smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_sweep_kernel(k_sweep_potts_tn<L, RD>, a, nblk, potts_threads(block / 32), smem, s, per_sm);
 }
 
 template <int RD>
-static cudaError_t launch_potts_tn_rd(int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_potts_tn_rd(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     switch (L) {
-    case 8: return launch_one_tnp<8, RD>(a, block, s);
-    case 16: return launch_one_tnp<16, RD>(a, block, s);
-    case 24: return launch_one_tnp<24, RD>(a, block, s);
-    case 32: return launch_one_tnp<32, RD>(a, block, s);
-    case 48: return launch_one_tnp<48, RD>(a, block, s);
+    case 8: return launch_one_tnp<8, RD>(a, block, s, per_sm);
+    case 16: return launch_one_tnp<16, RD>(a, block, s, per_sm);
+    case 24: return launch_one_tnp<24, RD>(a, block, s, per_sm);
+    case 32: return launch_one_tnp<32, RD>(a, block, s, per_sm);
+    case 48: return launch_one_tnp<48, RD>(a, block, s, per_sm);
     case 64:  // the split table: only the two-row ring fits
-        if constexpr (RD == 2) return launch_one_tnp<64, 2>(a, block, s);
+        if constexpr (RD == 2) return launch_one_tnp<64, 2>(a, block, s, per_sm);
         return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
 }
 
-static cudaError_t launch_potts_tn(int L, int rd, const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_potts_tn(int L, int rd, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
-    if (rd == 4) return launch_potts_tn_rd<4>(L, a, block, s);
-    if (rd == 2) return launch_potts_tn_rd<2>(L, a, block, s);
+    if (rd == 4) return launch_potts_tn_rd<4>(L, a, block, s, per_sm);
+    if (rd == 2) return launch_potts_tn_rd<2>(L, a, block, s, per_sm);
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     if (!spin_sweep_supported(system, L) || !spin_sweep_tn_fits(system, L, a.B, block)) return cudaErrorInvalidValue;
     switch (system) {
-    case kIsing: return launch_sys_tn<kIsing>(L, a, block, s);
-    case kMuma: return launch_sys_tn<kMuma>(L, a, block, s);
-    case kPotts: return launch_potts_tn(L, potts_tn_depth(L, a.B, block), a, block, s);
+    case kIsing: return launch_sys_tn<kIsing>(L, a, block, s, per_sm);
+    case kMuma: return launch_sys_tn<kMuma>(L, a, block, s, per_sm);
+    case kPotts: return launch_potts_tn(L, potts_tn_depth(L, a.B, block), a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }

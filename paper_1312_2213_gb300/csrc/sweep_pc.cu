@@ -379,7 +379,7 @@ size_t spin_sweep_pc_smem_bytes(int system, int L, int B, int walkers_per_block)
 
 
 template <int SYS, int L>
-static cudaError_t launch_one_pc(const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_one_pc(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     const size_t smem = spin_sweep_pc_smem_bytes(SYS, L, a.B, block);
     size_t most = smem;  // of the largest block that fits
@@ -387,22 +387,21 @@ static cudaError_t launch_one_pc(const SpinSweepArgs &a, int block, cudaStream_t
     cudaError_t e = allow_dynamic_smem(k_sweep_spin_pc<SYS, L>, most);
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    k_sweep_spin_pc<SYS, L><<<nblk, 2 * block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_sweep_kernel(k_sweep_spin_pc<SYS, L>, a, nblk, 2 * block, smem, s, per_sm);
 }
 
 template <int SYS>
-static cudaError_t launch_sys_pc(int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_sys_pc(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     switch (L) {
-    case 4: return launch_one_pc<SYS, 4>(a, block, s);
-    case 8: return launch_one_pc<SYS, 8>(a, block, s);
-    case 12: return launch_one_pc<SYS, 12>(a, block, s);
-    case 16: return launch_one_pc<SYS, 16>(a, block, s);
-    case 24: return launch_one_pc<SYS, 24>(a, block, s);
-    case 32: return launch_one_pc<SYS, 32>(a, block, s);
-    case 48: return launch_one_pc<SYS, 48>(a, block, s);
-    case 64: return launch_one_pc<SYS, 64>(a, block, s);
+    case 4: return launch_one_pc<SYS, 4>(a, block, s, per_sm);
+    case 8: return launch_one_pc<SYS, 8>(a, block, s, per_sm);
+    case 12: return launch_one_pc<SYS, 12>(a, block, s, per_sm);
+    case 16: return launch_one_pc<SYS, 16>(a, block, s, per_sm);
+    case 24: return launch_one_pc<SYS, 24>(a, block, s, per_sm);
+    case 32: return launch_one_pc<SYS, 32>(a, block, s, per_sm);
+    case 48: return launch_one_pc<SYS, 48>(a, block, s, per_sm);
+    case 64: return launch_one_pc<SYS, 64>(a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -414,13 +413,13 @@ bool spin_sweep_pc_fits(int system, int L, int B, int walkers_per_block)
 }
 
 
-cudaError_t launch_spin_sweep_pc(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+cudaError_t launch_spin_sweep_pc(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     if (!spin_sweep_supported(system, L) || !spin_sweep_pc_fits(system, L, a.B, block)) return cudaErrorInvalidValue;
     switch (system) {
-    case kIsing: return launch_sys_pc<kIsing>(L, a, block, s);
-    case kMuma: return launch_sys_pc<kMuma>(L, a, block, s);
-    case kPotts: return launch_sys_pc<kPotts>(L, a, block, s);
+    case kIsing: return launch_sys_pc<kIsing>(L, a, block, s, per_sm);
+    case kMuma: return launch_sys_pc<kMuma>(L, a, block, s, per_sm);
+    case kPotts: return launch_sys_pc<kPotts>(L, a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }

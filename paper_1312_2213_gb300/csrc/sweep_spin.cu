@@ -471,48 +471,46 @@ bool spin_sweep_supported(int system, int L)
 }
 
 template <int SYS, int L>
-static cudaError_t launch_one(const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_one(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     const size_t smem = spin_sweep_smem_bytes(SYS, a.B);
     cudaError_t e = allow_dynamic_smem(k_sweep_spin<SYS, L>, smem);  // (the same for every launch)
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    k_sweep_spin<SYS, L><<<nblk, block, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_sweep_kernel(k_sweep_spin<SYS, L>, a, nblk, block, smem, s, per_sm);
 }
 
 
 template <int SYS>
-static cudaError_t launch_sys(int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+static cudaError_t launch_sys(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     switch (L) {
-    case 4: return launch_one<SYS, 4>(a, block, s);
-    case 8: return launch_one<SYS, 8>(a, block, s);
-    case 12: return launch_one<SYS, 12>(a, block, s);
-    case 16: return launch_one<SYS, 16>(a, block, s);
-    case 24: return launch_one<SYS, 24>(a, block, s);
-    case 32: return launch_one<SYS, 32>(a, block, s);
-    case 48: return launch_one<SYS, 48>(a, block, s);
-    case 64: return launch_one<SYS, 64>(a, block, s);
+    case 4: return launch_one<SYS, 4>(a, block, s, per_sm);
+    case 8: return launch_one<SYS, 8>(a, block, s, per_sm);
+    case 12: return launch_one<SYS, 12>(a, block, s, per_sm);
+    case 16: return launch_one<SYS, 16>(a, block, s, per_sm);
+    case 24: return launch_one<SYS, 24>(a, block, s, per_sm);
+    case 32: return launch_one<SYS, 32>(a, block, s, per_sm);
+    case 48: return launch_one<SYS, 48>(a, block, s, per_sm);
+    case 64: return launch_one<SYS, 64>(a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }
 
 
-cudaError_t launch_spin_sweep(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s)
+cudaError_t launch_spin_sweep(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     if (!spin_sweep_supported(system, L)) return cudaErrorInvalidValue;
     if (potts_gt(system, L)) {
         const size_t smem = (size_t)a.B * sizeof(uint32_t);
         cudaError_t e = allow_dynamic_smem(k_sweep_potts_gt<64>, smem);  // (the same for every launch)
         if (e != cudaSuccess) return e;
-        k_sweep_potts_gt<64><<<(a.p + block - 1) / block, block, smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_sweep_kernel(k_sweep_potts_gt<64>, a, (a.p + block - 1) / block, block, smem, s, per_sm);
     }
     switch (system) {
-    case kIsing: return launch_sys<kIsing>(L, a, block, s);
-    case kMuma: return launch_sys<kMuma>(L, a, block, s);
-    case kPotts: return launch_sys<kPotts>(L, a, block, s);
+    case kIsing: return launch_sys<kIsing>(L, a, block, s, per_sm);
+    case kMuma: return launch_sys<kMuma>(L, a, block, s, per_sm);
+    case kPotts: return launch_sys<kPotts>(L, a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }
