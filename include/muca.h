@@ -165,7 +165,8 @@ int muca_init_ex(muca_ctx **out, int system, int L_or_N, int q, int p, uint64_t 
  *                 32 (32/lanes walkers share a warp; with 1 lane a walker's lane takes
  *                 both bonds of the moved bead); 0 (default) means 16.  A grouping whose
  *                 warp does not fit a block's shared memory falls back to the next larger
- *                 one, and the block shrinks to the warps that fit.  The pair terms are
+ *                 one, and the block shrinks to the warps that fit; one with a bead a
+ *                 lane at most may run as a smaller one with the same bits.  The pair terms are
  *                 FP32 and their grouping over lanes changes their rounding, so
  *                 runs with different values agree within the FP32 tolerance,
  *                 not bit for bit.  Any time.

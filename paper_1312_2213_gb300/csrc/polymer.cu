@@ -374,12 +374,14 @@ __device__ __forceinline__ float bond_between(const Shadow &p, const Shadow &r, 
 // 4-vectors, in the order of pos; ONE: old and proposed side by side, three), and rec = (energy
 // change of the left bond, left bead where it was / left bead moved; of the right bond, right bead
 // where it is; ln of the acceptance word); a change is NaN where the bond breaks.
+// Beads of a chunk: one a lane, two at 8 lanes (up to 5 % faster with 2048 walkers).  More beads than lanes
+// to prepare them cost shared memory and hide nothing: with 16 in every grouping a one-lane warp's 32
+// slots of N = 13 took 87 KB, two warps an SM, and 32768 walkers 6.13 ms for 46 sweeps instead of 1.62.
 template <int G>
-__host__ __device__ constexpr int poly_chunk() { return G > 16 ? G : 16; }
+__host__ __device__ constexpr int poly_chunk() { return G == 8 ? 16 : G; }
 
 template <int G, int MOVES, bool ONE>
 struct PolySlot {
-    static constexpr int CH = poly_chunk<G>();
     static constexpr int BV = ONE ? 3 : 6;  // 4-vectors of a chunk bead
     float4 *pos;     // [3][nP]
     float4 *bead;    // [CH][BV]
@@ -389,14 +391,19 @@ struct PolySlot {
     float *nr;       // [CH] energy of the right bond with the bead moved
     float *eb;       // [N + 1]
     int nP;
-    static __host__ __device__ int pairs(int N) { return ONE ? G : (N + 2 * G - 1) / (2 * G) * G; }
+    static __host__ __device__ int pairs(int N) { return ONE ? G : (N <= G ? N : (N + 2 * G - 1) / (2 * G) * G); }
+    // beads of a chunk that have records (a short chain's chunk is the chain; 16 lanes: always 16, which
+    // the unrolled loop counts on)
+    static __host__ __device__ int records(int N) { return (G == 16 && !MOVES) || N > poly_chunk<G>() ? poly_chunk<G>() : N; }
     static __host__ __device__ size_t bytes(int N)
     {
-        const size_t b = (size_t)48 * pairs(N) + (size_t)CH * (16 * BV + 16 + (MOVES ? 28 : 12) + 4) + 4 * (size_t)(N + 1);
-        return (b + 15) / 16 * 16;
+        const size_t b = (size_t)48 * pairs(N) + (size_t)records(N) * (16 * BV + 16 + (MOVES ? 28 : 12) + 4) + 4 * (size_t)(N + 1);
+        // (an odd number of 16-byte units where several walkers share a warp, for the banks)
+        return G < 16 ? ((b + 15) / 16 | 1) * 16 : (b + 15) / 16 * 16;
     }
     __device__ PolySlot(unsigned char *p, int N)
     {
+        const int CH = records(N);
         nP = pairs(N);
         pos = (float4 *)p;
         bead = pos + 3 * nP;
@@ -486,7 +493,7 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float v)
     c = (t - s) - y;
     s = t;
 }
-enum : uint32_t { kReady = 0u, kLate = 1u, kNoPoint = 2u };
+enum : uint32_t { kReady = 0u, kLate = 1u, kNoPoint = 2u, kLateNext = 3u };
 
 // Sweeps: G lanes per walker, 32/G walkers a warp, all on the same bead i.  The two bonds of bead i
 // (FENE) are taken by lanes 0 and 1 of the group, the other partners (LJ, |i - j| >= 2) by lanes
@@ -513,6 +520,11 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
     constexpr int W = 32 / G;
     constexpr int CH = poly_chunk<G>();
     constexpr bool ONE = NP == kOnePartner;
+    // One or two lanes a walker have no others to prepare bonds beside them, so they evaluate the two
+    // bonds of an attempt in it, of one outcome of the bead before instead of both (N = 5, 32768 walkers,
+    // 122 sweeps: 1.32 against 1.51 ms, one lane); with rotations every grouping does.
+    constexpr bool LATE = MOVES || G <= 2;
+    constexpr bool HOLD = !MOVES && G == 1;  // the bead's master coordinates and step stay in registers
     constexpr int NV = ONE ? 1 : (NP > 0 ? NP : 1);  // 4-vectors evaluated ahead
     using Slot = PolySlot<G, MOVES, ONE>;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -570,6 +582,8 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
 #pragma unroll 1
         for (int c0 = 0; c0 < N; c0 += CH) {
             // ---- prepare the chunk, a bead a lane
+            long long x_own[3] = {0, 0, 0};  // HOLD: this lane's bead of the chunk
+            int s_own[3] = {0, 0, 0};
 #pragma unroll 1
             for (int t = li; t < CH; t += G) {
                 const int j = c0 + t;
@@ -592,9 +606,11 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                     uint32_t how = kReady;
                     if (mv.x >= 0x80000000u) {  // spherical rotation about a bonded neighbour
                         double n[3];
+                        const bool next = j == 0 || (j != N - 1 && (mv.y & 1u));
                         if (!poly_unit(j, g, wid, mv, a.rk, n)) {
                             how = kNoPoint;
-                        } else if (j == 0 || (j != N - 1 && (mv.y & 1u))) {  // about bead j + 1, not visited yet
+                        } else if (G > 2 && next) {  // about bead j + 1, not visited yet
+                            // (one or two lanes take both pivots in the attempt: the binary64 work once)
                             const long long P0 = Xg[j + 1], P1 = Xg[N + j + 1], P2 = Xg[2 * N + j + 1];
                             const double d = poly_distance(poly_axis_diff(X0, P0), poly_axis_diff(X1, P1),
                                                            poly_axis_diff(X2, P2));
@@ -605,7 +621,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                             grid_to_ff(n1 - A1, yn, lyn);
                             grid_to_ff(n2 - A2, zn, lzn);
                         } else {  // about bead j - 1: when it has been visited
-                            how = kLate;
+                            how = next ? kLateNext : kLate;
                             n0 = __double_as_longlong(n[0]);
                             n1 = __double_as_longlong(n[1]);
                             n2 = __double_as_longlong(n[2]);
@@ -615,6 +631,13 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                     S.nx[3 * t + 1] = n1;
                     S.nx[3 * t + 2] = n2;
                     S.how[t] = how;
+                } else if (HOLD) {
+                    x_own[0] = Xg[j];
+                    x_own[1] = Xg[N + j];
+                    x_own[2] = Xg[2 * N + j];
+                    s_own[0] = sx;
+                    s_own[1] = sy;
+                    s_own[2] = sz;
                 } else {
                     S.how[3 * t] = r.x;
                     S.how[3 * t + 1] = r.y;
@@ -626,7 +649,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 S.rec[t] = make_float4(0.0f, 0.0f, 0.0f, logf((float)r.w * 0x1p-32f));
             }
             __syncwarp();
-            if (!MOVES) {
+            if (!LATE) {
 #pragma unroll 1
                 for (int t = li; t < CH; t += G) {
                     const int j = c0 + t;
@@ -720,10 +743,11 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 if (MOVES) {
                     const uint32_t how = S.how[t];
                     no_point = how == kNoPoint;
-                    if (__any_sync(0xffffffffu, how == kLate)) {
+                    const bool turn = how == kLate || (G <= 2 && how == kLateNext);
+                    if (__any_sync(0xffffffffu, turn)) {
                         // about bead i - 1, where it is now; lanes 0, 1, 2 of the group an axis each
                         // (fewer lanes take the axes in turn)
-                        const int pv = i > 0 ? i - 1 : 0;
+                        const int pv = G <= 2 && how == kLateNext ? i + 1 : (i > 0 ? i - 1 : 0);
                         double dd[3];
                         if (G >= 4) {
                             const int c = min(li, 2);
@@ -735,7 +759,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                             for (int k = 0; k < 3; ++k) dd[k] = poly_axis_diff(Xg[k * N + i], Xg[k * N + pv]);
                         }
                         const double d = poly_distance(dd[0], dd[1], dd[2]);
-                        if (how == kLate) {
+                        if (turn) {
                             for (int c = li; c < 3; c += G) {
                                 const long long nn =
                                     poly_rotated(Xg[c * N + pv], __longlong_as_double(S.nx[3 * t + c]), d);
@@ -759,7 +783,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 for (int k = 0; k < (G == 1 ? 2 : 1); ++k) {
                     const bool left = (G == 1) ? k == 0 : li == 0;
                     float d = left ? (acc ? rec.y : rec.x) : rec.z;
-                    if (MOVES) {
+                    if (LATE) {
                         d = 0.0f;
                         if ((G == 1 || li < 2) && (left ? i > 0 : i + 1 < N)) {
                             vb[k] = bond_between(S.get_proposed(t), S.get(left ? i - 1 : i + 1), a);
@@ -775,12 +799,14 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 // the bonded beads and i itself
                 const unsigned u = (unsigned)(li - i + 1);
 #pragma unroll 1
-                for (int m = 0; li + 2 * G * m < N; ++m) {
-                        float d0, d1;
-                        lj_changes<Slot, ONE>(S, t, G * m + li, a, d0, d1);
-                        if (u + 2 * G * m > 2u) kahan_add(s, c, d0);
-                        if (!ONE && u + 2 * G * m + G > 2u && li + 2 * G * m + G < N) kahan_add(s, c, d1);
-                    }
+                for (int e = (G == 1 ? 1 : 0); li + 2 * G * e < N; ++e) {
+                    // (one lane: the pair i / 2 is the bead and one bonded to it, so the others only)
+                    const int m = G == 1 && e <= i / 2 ? e - 1 : e;
+                    float d0, d1;
+                    lj_changes<Slot, ONE>(S, t, G * m + li, a, d0, d1);
+                    if (u + 2 * G * m > 2u) kahan_add(s, c, d0);
+                    if (!ONE && u + 2 * G * m + G > 2u && li + 2 * G * m + G < N) kahan_add(s, c, d1);
+                }
                 // |lane sum| >= 2^22 only for overlapping beads: such a move is rejected
                 const bool huge = !(fabsf(s) < 4194304.0f);
                 const bool refused = group_any<G>(huge || broken, gi) || no_point;
@@ -819,7 +845,7 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
                 }
                 if (acc) {
                     for (int k = li; k < 6; k += G) S.set(i, k, -S.proposed(t, k));
-                    if (MOVES) {
+                    if (LATE) {
                         if (G == 1) {
                             if (i > 0) S.eb[i] = vb[0];
                             if (i + 1 < N) S.eb[i + 1] = vb[1];
@@ -844,9 +870,14 @@ __global__ void __launch_bounds__(kMaxSweepBlock) k_sweep_polymer(const PolyArgs
             }
             nacc += (unsigned)__popc(accs);
             // the bond into the next chunk (the others are rebuilt with the next sweep)
-            if (!MOVES && li == 0 && ((accs >> (nt - 1)) & 1u) && c0 + nt < N) S.eb[c0 + nt] = S.nr[nt - 1];
+            if (!LATE && li == 0 && ((accs >> (nt - 1)) & 1u) && c0 + nt < N) S.eb[c0 + nt] = S.nr[nt - 1];
             // ---- the accepted moves on the master coordinates (32 x 32-bit products: the grid step fits an int)
-            if (!MOVES && active) {
+            if (HOLD) {
+                if (active && ((accs >> li) & 1u)) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) Xg[c * N + c0 + li] = x_own[c] + (long long)s_own[c] * (long long)a.step_q;
+                }
+            } else if (!MOVES && active) {
 #pragma unroll 1
                 for (int t = li; t < nt; t += G) {
                     if ((accs >> t) & 1u) {
@@ -988,11 +1019,11 @@ static cudaError_t launch_g(const PolyArgs &a, int block, cudaStream_t s)
 // weight lookups, the decision) is shared by the 32/G walkers of a warp, the pair
 // terms are spread over G lanes.  A request for a grouping whose warp does not fit
 // the shared memory of a block falls back to the next larger G.  Measured on GB300
-// with 2048 walkers (pilot window, N = 13, 46 sweeps): 1.54, 1.07, 0.68, 0.46, 0.30 and
-// 0.47 ms with 1, 2, 4, 8, 16 and 32 lanes.  Fewer lanes share the fixed cost among more
-// walkers but leave 2048 G / 32 warps to hide latency and prepare more beads one after
-// the other, and only 16 has the loops unrolled by the partners of a lane; so 16 is the
-// default.
+// with 2048 walkers (pilot window, N = 13, 751 sweeps): 21.7, 14.3,
+// 10.7, 7.0, 4.5 and 7.3 ms with 1, 2, 4, 8, 16 and 32 lanes (the last before it ran as 16).
+// Fewer lanes share the fixed cost among more walkers but leave 2048 G / 32 warps to hide
+// latency and prepare more beads one after the other, and only 16 has the loops unrolled by the
+// partners of a lane; so 16 is the default.
 // (What fits is still counted in the bytes of a slot that holds a whole sweep's random words: the
 // lanes decide the rounding of the FP32 sums, so a request keeps the grouping it always had.  The
 // slots above are smaller where this line matters.)
@@ -1008,6 +1039,11 @@ int poly_lanes(const PolyArgs &a, int requested)
              requested == 32) ? requested : 16;
     if (g == 1 && !poly_fits(a, 1)) g = 2;
     if (g == 2 && !poly_fits(a, 2)) g = 4;
+    // With at most a bead a lane, further lanes only add zeros to the same sums, so a smaller grouping
+    // gives the same bits: 32768 walkers of N = 2, 305 sweeps, 1.09 ms with 2 lanes (4: 2.15, 8: 4.0,
+    // 32: 14.0 ms), of N = 3, 203 sweeps, 4.96 ms with 16 (32: 10.8).
+    if (a.N == 2 && (g == 4 || g == 8 || g == 32)) g = 2;
+    if (a.N <= 16 && g == 32) g = 16;
     return g;
 }
 
