@@ -1,0 +1,36 @@
+"""Many walkers at small L: blocks small enough to share an SM do, so that no launch shape falls behind
+for want of registers."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _ms(system, L, q, p, block, sweeps):
+    import torch
+
+    import paper_1312_2213_gb300 as m
+
+    g = m.Muca(system, L, q, p, 7, beta=0.4407 if system == 2 else None, block=block)
+    for _ in range(6):
+        g.iterate(20)
+        g.merge_and_update()
+    best = None
+    for _ in range(4):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        a.record()
+        g.iterate(sweeps)
+        b.record()
+        torch.cuda.synchronize()
+        t = a.elapsed_time(b)
+        best = t if best is None else min(best, t)
+    g.close()
+    return best
+
+
+@pytest.mark.parametrize("L,sweeps", [(8, 1200), (16, 300)])
+def test_potts_blocks_of_32_and_64_walkers(L, sweeps):
+    """16384 walkers: blocks of 32 keep up with blocks of 64 (they took a fifth longer with two of
+    them an SM)."""
+    t32, t64 = (_ms(1, L, 8, 16384, b, sweeps) for b in (32, 64))
+    assert t32 < 1.1 * t64, (t32, t64)
