@@ -487,8 +487,9 @@ __device__ __forceinline__ void sweep_block_tn(const SpinSweepArgs &a, int w0, i
     checks_end(a.state);
 }
 
-template <int SYS, int L>
-__global__ void __launch_bounds__(kMaxSweepBlock, 1) k_sweep_spin_tn(const SpinSweepArgs a)
+// PER_SM: blocks of 64 walkers (256 threads) an SM is to hold; 1 leaves the registers to the compiler.
+template <int SYS, int L, int PER_SM>
+__global__ void __launch_bounds__(PER_SM > 1 ? 256 : kMaxSweepBlock, PER_SM) k_sweep_spin_tn(const SpinSweepArgs a)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     sweep_block_tn<SYS, L>(a, blockIdx.x * (blockDim.x / kCodeWarpsPerWalkerWarp), blockIdx.x, smem);
@@ -1320,15 +1321,35 @@ static int potts_tn_depth(int L, int B, int walkers_per_block)
 }
 
 
-template <int SYS, int L>
-static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
+template <int SYS, int L, int PER_SM>
+static cudaError_t launch_per_sm_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     const size_t smem = spin_sweep_tn_smem_bytes(SYS, L, a.B, block);
     const int largest = spin_sweep_tn_fits(SYS, L, a.B, 64) ? 64 : 32;
-    cudaError_t e = allow_dynamic_smem(k_sweep_spin_tn<SYS, L>, spin_sweep_tn_smem_bytes(SYS, L, a.B, largest));
+    cudaError_t e = allow_dynamic_smem(k_sweep_spin_tn<SYS, L, PER_SM>, spin_sweep_tn_smem_bytes(SYS, L, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    return launch_sweep_kernel(k_sweep_spin_tn<SYS, L>, a, nblk, kCodeWarpsPerWalkerWarp * block, smem, s, per_sm);
+    return launch_sweep_kernel(k_sweep_spin_tn<SYS, L, PER_SM>, a, nblk, kCodeWarpsPerWalkerWarp * block, smem, s, per_sm);
+}
+
+// L = 8: the registers the compiler takes leave room for two blocks an SM; with more walkers than two
+// blocks an SM hold, four in 64 registers a thread are faster (65536 walkers, 585 sweeps: Ising 5.90 / 5.15 ms,
+// MUMA 6.10 / 5.46; 16384 walkers, 2343 sweeps: 6.9 / 7.4 and 7.2 / 7.4).  MUMA with fewer walkers takes the
+// form with room for three (2048 walkers, 4687 sweeps: 9.1 / 8.5 ms; Ising is 1 % slower with it).  At the larger
+// sizes two blocks, then one, are all that the walkers and the table leave (L = 12 and 16 with room for three
+// are up to 4 % slower below 32768 walkers).
+template <int SYS, int L>
+static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
+{
+    if constexpr (L == 8) {
+        int dev = 0, nsm = 0;
+        if (cudaGetDevice(&dev) == cudaSuccess &&
+            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && a.p > 2 * 64 * nsm)
+            return launch_per_sm_tn<SYS, L, 4>(a, block, s, per_sm);
+        return launch_per_sm_tn<SYS, L, SYS == kMuma ? 3 : 1>(a, block, s, per_sm);
+    } else {
+        return launch_per_sm_tn<SYS, L, 1>(a, block, s, per_sm);
+    }
 }
 
 template <int SYS>

@@ -34,3 +34,11 @@ def test_potts_blocks_of_32_and_64_walkers(L, sweeps):
     them an SM)."""
     t32, t64 = (_ms(1, L, 8, 16384, b, sweeps) for b in (32, 64))
     assert t32 < 1.1 * t64, (t32, t64)
+
+
+@pytest.mark.parametrize("system", [0, 2])
+def test_ising_and_muma_L8_with_many_walkers(system):
+    """131072 walkers at L = 8 take less than 6.3 times as long as 16384 (8 times the work in blocks that
+    share the SMs; with two blocks an SM it took 6.7)."""
+    t16, t128 = (_ms(system, 8, 2, p, None, 300) for p in (16384, 131072))
+    assert t128 < 6.3 * t16, (t16, t128)
