@@ -6,8 +6,9 @@ combination gives bit-identical lattices, histograms and weights.  For the polym
 for the threads per block (the lanes per walker do change the FP32 rounding, so they are left as
 set).  The tuner times each valid combination on a scratch context of the same system, size and
 walker count (a short iterate after a warm-up, CUDA events), keeps the fastest, and caches the
-choice per (system, size, q, walkers, GPU) in a JSON file, `$MUCA_TUNE_CACHE` or
-`~/.cache/muca_autotune.json`.
+choice per (kernels, system, size, q, walkers, GPU) in a JSON file, `$MUCA_TUNE_CACHE` or
+`~/.cache/muca_autotune.json`.  The polymer's own default spreads the walkers over the SMs, which no
+fixed block does, so it is one of the candidates.
 
     from paper_1312_2213_gb300 import Muca, ISING2D, autotune
     g = Muca(ISING2D, 32, 2, 8192, seed)
@@ -15,21 +16,34 @@ choice per (system, size, q, walkers, GPU) in a JSON file, `$MUCA_TUNE_CACHE` or
 """
 from __future__ import annotations
 
+import functools
+import glob
+import hashlib
 import json
 import os
 
 from . import ISING2D_MUMA, POLYMER3D, Muca
 
 SPIN_CANDIDATES = [(2, 32), (2, 64), (1, 32), (1, 64), (1, 128), (1, 256), (0, 64), (0, 128), (0, 256)]
-POLY_CANDIDATES = [128, 256, 512]
+POLY_CANDIDATES = [None, 128, 256, 512]  # None: the library's default shape
 
 
 def cache_path() -> str:
     return os.environ.get("MUCA_TUNE_CACHE") or os.path.join(os.path.expanduser("~"), ".cache", "muca_autotune.json")
 
 
+@functools.lru_cache(maxsize=None)
+def _kernels() -> str:
+    """Tag of the kernels the timings belong to: a choice made for others is not looked up."""
+    h = hashlib.sha256()
+    for path in sorted(glob.glob(os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc", "*"))):
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
 def _key(system, L, q, p, device):
-    return "%d/%d/%d/%d/%s" % (system, L, q, p, device)
+    return "%s/%d/%d/%d/%d/%s" % (_kernels(), system, L, q, p, device)
 
 
 def _device_name() -> str:
@@ -94,7 +108,7 @@ def _time_poly(N, p, block, sweeps, window):
 def tune(system: int, L: int, q: int, p: int, beta: float = 0.4407, window=None, sweeps: int | None = None,
          use_cache: bool = True, timer=None) -> dict:
     """Fastest launch shape for the configuration: {"pipeline", "block", "ms", "timings"} for lattice
-    systems, {"block", "ms", "timings"} for the polymer.  `timer` replaces the CUDA-event timing
+    systems, {"block", "ms", "timings"} for the polymer (block None: the library's default).  `timer` replaces the CUDA-event timing
     (for tests)."""
     path = cache_path()
     device = _device_name() if timer is None else "test"
@@ -106,11 +120,14 @@ def tune(system: int, L: int, q: int, p: int, beta: float = 0.4407, window=None,
     if system == POLYMER3D:
         sw = sweeps or max(2, int(2e7 / (p * L)))
         for block in POLY_CANDIDATES:
-            t = (timer or (lambda b: _time_poly(L, p, b, sw, window)))(block)
+            try:
+                t = (timer or (lambda b: _time_poly(L, p, b, sw, window)))(block)
+            except Exception:
+                t = None  # a shape this configuration cannot run
             if t is not None:
-                timings[str(block)] = t
+                timings["default" if block is None else str(block)] = t
         best = min(timings, key=timings.get)
-        res = {"block": int(best), "ms": timings[best], "timings": timings}
+        res = {"block": None if best == "default" else int(best), "ms": timings[best], "timings": timings}
     else:
         sw = sweeps or max(2, int(4e8 / (p * L * L)))
         for pipeline, block in SPIN_CANDIDATES:
@@ -196,7 +213,7 @@ def tune_batch(specs, sweeps, timer=None, use_cache: bool = True) -> dict:
     sweeps = [int(x) for x in sweeps]
     path = cache_path()
     device = _device_name() if timer is None else "test"
-    key = "batch/%s/%s/%s" % (json.dumps(specs), json.dumps(sweeps), device)
+    key = "batch/%s/%s/%s/%s" % (_kernels(), json.dumps(specs), json.dumps(sweeps), device)
     data = _load(path) if use_cache else {}
     if use_cache and key in data:
         return data[key]
@@ -244,7 +261,8 @@ def apply(g: Muca, **kw) -> dict:
     """Tune (or look up) the context's configuration and set the result on it; call before its
     first iterate."""
     res = tune(g.system, g.L, g.q, g.p, window=g.window, **kw)
-    g.set_param("block", res["block"])
+    if res["block"] is not None:
+        g.set_param("block", res["block"])
     if g.system != POLYMER3D:
         g.set_param("pipeline", res["pipeline"])
     return res
