@@ -47,15 +47,17 @@ N = L * L
 # threshold load 1, integer compare 2, flip/select 3, bin update 2, histogram atomic 1, loop 1.
 INSTR_PER_ATTEMPT = 30
 # Cycles an attempt of one walker's chain in this design's sweep inside a row, from clock reads in
-# the Ising consumer (L = 32, GB300 at 2.07 GHz).  p f / CHAIN_CYCLES bounds the
+# the Ising consumer (L = 32, GB300 at 2.07 GHz; hand-overs between rows and sweeps excluded, and the
+# multimagnetic chain is no shorter).  p f / CHAIN_CYCLES bounds the
 # attempts/s of the sweep kernel, and its rate is reported against it as well (the issue-peak
 # fraction counts all schedulers, which one chain per walker cannot fill at p = 8192).
 CHAIN_CYCLES = 39.7
 # DRAM bytes (read + write) per launch of the timed sweep kernel, from one ncu capture of the current
-# k_sweep_spin_tn build (dram__bytes_read.sum + dram__bytes_write.sum; mean of the Ising and MUMA
-# launches: 1.25 MB and 2.17 MB read, nothing written).  It is the walker state and does not grow
-# with the sweep count.  Set to None whenever the kernel changes until it is measured again.
-TRAFFIC_PER_LAUNCH = 1.71e6
+# k_sweep_spin_tn build (dram__bytes_read.sum + dram__bytes_write.sum; mean of four Ising and four
+# MUMA launches of 50 sweeps: 1.37 MB and 2.30 MB read, nothing written).  It is the walker state and
+# does not grow with the sweep count.  Set to None whenever the kernel changes until it is measured
+# again.
+TRAFFIC_PER_LAUNCH = 1.83e6
 # The headline metric as the benchmark specification names it; the workload it is quoted on here
 # (2D Ising L = 32, p = 8192: MUCA in E plus the multimagnetic run) is in the line's "config".
 METRIC = "MUCA move attempts/s on 1 GB300 (batched vs plain) + fraction of issue roofline"
