@@ -495,15 +495,11 @@ __global__ void __launch_bounds__(PER_SM > 1 ? 256 : kMaxSweepBlock, PER_SM) k_s
     sweep_block_tn<SYS, L>(a, blockIdx.x * (blockDim.x / kCodeWarpsPerWalkerWarp), blockIdx.x, smem);
 }
 
-static int potts_tn_depth(int L, int B, int walkers_per_block);
-static size_t potts_tn_smem_bytes(int L, int RD, int B, int walkers_per_block);
+static size_t potts_tn_smem_bytes(int L, int B, int walkers_per_block);
 
 size_t spin_sweep_tn_smem_bytes(int system, int L, int B, int walkers_per_block)
 {
-    if (system == kPotts) {
-        const int rd = potts_tn_depth(L, B, walkers_per_block);
-        return potts_tn_smem_bytes(L, rd ? rd : 2, B, walkers_per_block);
-    }
+    if (system == kPotts) return potts_tn_smem_bytes(L, B, walkers_per_block);
     const int ncw = walkers_per_block / 32;
     return ((size_t)B * (num_cols(system) + 1) * 4 + 15) / 16 * 16 + (size_t)ncw * tn_ring_bytes(L) +
            (size_t)ncw * 2 * kRing * sizeof(unsigned long long);
@@ -520,8 +516,7 @@ size_t spin_sweep_tn_smem_bytes(int system, int L, int B, int walkers_per_block)
 // adds the up neighbour's term the same way, four sites at a time, from the
 // final row above (kept in bytes), and the last site's right neighbour (site 0
 // of the same row, final by then) once a row.  The chain itself is the one of
-// the Ising code form.  RD is the ring depth in rows (4, or 2 where a deeper ring
-// does not fit next to the threshold table).
+// the Ising code form.  RD is the ring depth in rows (potts_tn_depth).
 __device__ __forceinline__ uint32_t nib_half_to_bytes(uint32_t w, int half)  // 4 nibbles -> 4 bytes
 {
     const uint32_t t = __byte_perm(w, 0u, half ? 0x3322u : 0x1100u);
@@ -549,14 +544,11 @@ __device__ __forceinline__ uint32_t bytes_to_nibs(uint32_t w0, uint32_t w1)  // 
 // (4096 walkers 60.2 / 47.6), L = 24 77.6 / 61.0, L = 16 90.0 / 63.9 (q = 10, 2048 walkers 71.3 / 52.8),
 // L = 8 127 / 74; q = 10 L = 48, 2048 walkers 56.1 / 48.9; L = 64, 8192 walkers 81.5 / 77.6 (four parts
 // 81.4: production bounds it, two rows being all that fits beside the table), 4096 walkers 63.4 / 54.0.
-__host__ __device__ constexpr int potts_parts(int L, int ncw)  // parts with work
-{
-    return ncw == 2 ? (L / 4 < 5 ? L / 4 : 5) : (L / 4 < 6 ? L / 4 : 6);
-}
+__host__ __device__ constexpr int potts_parts(int ncw) { return ncw == 2 ? 5 : 6; }  // of a row (L = 48, 64)
 __host__ __device__ constexpr int potts_part_groups(int L, int ncw, int part)
 {
     // as even as whole groups allow, the surplus with the first parts
-    return L / 4 / potts_parts(L, ncw) + (part < L / 4 % potts_parts(L, ncw) ? 1 : 0);
+    return L / 4 / potts_parts(ncw) + (part < L / 4 % potts_parts(ncw) ? 1 : 0);
 }
 __host__ __device__ constexpr int potts_part_max(int L)  // most groups a part has, over both layouts
 {
@@ -1175,7 +1167,7 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const CodeRole role = potts_role(warp, ncw);
     constexpr bool ROWS = RD == 4;            // producers take whole rows in turn, else groups of every row
-    const int NP = ROWS ? RD : potts_parts(L, ncw);  // further producers are idle
+    const int NP = ROWS ? RD : potts_parts(ncw);  // further producers are idle
     const int pair = role.pair, part = role.part;
     const bool producer = role.kind == kRoleProducer && part < NP, consumer = role.kind == kRoleConsumer;
     int g0 = 0, ng = 0;  // a producer's groups of the row
@@ -1302,24 +1294,22 @@ __global__ void __launch_bounds__(potts_threads(2, RD), 1) k_sweep_potts_tn(cons
     sweep_block_tnp<L, RD>(a, blockIdx.x * (blockDim.x == (unsigned)potts_threads(2, RD) ? 64 : 32), blockIdx.x, smem);
 }
 
-static size_t potts_tn_smem_bytes(int L, int RD, int B, int walkers_per_block)
+// Rows of the ring: four up to L = 32, two at L = 48 and 64, where four do not fit beside the table (at
+// L = 64 they would beside 32-walker blocks, not beside the default 64).
+constexpr int potts_tn_depth(int L) { return L <= 32 ? 4 : 2; }
+
+static size_t potts_tn_smem_bytes(int L, int B, int walkers_per_block)
 {
-    const int ncw = walkers_per_block / 32;
+    const int ncw = walkers_per_block / 32, RD = potts_tn_depth(L);
     return tnp_table_bytes(L, B) + (size_t)ncw * tnp_warp_bytes(L, RD) +
            (size_t)ncw * 2 * RD * sizeof(unsigned long long);
 }
 
-// Deepest ring (4 or 2 rows) whose block fits in shared memory; 0 if none does.
-static int potts_tn_depth(int L, int B, int walkers_per_block)
+static bool potts_tn_fits(int L, int B, int walkers_per_block)
 {
-    if (L < 8 || L > 64 || L % 8 != 0 || !sweep_L_supported(L)) return 0;
-    // L = 64 (the split table) is built with the two-row ring only: the four-row one fits
-    // 32-walker blocks but not the default 64
-    if (L < 64 && potts_tn_smem_bytes(L, 4, B, walkers_per_block) <= 227u * 1024u) return 4;
-    if (potts_tn_smem_bytes(L, 2, B, walkers_per_block) <= 227u * 1024u) return 2;
-    return 0;
+    return L >= 8 && L % 8 == 0 && sweep_L_supported(L) &&
+           potts_tn_smem_bytes(L, B, walkers_per_block) <= 227u * 1024u;
 }
-
 
 template <int SYS, int L, int PER_SM>
 static cudaError_t launch_per_sm_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
@@ -1335,9 +1325,9 @@ static cudaError_t launch_per_sm_tn(const SpinSweepArgs &a, int block, cudaStrea
 // L = 8: the registers the compiler takes leave room for two blocks an SM; with more walkers than two
 // blocks an SM hold, four in 64 registers a thread are faster (65536 walkers, 585 sweeps: Ising 5.90 / 5.15 ms,
 // MUMA 6.10 / 5.46; 16384 walkers, 2343 sweeps: 6.9 / 7.4 and 7.2 / 7.4).  MUMA with fewer walkers takes the
-// form with room for three (2048 walkers, 4687 sweeps: 9.1 / 8.5 ms; Ising is 1 % slower with it).  At the larger
-// sizes two blocks, then one, are all that the walkers and the table leave (L = 12 and 16 with room for three
-// are up to 4 % slower below 32768 walkers).
+// form with room for three (2048 walkers, 4687 sweeps: 9.1 / 8.5 ms; Ising is 1 % slower with it).  L = 12
+// and 16 with room for three gain 4-8 % at 65536 walkers and lose up to 20 % below; from L = 24 up the
+// tables leave two blocks, then one.
 template <int SYS, int L>
 static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
@@ -1370,44 +1360,35 @@ static cudaError_t launch_sys_tn(int L, const SpinSweepArgs &a, int block, cudaS
 bool spin_sweep_tn_fits(int system, int L, int B, int walkers_per_block)
 {
     if (system == kPotts)
-        return (walkers_per_block == 32 || walkers_per_block == 64) && potts_tn_depth(L, B, walkers_per_block) != 0;
+        return (walkers_per_block == 32 || walkers_per_block == 64) && potts_tn_fits(L, B, walkers_per_block);
     return (system == kIsing || system == kMuma) && L >= 2 * kRing &&
            (walkers_per_block == 32 || walkers_per_block == 64) &&
            spin_sweep_tn_smem_bytes(system, L, B, walkers_per_block) <= 227u * 1024u;
 }
 
-template <int L, int RD>
+template <int L>
 static cudaError_t launch_one_tnp(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
-    const size_t smem = potts_tn_smem_bytes(L, RD, a.B, block);
-    const int largest = potts_tn_depth(L, a.B, 64) == RD ? 64 : 32;
-    cudaError_t e = allow_dynamic_smem(k_sweep_potts_tn<L, RD>, potts_tn_smem_bytes(L, RD, a.B, largest));
+    constexpr int RD = potts_tn_depth(L);
+    const size_t smem = potts_tn_smem_bytes(L, a.B, block);
+    const int largest = potts_tn_fits(L, a.B, 64) ? 64 : 32;
+    cudaError_t e = allow_dynamic_smem(k_sweep_potts_tn<L, RD>, potts_tn_smem_bytes(L, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
     return launch_sweep_kernel(k_sweep_potts_tn<L, RD>, a, nblk, potts_threads(block / 32, RD), smem, s, per_sm);
 }
 
-template <int RD>
-static cudaError_t launch_potts_tn_rd(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
+static cudaError_t launch_potts_tn(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     switch (L) {
-    case 8: return launch_one_tnp<8, RD>(a, block, s, per_sm);
-    case 16: return launch_one_tnp<16, RD>(a, block, s, per_sm);
-    case 24: return launch_one_tnp<24, RD>(a, block, s, per_sm);
-    case 32: return launch_one_tnp<32, RD>(a, block, s, per_sm);
-    case 48: return launch_one_tnp<48, RD>(a, block, s, per_sm);
-    case 64:  // the split table: only the two-row ring fits
-        if constexpr (RD == 2) return launch_one_tnp<64, 2>(a, block, s, per_sm);
-        return cudaErrorInvalidValue;
+    case 8: return launch_one_tnp<8>(a, block, s, per_sm);
+    case 16: return launch_one_tnp<16>(a, block, s, per_sm);
+    case 24: return launch_one_tnp<24>(a, block, s, per_sm);
+    case 32: return launch_one_tnp<32>(a, block, s, per_sm);
+    case 48: return launch_one_tnp<48>(a, block, s, per_sm);
+    case 64: return launch_one_tnp<64>(a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
-}
-
-static cudaError_t launch_potts_tn(int L, int rd, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
-{
-    if (rd == 4) return launch_potts_tn_rd<4>(L, a, block, s, per_sm);
-    if (rd == 2) return launch_potts_tn_rd<2>(L, a, block, s, per_sm);
-    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
@@ -1416,7 +1397,7 @@ cudaError_t launch_spin_sweep_tn(int system, int L, const SpinSweepArgs &a, int 
     switch (system) {
     case kIsing: return launch_sys_tn<kIsing>(L, a, block, s, per_sm);
     case kMuma: return launch_sys_tn<kMuma>(L, a, block, s, per_sm);
-    case kPotts: return launch_potts_tn(L, potts_tn_depth(L, a.B, block), a, block, s, per_sm);
+    case kPotts: return launch_potts_tn(L, a, block, s, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }
