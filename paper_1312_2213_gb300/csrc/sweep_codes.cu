@@ -532,9 +532,9 @@ __device__ __forceinline__ uint32_t bytes_to_nibs(uint32_t w0, uint32_t w1)  // 
 // instructions against the consumer's 18; one warp issues an instruction every 2.5 cycles at best and
 // the multiply and logic pipes of a scheduler sustain a Philox block in 88 cycles, so production (not
 // the chain) bounds the blocks of two walker warps and is spread over more warps than the Ising
-// form's.  The block has 12 warps for two walker warps, 8 or 6 for one, warp w on scheduler w mod 4:
+// form's.  The block has 12 warps for two walker warps, 8 for one, warp w on scheduler w mod 4:
 //   ncw = 2: [C0, C1, P0.0, P1.0,  P0.3, P1.3, P0.1, P1.1,  P0.4, P1.4, P0.2, P1.2]
-//   ncw = 1: [C0, P0.0, P0.1, P0.2,  -, P0.3, P0.4, P0.5], without the last two where four produce
+//   ncw = 1: [C0, P0.0, P0.1, P0.2,  -, P0.3, P0.4, P0.5]
 // so a consumer shares its scheduler with one or two of its producers or with none.
 // Where the ring has four rows (L <= 32) four producers take whole rows in turn (produce_potts_rows).
 // With two rows (L = 48 and 64) all work on the same row: parts 0..n-1 own contiguous groups of four
@@ -563,10 +563,14 @@ __device__ __forceinline__ CodeRole potts_role(int warp, int ncw)
     const int pair = warp & 1, row = warp >> 2;
     return CodeRole{kRoleProducer, pair, (warp & 2) ? row : row + 2};
 }
-// Threads of a block.  An idle warp holds registers: with eight warps two 32-walker blocks of L = 16 fitted
-// an SM, with six three do (q = 8, 16384 walkers in 32-walker blocks, 585 sweeps: 11.4 / 9.6 ms; L = 8,
-// 2343 sweeps, 11.1 / 8.6; L = 24, 32768 walkers, 130 sweeps, 9.3 / 7.5).
-constexpr int potts_threads(int ncw, int RD) { return ncw == 2 ? 384 : (RD == 4 ? 192 : 256); }
+// Threads of a block.  An idle warp holds registers: with eight warps two 32-walker blocks of L = 16 fit
+// an SM, with the six that four producers need three do, so a launch of more blocks than SMs drops the
+// last two (q = 8, 16384 walkers in 32-walker blocks, 585 sweeps: 11.4 / 9.6 ms; L = 8, 2343 sweeps,
+// 11.1 / 8.6; L = 24, 32768 walkers, 130 sweeps, 9.3 / 7.5).  Where every block can have an SM to itself the idle
+// warps cost nothing, and a batch may place its blocks better with them: the nine-system mix with 332 walkers
+// as a graph of five iterations of 25 sweeps takes 10.95 ms, with six warps 12.25 (why is not known).
+constexpr int potts_threads(int ncw) { return ncw == 2 ? 384 : 256; }
+constexpr int kPottsThreadsDense = 192;  // one walker warp, four producers
 
 // The split table (L = 64, see potts_split_full): the acceptance words travel as their
 // upper 16 bits, two to a 32-bit word (uint2 per 4 sites instead of uint4).
@@ -1162,7 +1166,7 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
     constexpr int C = 9;
     constexpr int RS = R::RSW;  // words a table row
     constexpr size_t S = (size_t)(L / 4) * 32;
-    const int ncw = blockDim.x == (unsigned)potts_threads(2, RD) ? 2 : 1;
+    const int ncw = blockDim.x == (unsigned)potts_threads(2) ? 2 : 1;
     // (from lane 0, so that the compiler knows it is the same for the warp)
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const CodeRole role = potts_role(warp, ncw);
@@ -1288,10 +1292,10 @@ __device__ __forceinline__ void sweep_block_tnp(const SpinSweepArgs &a, int w0, 
 template <int L, int RD>
 // At most 64 walkers (384 threads) a block: the L = 48 and 64 forms need more than the 128
 // registers a thread that 512-thread blocks would leave.
-__global__ void __launch_bounds__(potts_threads(2, RD), 1) k_sweep_potts_tn(const SpinSweepArgs a)
+__global__ void __launch_bounds__(potts_threads(2), 1) k_sweep_potts_tn(const SpinSweepArgs a)
 {
     extern __shared__ __align__(16) uint32_t smem[];
-    sweep_block_tnp<L, RD>(a, blockIdx.x * (blockDim.x == (unsigned)potts_threads(2, RD) ? 64 : 32), blockIdx.x, smem);
+    sweep_block_tnp<L, RD>(a, blockIdx.x * (blockDim.x == (unsigned)potts_threads(2) ? 64 : 32), blockIdx.x, smem);
 }
 
 // Rows of the ring: four up to L = 32, two at L = 48 and 64, where four do not fit beside the table (at
@@ -1309,6 +1313,15 @@ static bool potts_tn_fits(int L, int B, int walkers_per_block)
 {
     return L >= 8 && L % 8 == 0 && sweep_L_supported(L) &&
            potts_tn_smem_bytes(L, B, walkers_per_block) <= 227u * 1024u;
+}
+
+// SMs of the current device (152 on GB300, also if it cannot be asked).
+static int device_sms()
+{
+    int dev = 0, nsm = 0;
+    const bool known = cudaGetDevice(&dev) == cudaSuccess &&
+                       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && nsm > 0;
+    return known ? nsm : 152;
 }
 
 template <int SYS, int L, int PER_SM>
@@ -1332,10 +1345,7 @@ template <int SYS, int L>
 static cudaError_t launch_one_tn(const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
 {
     if constexpr (L == 8) {
-        int dev = 0, nsm = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && a.p > 2 * 64 * nsm)
-            return launch_per_sm_tn<SYS, L, 4>(a, block, s, per_sm);
+        if (a.p > 2 * 64 * device_sms()) return launch_per_sm_tn<SYS, L, 4>(a, block, s, per_sm);
         return launch_per_sm_tn<SYS, L, SYS == kMuma ? 3 : 1>(a, block, s, per_sm);
     } else {
         return launch_per_sm_tn<SYS, L, 1>(a, block, s, per_sm);
@@ -1375,7 +1385,8 @@ static cudaError_t launch_one_tnp(const SpinSweepArgs &a, int block, cudaStream_
     cudaError_t e = allow_dynamic_smem(k_sweep_potts_tn<L, RD>, potts_tn_smem_bytes(L, a.B, largest));
     if (e != cudaSuccess) return e;
     const int nblk = (a.p + block - 1) / block;
-    return launch_sweep_kernel(k_sweep_potts_tn<L, RD>, a, nblk, potts_threads(block / 32, RD), smem, s, per_sm);
+    const int threads = RD == 4 && block == 32 && nblk > device_sms() ? kPottsThreadsDense : potts_threads(block / 32);
+    return launch_sweep_kernel(k_sweep_potts_tn<L, RD>, a, nblk, threads, smem, s, per_sm);
 }
 
 static cudaError_t launch_potts_tn(int L, const SpinSweepArgs &a, int block, cudaStream_t s, int *per_sm)
