@@ -461,8 +461,8 @@ int create(muca_ctx **out, int system, int L, int q, int p, uint64_t seed, void 
     if (!c) return fail(MUCA_ERR_OOM, "host allocation failed");
     fill_shape(c, system, L, q, p);
     // q-Potts with few walkers: when every 32-walker block has an SM to itself, one consumer warp
-    // an SM decides faster than two (measured at p = 2048: 71 against 92 cycles an attempt at
-    // L = 16, 60 against 72 at L = 32)
+    // an SM decides faster than two (52.8 against 63.9 cycles an attempt at L = 16, 47.6 against
+    // 57.8 at L = 32)
     if (system == kPotts && c->block == 64 && spin_sweep_tn_fits(system, L, c->B, 32)) {
         int dev = 0, nsm = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&

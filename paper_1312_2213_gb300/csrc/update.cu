@@ -27,7 +27,8 @@ namespace muca {
 
 // Merge: 32 bins x 8 slot rows a block.  A thread that walked all ceil(p / block) slots of its bin
 // alone waited for one L2 round trip after the other (52 us for 128 slots of 8193 bins, 34 us for
-// the nine systems of the mix); eight rows with four loads in flight each take 6.3 and 4.6 us.
+// the nine systems of the mix); eight rows take 6.3 and 4.6 us.  (A row still goes slot by slot: a
+// slot's count is cleared before the next is read.)
 constexpr int kMergeBins = 32, kMergeRows = 8;
 
 __device__ __forceinline__ void merge_body(const UpdateArgs &a)
