@@ -220,7 +220,7 @@ def muca_batch_free(b):
 
 class Batch:
     """Several Muca systems advanced together: per iteration every system's own sweep kernel on a
-    stream of its own, side by side (form 1, default), or one persistent sweep launch over all
+    stream of its own or queued behind a heavier one where the SMs are taken (form 1, default), or one persistent sweep launch over all
     systems (form 0); then batched merge, recursion and thresholds; optionally the whole run as
     one CUDA graph."""
 

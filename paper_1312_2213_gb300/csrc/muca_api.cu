@@ -1331,7 +1331,7 @@ struct muca_batch {
     cudaGraphExec_t exec = nullptr;
     int g_iter = 0;
     int64_t g_sweeps = 0;
-    // form 1: every system's own sweep launch on a stream of its own, forked from and joined
+    // form 1: every system's own sweep launch on one of these streams (batch_lanes.h), forked from and joined
     // back into the batch stream (captured as parallel graph branches)
     int form = 0;  // set to 1 (the default) by muca_batch_create
     std::vector<cudaStream_t> sub;
